@@ -102,7 +102,9 @@ typedef struct {
  *               coefficients and vectors and FP64-accumulated dot products.
  *   precond     VOFP_PRECOND_JACOBI (diagonal) or VOFP_PRECOND_RBSGS (red-black symmetric
  *               Gauss-Seidel, applied as CG on the black unknowns after eliminating the red ones
- *               (Eisenstat's form); both modes, and the bench default in mixed mode).
+ *               (Eisenstat's form); both modes, and the bench default in mixed mode).  In mixed
+ *               mode, from 2^16 cells on, its inner CG also has a coarse-grid correction: an
+ *               additive V-cycle on 2x2x2 aggregates smoothed by red-black Gauss-Seidel.
  *   rtol        the solve returns VOFP_OK only when the residual recomputed from the returned x,
  *               ||b_hat - A_hat x|| (2-norm over the unknowns, FP64), is at most rtol ||b_hat||.
  *               The iteration aims slightly below rtol; when the recomputed residual is still
@@ -115,8 +117,9 @@ typedef struct {
  *               steps (the FP64 residual replaces the FP32 one, a "reliable update"); 1 restarts
  *               the inner PCG from p = r at every refinement step.
  *   check_every convergence is tested every check_every iterations (even, 2 .. 64; 0 = default:
- *               64 in mixed mode from 2^20 cells on, where an inner solve runs on to the end of
- *               its 64 iterations past its stop and saves refinement steps, 8 otherwise).
+ *               16 where the coarse-grid correction runs, 64 in the other mixed solves from 2^20
+ *               cells on, where an inner solve runs on to the end of its 64 iterations past its
+ *               stop and saves refinement steps, 8 otherwise).
  *   x0_zero     1: ignore the contents of x and start from 0.
  *   host_loop   0: the loop runs as a CUDA graph with a device-side WHILE condition (no host round
  *               trip per iteration).  1: the host launches each kernel and reads the convergence

@@ -647,7 +647,9 @@ void launch_main_t(vofp_ctx* c, cudaStream_t st, const float* po, float* pn, boo
     using G = RbcGeomT<RPT>;
     const Dims d = c->d;
     const int nh = d.nx / 2;
-    const CUtensorMap *mr = tensor_map_f32_x(c, c->rbc_r, nh, G::BWC, G::TH + 4),
+    // the direction's source: z with the coarse-grid correction, r without
+    const float* src = c->mg_ok ? c->mg_z : c->rbc_r;
+    const CUtensorMap *mr = tensor_map_f32_x(c, src, nh, G::BWC, G::TH + 4),
                       *mp = tensor_map_f32_x(c, po, nh, G::BWC, G::TH + 4),
                       *mx = tensor_map_f32(c, c->Txf, G::BWF, G::TH + 2),
                       *my = tensor_map_f32(c, c->Tyf, G::BWF, G::TH + 3),
@@ -662,7 +664,7 @@ void launch_main_t(vofp_ctx* c, cudaStream_t st, const float* po, float* pn, boo
     maps.tx = *mx;
     maps.ty = *my;
     maps.tz = *mz;
-    const RbcExc ex{(const float*)c->rbc_r, (const int*)c->rbc_enb, (const float*)c->rbc_eT, c->rbc_dE,
+    const RbcExc ex{src, (const int*)c->rbc_enb, (const float*)c->rbc_eT, c->rbc_dE,
                     c->rbc_nh, c->rbc_ne};
     launch_dep(c, pdl, k_rbc_tma<kRbcStages, RPT>, dim3(c->rbc_nblocks), dim3(kBX, kBY),
                cg_rbc_smem<kRbcStages, RPT>(), st, maps, d, c->rbc_split, ex, po, pn, c->rbc_x, c->rbc_q,
@@ -710,6 +712,11 @@ void rbc_iteration(vofp_ctx* c, cudaStream_t st, const float* po, float* pn, cud
     const bool pdl = c->pdl != 0 && use_h != 0;
     launch_main(c, st, po, pn, pdl);
     rbc_aux(c, st, po, pn, pdl);
+    if (c->mg_ok) {
+        mg_update(c, st, pdl, h, use_h);
+        mg_precondition(c, st, pdl, 0);
+        return;
+    }
     const long long nc = c->rbc_nh + c->rbc_ne;
     // the update: one wave of four 256-thread blocks per SM (its register cap); two waves of eight
     // per SM took 7.5 us more per iteration at 512x256x128

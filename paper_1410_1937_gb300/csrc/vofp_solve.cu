@@ -653,14 +653,20 @@ void launch_cg_iteration(vofp_ctx* c, cudaStream_t st, V* r, V* po, V* pn, V* xv
                          const V* Tx, const V* Ty, const V* Tz, bool inner, bool rb,
                          cudaGraphConditionalHandle h, int use_h) {
     const uint32_t* bits = rb ? c->excl_bits : c->slave_bits;
+    const bool mg = sizeof(V) == 4 && inner && rb && c->mg_ok;
     if (rb) {
-        launch_cg_rb<V>(c, st, Tx, Ty, Tz, r, po, pn, xv, q);
+        launch_cg_rb<V>(c, st, Tx, Ty, Tz, mg ? reinterpret_cast<const V*>(c->mg_z) : r, po, pn, xv, q);
     } else {
         launch_cg_stencil<V>(c, st, Tx, Ty, Tz, r, po, pn, xv, q);
     }
     if (c->ngroups > 0)
         launch(c, k_group_patch<V>, ceil_div(c->ngroups, kNT), kNT, st, c->ngroups, c->gptr, c->gcells, c->gcorr, q, pn,
                1, c->sc, c->partials, c->counters);
+    if (mg) {
+        mg_update(c, st, c->pdl != 0 && use_h != 0, h, use_h);
+        mg_precondition(c, st, c->pdl != 0 && use_h != 0, 0);
+        return;
+    }
     if (inner)
         launch(c, k_cg_update<V, true>, stream_grid(c->d.n / (sizeof(V) == 8 ? 2 : 4) + 1), kNT, st,
                c->d.n, r, (const V*)q, bits, c->sc, c->partials, c->counters, h, use_h, (const double*)nullptr, 0);
@@ -801,6 +807,7 @@ void launch_outer_head(vofp_ctx* c, cudaStream_t st, bool rb, cudaGraphCondition
         else
             launch(c, k_inner_prep, stream_grid(c->d.n), kNT, st, c->d.n, (const double*)c->q,
                    (const uint32_t*)c->excl_bits, c->rf, c->xf, c->pf0, c->sc, c->partials, c->counters);
+        if (c->mg_ok) mg_precondition(c, st, c->pdl != 0 && use_h != 0, 1);
     } else {
         launch(c, k_inner_prep, stream_grid(c->d.n), kNT, st, c->d.n, (const double*)c->r,
                (const uint32_t*)c->slave_bits, c->rf, c->xf, c->pf0, c->sc, c->partials, c->counters);
@@ -808,7 +815,7 @@ void launch_outer_head(vofp_ctx* c, cudaStream_t st, bool rb, cudaGraphCondition
 }
 int outer_head_kernels(const vofp_ctx* c, bool rb) {
     const int g = c->ngroups > 0 ? 1 : 0;
-    return 1 + g + 1 + (rb ? 2 + g : 0) + 1;
+    return 1 + g + 1 + (rb ? 2 + g + (c->mg_ok ? 1 + mg_precondition_kernels(c) : 0) : 0) + 1;
 }
 void launch_inner_body(vofp_ctx* c, cudaStream_t st, int U, bool rb, cudaGraphConditionalHandle hi, int use_h) {
     if (rb && c->rbc_ok) {
@@ -848,16 +855,17 @@ int outer_tail_kernels(const vofp_ctx* c, bool rb) {
 }
 // kernels of one mixed inner iteration
 int inner_iteration_kernels(const vofp_ctx* c, bool rb) {
+    const int pre = rb && c->mg_ok ? mg_precondition_kernels(c) : 0;
     if (rb && c->rbc_ok)   // iteration kernel (exception rows inside), fix rows, update
-        return 2 + (c->rbc_nf + (c->rbc_gm ? c->ngroups : 0) > 0 ? 1 : 0);
-    return iteration_kernels(c, rb);
+        return 2 + (c->rbc_nf + (c->rbc_gm ? c->ngroups : 0) > 0 ? 1 : 0) + pre;
+    return iteration_kernels(c, rb) + pre;
 }
 
-int graph_key(int U, bool rb) { return U * 2 + (rb ? 1 : 0); }
+int graph_key(const vofp_ctx* c, int U, bool rb) { return U * 4 + (rb ? 1 : 0) + (c->mg_ok ? 2 : 0); }
 
 // FP64 loop: WHILE { U x [red half-stencil (RB), stencil, patch, update]; true-residual check }
 vofp_status build_graph_fp64(vofp_ctx* c, int U, bool rb) {
-    if (c->graph_fp64 && c->graph_fp64_key == graph_key(U, rb)) return VOFP_OK;
+    if (c->graph_fp64 && c->graph_fp64_key == graph_key(c, U, rb)) return VOFP_OK;
     const long long launches0 = c->launches;
     if (c->graph_fp64) {
         cudaGraphExecDestroy(c->graph_fp64);
@@ -877,7 +885,7 @@ vofp_status build_graph_fp64(vofp_ctx* c, int U, bool rb) {
     VOFP_CUDA_TRY(c, cudaGraphInstantiate(&c->graph_fp64, g, 0));
     cudaGraphDestroy(g);
     cudaStreamDestroy(cs);
-    c->graph_fp64_key = graph_key(U, rb);
+    c->graph_fp64_key = graph_key(c, U, rb);
     c->launches = launches0;
     return VOFP_OK;
 }
@@ -943,7 +951,7 @@ vofp_status build_graph_mixed_once(vofp_ctx* c, int U, bool rb) {
         c->set_error(std::string("cudaGraphInstantiate: ") + cudaGetErrorString(ie));
         return VOFP_ERR_CUDA;
     }
-    c->graph_mixed_key = graph_key(U, rb);
+    c->graph_mixed_key = graph_key(c, U, rb);
     return VOFP_OK;
 }
 
@@ -951,7 +959,7 @@ vofp_status build_graph_mixed_once(vofp_ctx* c, int U, bool rb) {
 // launch where the driver accepts that inside the conditional body; otherwise rebuilt once with
 // ordinary edges (and kept so for the context).
 vofp_status build_graph_mixed(vofp_ctx* c, int U, bool rb) {
-    if (c->graph_mixed && c->graph_mixed_key == graph_key(U, rb)) return VOFP_OK;
+    if (c->graph_mixed && c->graph_mixed_key == graph_key(c, U, rb)) return VOFP_OK;
     c->launch_err = cudaSuccess;
     const long long launches0 = c->launches;
     vofp_status s = build_graph_mixed_once(c, U, rb);
@@ -1087,7 +1095,8 @@ vofp_status solve_pass(vofp_ctx* c, const double* b, double* x, const vofp_solve
     vofp_status s = ensure_workspace(c);
     if (s) return s;
     // colour-compact vectors of the red-black inner solve (built once per operator)
-    if (o->mode == VOFP_MODE_MIXED && o->precond == VOFP_PRECOND_RBSGS && (s = rbc_ensure(c))) return s;
+    // and the hierarchy of its coarse-grid correction
+    if (o->mode == VOFP_MODE_MIXED && o->precond == VOFP_PRECOND_RBSGS && ((s = rbc_ensure(c)) || (s = mg_ensure(c)))) return s;
     const long long N = c->d.n;
     cudaStream_t st = c->stream;
     // Default: the FP64 loop checks its true residual every 8 iterations, and so does the mixed
@@ -1098,7 +1107,14 @@ vofp_status solve_pass(vofp_ctx* c, const double* b, double* x, const vofp_solve
     // an inner solve can reach the FP32 rounding floor within 64 iterations, and the steps taken
     // there, kept as the next inner solve's direction, stalled it (a 16^3 sphere, Jacobi: 100032
     // iterations without converging).
-    const int U = o->check_every > 0 ? o->check_every : (o->mode == VOFP_MODE_MIXED && N >= (1LL << 20) ? 64 : 8);
+    const bool mg = o->mode == VOFP_MODE_MIXED && o->precond == VOFP_PRECOND_RBSGS && c->mg_ok;
+    // With the coarse-grid correction an inner solve takes 10-20 iterations at any size: every 16 from
+    // 2^16 cells on (512x256x128 to 1e-12: 106 ms, 110 testing every 8, 115 every 32), 8 below, where
+    // 16 already reach the FP32 floor of the smallest grids.
+    const int U = o->check_every > 0 ? o->check_every
+                  : o->mode != VOFP_MODE_MIXED ? 8
+                  : mg ? (N >= (1LL << 16) ? 16 : 8)
+                       : (N >= (1LL << 20) ? 64 : 8);
     VOFP_CUDA_TRY(c, cudaEventRecord(c->ev0, st));
     double sums[3];
     if ((s = prepare_rhs(c, b, sums))) return s;
@@ -1247,6 +1263,21 @@ vofp_status solve(vofp_ctx* c, const double* b, double* x, const vofp_solve_opts
     vofp_solve_info acc{};
     vofp_status r = solve_pass(c, b, x, o, &acc);
     const long long max_iter = o->max_iter > 0 ? o->max_iter : 100000;
+    if (r == VOFP_ERR_BREAKDOWN && c->mg_ok && o->mode == VOFP_MODE_MIXED && o->precond == VOFP_PRECOND_RBSGS &&
+        std::isfinite(acc.rel_residual) && acc.iterations < max_iter) {
+        // the coarse-grid correction lost positivity: the plain red-black iteration from the iterate
+        c->mg_ok = false;
+        vofp_solve_opts o2 = *o;
+        o2.x0_zero = 0;
+        o2.max_iter = (int)(max_iter - acc.iterations);
+        vofp_solve_info i2{};
+        c->err.clear();
+        r = solve_pass(c, b, x, &o2, &i2);
+        i2.iterations += acc.iterations;
+        i2.outer_iterations += acc.outer_iterations;
+        i2.seconds += acc.seconds;
+        acc = i2;
+    }
     for (int restart = 0; r == VOFP_OK && !(acc.rel_residual <= o->rtol); ++restart) {
         if (acc.iterations >= max_iter) {
             r = VOFP_ERR_NOT_CONVERGED;
