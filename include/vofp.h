@@ -103,8 +103,9 @@ typedef struct {
  *   precond     VOFP_PRECOND_JACOBI (diagonal) or VOFP_PRECOND_RBSGS (red-black symmetric
  *               Gauss-Seidel, applied as CG on the black unknowns after eliminating the red ones
  *               (Eisenstat's form); both modes, and the bench default in mixed mode).  In mixed
- *               mode, from 2^16 cells on, its inner CG also has a coarse-grid correction: an
- *               additive V-cycle on 2x2x2 aggregates smoothed by red-black Gauss-Seidel.
+ *               mode, from 2^16 cells and for rtol <= 1e-7, its inner CG also has a coarse-grid
+ *               correction: an additive V-cycle on 2x2x2 aggregates smoothed by red-black
+ *               Gauss-Seidel.
  *   rtol        the solve returns VOFP_OK only when the residual recomputed from the returned x,
  *               ||b_hat - A_hat x|| (2-norm over the unknowns, FP64), is at most rtol ||b_hat||.
  *               The iteration aims slightly below rtol; when the recomputed residual is still

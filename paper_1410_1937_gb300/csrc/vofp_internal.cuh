@@ -82,6 +82,10 @@ struct MgLevel {
 // 5 times faster than the plain iteration (64x48x40 to 1e-12: 12 against 19 ms); at 16^3 to 48x40x32
 // the two took about the same to 1.4 times
 constexpr long long kMgMinCells = 1 << 16;
+// ... and the loosest tolerance that does.  The correction is the faster one at every tolerance (256x128x64
+// to 1e-6: 13.9 against 39.4 ms, 512x256x128 49 against 232 ms), but a pressure solved more loosely is
+// settled only to its first few digits, and which ones depends on the iteration: such solves keep theirs
+constexpr double kMgMaxRtol = 1e-7;
 
 }  // namespace vofp
 
@@ -192,6 +196,10 @@ struct vofp_ctx {
     // VOF operator (vofp_vof.cu): corrected stage velocities, two stage buffers, interface planes
     double *vof_uxh = nullptr, *vof_uyh = nullptr, *vof_wmh = nullptr, *vof_wph = nullptr;
     double *vof_phi = nullptr, *vof_plic = nullptr;
+    int* vof_list = nullptr;          // cells with 0 < phi < 1 of the coming stage
+    double* vof_rec = nullptr;        // 1 / width of the cells along x, y, z
+    uint32_t* vof_lim = nullptr;      // high words of 0.49 width / dt
+    unsigned int* vof_count = nullptr;   // list lengths per stage
     double* rk2_buf = nullptr;        // RK2 step (vofp_rk2.cu): face fields and cell arrays
     long long rbc_cap = 0;            // allocated compact length
     int rbc_blocks_per_sm = 0;
@@ -199,7 +207,8 @@ struct vofp_ctx {
     int rbc_nblocks = 0;              // iteration kernel blocks and work split (see rbc_split)
     vofp::RbcSplit rbc_split{};
     // coarse-grid correction of the mixed red-black solve (vofp_mg.cu)
-    bool mg_built = false, mg_ok = false;   // looked at / in use for the current operator
+    bool mg_built = false, mg_ok = false;   // looked at / usable for the current operator
+    bool mg_use = false;                    // in use in the current solve
     std::vector<vofp::MgLevel> mg;
     float *mg_w = nullptr, *mg_z = nullptr; // weights and z of the inner vectors
     uint32_t* mg_mask = nullptr;      // per aggregate (a byte): its even cells that are group masters
@@ -249,6 +258,7 @@ void rbc_iteration(vofp_ctx* c, cudaStream_t st, const float* po, float* pn, cud
 void rbc_finish_xf(vofp_ctx* c, cudaStream_t st);                 // xf (full grid) = x_c + alpha p0_c
 int rbc_pq_parts(const vofp_ctx* c);   // block partials of p.Ap the compact iteration leaves for the update
 // coarse-grid correction of the mixed red-black solve (vofp_mg.cu)
+bool mg_wanted(const vofp_ctx* c, double rtol);   // whether a mixed red-black solve takes it
 vofp_status mg_ensure(vofp_ctx* c);    // hierarchy of the current operator; sets c->mg_ok
 void mg_precondition(vofp_ctx* c, cudaStream_t st, bool pdl, int start);   // z and beta from r
 void mg_update(vofp_ctx* c, cudaStream_t st, bool pdl, cudaGraphConditionalHandle h, int use_h);

@@ -797,16 +797,20 @@ void launch_update(vofp_ctx* c, cudaStream_t st, bool pdl, cudaGraphConditionalH
 
 }  // namespace
 
+// Grids below kMgMinCells and tolerances above kMgMaxRtol keep the plain iteration (VOFP_MG=0: every
+// solve does, 2: none).
+bool mg_wanted(const vofp_ctx* c, double rtol) {
+    const char* env = std::getenv("VOFP_MG");
+    const int use = env ? std::atoi(env) : 1;
+    return use == 2 || (use != 0 && c->d.n >= kMgMinCells && rtol <= kMgMaxRtol);
+}
+
 // The hierarchy and the weights of the current operator (mixed red-black solve; once per operator).
-// Grids below kMgMinCells keep the plain iteration (VOFP_MG=0: every grid does, 2: none).
 vofp_status mg_ensure(vofp_ctx* c) {
     if (c->mg_built) return VOFP_OK;
     c->mg_built = true;
     c->mg_ok = false;
     const Dims d = c->d;
-    const char* env = std::getenv("VOFP_MG");
-    const int use = env ? std::atoi(env) : 1;
-    if (use == 0 || (use != 2 && d.n < kMgMinCells)) return VOFP_OK;
     cudaStream_t st = c->stream;
     vofp_status s;
     if (c->mg.empty()) {

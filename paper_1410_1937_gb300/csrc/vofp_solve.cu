@@ -653,7 +653,7 @@ void launch_cg_iteration(vofp_ctx* c, cudaStream_t st, V* r, V* po, V* pn, V* xv
                          const V* Tx, const V* Ty, const V* Tz, bool inner, bool rb,
                          cudaGraphConditionalHandle h, int use_h) {
     const uint32_t* bits = rb ? c->excl_bits : c->slave_bits;
-    const bool mg = sizeof(V) == 4 && inner && rb && c->mg_ok;
+    const bool mg = sizeof(V) == 4 && inner && rb && c->mg_use;
     if (rb) {
         launch_cg_rb<V>(c, st, Tx, Ty, Tz, mg ? reinterpret_cast<const V*>(c->mg_z) : r, po, pn, xv, q);
     } else {
@@ -807,7 +807,7 @@ void launch_outer_head(vofp_ctx* c, cudaStream_t st, bool rb, cudaGraphCondition
         else
             launch(c, k_inner_prep, stream_grid(c->d.n), kNT, st, c->d.n, (const double*)c->q,
                    (const uint32_t*)c->excl_bits, c->rf, c->xf, c->pf0, c->sc, c->partials, c->counters);
-        if (c->mg_ok) mg_precondition(c, st, c->pdl != 0 && use_h != 0, 1);
+        if (c->mg_use) mg_precondition(c, st, c->pdl != 0 && use_h != 0, 1);
     } else {
         launch(c, k_inner_prep, stream_grid(c->d.n), kNT, st, c->d.n, (const double*)c->r,
                (const uint32_t*)c->slave_bits, c->rf, c->xf, c->pf0, c->sc, c->partials, c->counters);
@@ -815,7 +815,7 @@ void launch_outer_head(vofp_ctx* c, cudaStream_t st, bool rb, cudaGraphCondition
 }
 int outer_head_kernels(const vofp_ctx* c, bool rb) {
     const int g = c->ngroups > 0 ? 1 : 0;
-    return 1 + g + 1 + (rb ? 2 + g + (c->mg_ok ? 1 + mg_precondition_kernels(c) : 0) : 0) + 1;
+    return 1 + g + 1 + (rb ? 2 + g + (c->mg_use ? 1 + mg_precondition_kernels(c) : 0) : 0) + 1;
 }
 void launch_inner_body(vofp_ctx* c, cudaStream_t st, int U, bool rb, cudaGraphConditionalHandle hi, int use_h) {
     if (rb && c->rbc_ok) {
@@ -855,13 +855,13 @@ int outer_tail_kernels(const vofp_ctx* c, bool rb) {
 }
 // kernels of one mixed inner iteration
 int inner_iteration_kernels(const vofp_ctx* c, bool rb) {
-    const int pre = rb && c->mg_ok ? mg_precondition_kernels(c) : 0;
+    const int pre = rb && c->mg_use ? mg_precondition_kernels(c) : 0;
     if (rb && c->rbc_ok)   // iteration kernel (exception rows inside), fix rows, update
         return 2 + (c->rbc_nf + (c->rbc_gm ? c->ngroups : 0) > 0 ? 1 : 0) + pre;
     return iteration_kernels(c, rb) + pre;
 }
 
-int graph_key(const vofp_ctx* c, int U, bool rb) { return U * 4 + (rb ? 1 : 0) + (c->mg_ok ? 2 : 0); }
+int graph_key(const vofp_ctx* c, int U, bool rb) { return U * 4 + (rb ? 1 : 0) + (c->mg_use ? 2 : 0); }
 
 // FP64 loop: WHILE { U x [red half-stencil (RB), stencil, patch, update]; true-residual check }
 vofp_status build_graph_fp64(vofp_ctx* c, int U, bool rb) {
@@ -1095,8 +1095,13 @@ vofp_status solve_pass(vofp_ctx* c, const double* b, double* x, const vofp_solve
     vofp_status s = ensure_workspace(c);
     if (s) return s;
     // colour-compact vectors of the red-black inner solve (built once per operator)
+    if (o->mode == VOFP_MODE_MIXED && o->precond == VOFP_PRECOND_RBSGS && (s = rbc_ensure(c))) return s;
     // and the hierarchy of its coarse-grid correction
-    if (o->mode == VOFP_MODE_MIXED && o->precond == VOFP_PRECOND_RBSGS && ((s = rbc_ensure(c)) || (s = mg_ensure(c)))) return s;
+    c->mg_use = false;
+    if (o->mode == VOFP_MODE_MIXED && o->precond == VOFP_PRECOND_RBSGS && mg_wanted(c, o->rtol)) {
+        if ((s = mg_ensure(c))) return s;
+        c->mg_use = c->mg_ok;
+    }
     const long long N = c->d.n;
     cudaStream_t st = c->stream;
     // Default: the FP64 loop checks its true residual every 8 iterations, and so does the mixed
@@ -1107,7 +1112,7 @@ vofp_status solve_pass(vofp_ctx* c, const double* b, double* x, const vofp_solve
     // an inner solve can reach the FP32 rounding floor within 64 iterations, and the steps taken
     // there, kept as the next inner solve's direction, stalled it (a 16^3 sphere, Jacobi: 100032
     // iterations without converging).
-    const bool mg = o->mode == VOFP_MODE_MIXED && o->precond == VOFP_PRECOND_RBSGS && c->mg_ok;
+    const bool mg = c->mg_use;
     // With the coarse-grid correction an inner solve takes 10-20 iterations at any size: every 16 from
     // 2^16 cells on (512x256x128 to 1e-12: 106 ms, 110 testing every 8, 115 every 32), 8 below, where
     // 16 already reach the FP32 floor of the smallest grids.
@@ -1263,8 +1268,7 @@ vofp_status solve(vofp_ctx* c, const double* b, double* x, const vofp_solve_opts
     vofp_solve_info acc{};
     vofp_status r = solve_pass(c, b, x, o, &acc);
     const long long max_iter = o->max_iter > 0 ? o->max_iter : 100000;
-    if (r == VOFP_ERR_BREAKDOWN && c->mg_ok && o->mode == VOFP_MODE_MIXED && o->precond == VOFP_PRECOND_RBSGS &&
-        std::isfinite(acc.rel_residual) && acc.iterations < max_iter) {
+    if (r == VOFP_ERR_BREAKDOWN && c->mg_use && std::isfinite(acc.rel_residual) && acc.iterations < max_iter) {
         // the coarse-grid correction lost positivity: the plain red-black iteration from the iterate
         c->mg_ok = false;
         vofp_solve_opts o2 = *o;
