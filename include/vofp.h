@@ -286,7 +286,7 @@ vofp_status vofp_vof_flux_correct(vofp_ctx* ctx, const double* ax, const double*
  *                and vofp_rhs_from_face_velocity); vol_frac device, cells.
  *   dt > 0, order 0 or 1.
  *   F_out        device, cells; may be F itself.
- * Scratch (allocated on the first call, kept by the context): about 9 doubles per cell.
+ * Scratch (allocated on the first call, kept by the context): about 11 doubles per cell.
  * Needs a context (grid), not a built operator. */
 vofp_status vofp_vof_advect(vofp_ctx* ctx, const double* F, const double* ax, const double* ay,
                             const double* az, const double* vol_frac, const double* u, const double* v,

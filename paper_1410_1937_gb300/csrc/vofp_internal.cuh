@@ -196,8 +196,8 @@ struct vofp_ctx {
     // VOF operator (vofp_vof.cu): corrected stage velocities, two stage buffers, interface planes
     double *vof_uxh = nullptr, *vof_uyh = nullptr, *vof_wmh = nullptr, *vof_wph = nullptr;
     double *vof_phi = nullptr, *vof_plic = nullptr;
-    int* vof_list = nullptr;          // cells with 0 < phi < 1 of the coming stage
-    double* vof_rec = nullptr;        // 1 / width of the cells along x, y, z
+    int* vof_list = nullptr;          // cells with 0 < phi < 1 of the coming stage, then the stage's other cells
+    double* vof_rec = nullptr;        // tables along x, y, z: 1 / width, -1/16 over the neighbours' distance
     uint32_t* vof_lim = nullptr;      // high words of 0.49 width / dt
     unsigned int* vof_count = nullptr;   // list lengths per stage
     double* rk2_buf = nullptr;        // RK2 step (vofp_rk2.cu): face fields and cell arrays
