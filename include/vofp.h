@@ -102,10 +102,10 @@ typedef struct {
  *               coefficients and vectors and FP64-accumulated dot products.
  *   precond     VOFP_PRECOND_JACOBI (diagonal) or VOFP_PRECOND_RBSGS (red-black symmetric
  *               Gauss-Seidel, applied as CG on the black unknowns after eliminating the red ones
- *               (Eisenstat's form); both modes, and the bench default in mixed mode).  In mixed
- *               mode, from 2^16 cells and for rtol <= 1e-7, its inner CG also has a coarse-grid
- *               correction: an additive V-cycle on 2x2x2 aggregates smoothed by red-black
- *               Gauss-Seidel.
+ *               (Eisenstat's form); both modes, and the bench default in mixed mode).  From 2^16
+ *               cells and for rtol <= 1e-7 its CG also has a coarse-grid correction: an additive
+ *               V-cycle on 2x2x2 aggregates smoothed by red-black Gauss-Seidel (in the precision
+ *               of the iteration's vectors).
  *   rtol        the solve returns VOFP_OK only when the residual recomputed from the returned x,
  *               ||b_hat - A_hat x|| (2-norm over the unknowns, FP64), is at most rtol ||b_hat||.
  *               The iteration aims slightly below rtol; when the recomputed residual is still

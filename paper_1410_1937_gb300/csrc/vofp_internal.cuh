@@ -73,14 +73,25 @@ struct Dims {
 
 // One level of the coarse-grid correction (vofp_mg.cu): coefficients of each cell's + faces, inverse
 // diagonal, the part of the diagonal that belongs to p = 0 domain faces, right-hand side, solution.
+template <typename T>
 struct MgLevel {
     int nx, ny, nz;
     long long n;
-    float *tx, *ty, *tz, *di, *ex, *b, *x;
+    T *tx, *ty, *tz, *di, *ex, *b, *x;
 };
-// smallest grid whose mixed red-black solve takes the coarse-grid correction: from here on it is 1.5 to
-// 5 times faster than the plain iteration (64x48x40 to 1e-12: 12 against 19 ms); at 16^3 to 48x40x32
-// the two took about the same to 1.4 times
+// The hierarchy of one precision: levels, weights and z of the iteration's vectors, and per merge group
+// the master's entry and its aggregate.
+template <typename T>
+struct MgSet {
+    bool built = false, ok = false;   // looked at / usable for the current operator
+    std::vector<MgLevel<T>> lv;
+    T *w = nullptr, *z = nullptr;
+    int* rep = nullptr;
+    long long cap = 0, rep_cap = 0;
+};
+// smallest grid whose red-black solves take the coarse-grid correction: from here on they are 1.1 to
+// 5 times faster than the plain iteration (64x48x40 to 1e-12, mixed: 12 against 19 ms, FP64: 16.2 against
+// 18.4); from 16^3 to 48x40x32 the mixed ones took 0.7 to 1 of its time, the FP64 ones 0.9 to 1.15
 constexpr long long kMgMinCells = 1 << 16;
 // ... and the loosest tolerance that does.  The correction is the faster one at every tolerance (256x128x64
 // to 1e-6: 13.9 against 39.4 ms, 512x256x128 49 against 232 ms), but a pressure solved more loosely is
@@ -206,15 +217,12 @@ struct vofp_ctx {
     int rbc_rpt = 2;                  // rows per thread of the compact iteration kernel (tile 32 x 8 rpt)
     int rbc_nblocks = 0;              // iteration kernel blocks and work split (see rbc_split)
     vofp::RbcSplit rbc_split{};
-    // coarse-grid correction of the mixed red-black solve (vofp_mg.cu)
-    bool mg_built = false, mg_ok = false;   // looked at / usable for the current operator
-    bool mg_use = false;                    // in use in the current solve
-    std::vector<vofp::MgLevel> mg;
-    float *mg_w = nullptr, *mg_z = nullptr; // weights and z of the inner vectors
+    // coarse-grid correction of the red-black solves (vofp_mg.cu)
+    vofp::MgSet<float> mgf;           // mixed mode
+    vofp::MgSet<double> mgd;          // FP64 mode
+    bool mg_use = false;              // in use in the current solve
     uint32_t* mg_mask = nullptr;      // per aggregate (a byte): its even cells that are group masters
     int* mg_even = nullptr;           // their entries, four per aggregate
-    int* mg_rep = nullptr;            // per merge group: the master's entry and its aggregate
-    long long mg_cap = 0, mg_rep_cap = 0;
     unsigned long long* mg_dmax = nullptr;
     int tma_blocks_deep32 = 0;        // resident blocks per SM of the six-stage FP32 stencil
     int rb_tma_blocks_per_sm = 0;
@@ -257,12 +265,12 @@ void rbc_iteration(vofp_ctx* c, cudaStream_t st, const float* po, float* pn, cud
                    int use_h);
 void rbc_finish_xf(vofp_ctx* c, cudaStream_t st);                 // xf (full grid) = x_c + alpha p0_c
 int rbc_pq_parts(const vofp_ctx* c);   // block partials of p.Ap the compact iteration leaves for the update
-// coarse-grid correction of the mixed red-black solve (vofp_mg.cu)
-bool mg_wanted(const vofp_ctx* c, double rtol);   // whether a mixed red-black solve takes it
-vofp_status mg_ensure(vofp_ctx* c);    // hierarchy of the current operator; sets c->mg_ok
-void mg_precondition(vofp_ctx* c, cudaStream_t st, bool pdl, int start);   // z and beta from r
-void mg_update(vofp_ctx* c, cudaStream_t st, bool pdl, cudaGraphConditionalHandle h, int use_h);
-int mg_precondition_kernels(const vofp_ctx* c);
+// coarse-grid correction of the red-black solves (vofp_mg.cu)
+bool mg_wanted(const vofp_ctx* c, double rtol);   // whether a red-black solve takes it
+vofp_status mg_ensure(vofp_ctx* c, bool fp64);    // hierarchy of the current operator; sets mgf.ok / mgd.ok
+void mg_precondition(vofp_ctx* c, cudaStream_t st, bool fp64, bool pdl, int start);   // z and beta from r
+void mg_update(vofp_ctx* c, cudaStream_t st, bool fp64, bool pdl, cudaGraphConditionalHandle h, int use_h);
+int mg_precondition_kernels(const vofp_ctx* c, bool fp64);
 void rbc_time_kernel(vofp_ctx* c, cudaStream_t st);               // one iteration kernel launch
 void rbc_time_aux(vofp_ctx* c, cudaStream_t st);                  // the exception and group kernels of one iteration
 template <typename V>

@@ -1,4 +1,4 @@
-// Coarse-grid correction of the red-black preconditioner in mixed mode.
+// Coarse-grid correction of the red-black preconditioner (templated on the precision of the iteration).
 //
 // CG on the red Schur complement (vofp_rbc.cuh, vofp_rb.cuh) has a residual r on the black unknowns
 // and no preconditioner of its own; its iteration count grows with the grid (2500 at 512x256x128 to
@@ -15,7 +15,9 @@
 // B is additive (z = r + B r, no second fine-grid sweep), so the fine grid costs one pass more over r
 // and the weights sq, and r.z = r.r + e_1.b_1 comes from the coarse vectors.  Measured (solves to
 // 1e-12, the plain iteration and with the correction): 512x256x128 5120 iterations in 574 ms, 432 in
-// 106 ms; 256x128x64 2368 in 86 ms, 336 in 25.6 ms; 64x48x40 832 in 18.7 ms, 272 in 12 ms.
+// 106 ms; 256x128x64 2368 in 86 ms, 336 in 25.6 ms; 64x48x40 832 in 18.7 ms, 272 in 12 ms.  FP64 mode
+// (hierarchy and vectors in FP64): 512x256x128 3248 iterations in 2178 ms, 416 in 411 ms; 128x64x64 872 in
+// 43.7 ms, 216 in 20 ms; 125x61x47 792 in 34.7 ms, 232 in 20.7 ms.
 //
 // Merge groups: the group's unknown is present at every member cell of the expanded vectors.  Its
 // master represents it in the restriction (weight sq); the other members, small cells whose own
@@ -38,9 +40,9 @@ constexpr int kPqBase = 3 * (kMaxPartials / 4);   // the compact iteration's blo
 constexpr int kBottomCells = 512;
 constexpr int kBottomThreads = 512;
 constexpr int kMaxBottom = 10;                    // levels from kBottomCells down to one cell
-// a level has at most half the cells (rounded up) of the one above: their sum is below this
-constexpr int kBottomFloats = 6 * (2 * kBottomCells + kMaxBottom);
-static_assert(kBottomFloats * sizeof(float) <= 48 * 1024, "static shared memory");
+// six values per cell; every chain of levels from at most 512 cells down has at most 1023 in all
+constexpr int kBottomValues = 6 * 2 * kBottomCells;
+static_assert(kBottomValues * sizeof(double) <= 48 * 1024, "static shared memory");
 
 int grid_n(long long n) {
     return (int)std::max(1LL, std::min((n + kNT - 1) / kNT, (long long)num_sms() * 8));
@@ -68,16 +70,17 @@ __device__ __forceinline__ int mg_exponent(const unsigned long long* dmax) {
     return (m > 0.0 && isfinite(m)) ? (ilogb(m) >> 1) : 0;
 }
 
+template <typename T>
 struct MgCoef {
-    const float *tx, *ty, *tz, *di;
+    const T *tx, *ty, *tz, *di;
 };
 
 // level 1 from the FP64 operator
+template <typename T>
 __global__ void k_mg_coarsen_fine(Dims d, int nx1, int ny1, int nz1, const double* __restrict__ Tx,
                                   const double* __restrict__ Ty, const double* __restrict__ Tz,
                                   const double* __restrict__ diag, const unsigned long long* dmax,
-                                  float* __restrict__ tx, float* __restrict__ ty, float* __restrict__ tz,
-                                  float* __restrict__ ex) {
+                                  T* __restrict__ tx, T* __restrict__ ty, T* __restrict__ tz, T* __restrict__ ex) {
     const long long n1 = (long long)nx1 * ny1 * nz1;
     const double g = scalbn(1.0, -2 * mg_exponent(dmax));
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n1; q += (long long)gridDim.x * blockDim.x) {
@@ -99,17 +102,18 @@ __global__ void k_mg_coarsen_fine(Dims d, int nx1, int ny1, int nz1, const doubl
                     if (j & 1) sy += y;
                     if (k & 1) sz += z;
                 }
-        tx[q] = (float)(sx * g);
-        ty[q] = (float)(sy * g);
-        tz[q] = (float)(sz * g);
-        ex[q] = (float)(se * g);
+        tx[q] = (T)(sx * g);
+        ty[q] = (T)(sy * g);
+        tz[q] = (T)(sz * g);
+        ex[q] = (T)(se * g);
     }
 }
 
-__global__ void k_mg_coarsen(int nx, int ny, int nz, const float* __restrict__ tx, const float* __restrict__ ty,
-                             const float* __restrict__ tz, const float* __restrict__ ex, int nx1, int ny1, int nz1,
-                             float* __restrict__ ctx, float* __restrict__ cty, float* __restrict__ ctz,
-                             float* __restrict__ cex) {
+template <typename T>
+__global__ void k_mg_coarsen(int nx, int ny, int nz, const T* __restrict__ tx, const T* __restrict__ ty,
+                             const T* __restrict__ tz, const T* __restrict__ ex, int nx1, int ny1, int nz1,
+                             T* __restrict__ ctx, T* __restrict__ cty, T* __restrict__ ctz,
+                             T* __restrict__ cex) {
     const long long n1 = (long long)nx1 * ny1 * nz1;
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n1; q += (long long)gridDim.x * blockDim.x) {
         const int I = int(q % nx1), J = int((q / nx1) % ny1), K = int(q / ((long long)nx1 * ny1));
@@ -123,16 +127,17 @@ __global__ void k_mg_coarsen(int nx, int ny, int nz, const float* __restrict__ t
                     if (j & 1) sy += (double)ty[c];
                     if (k & 1) sz += (double)tz[c];
                 }
-        ctx[q] = (float)sx;
-        cty[q] = (float)sy;
-        ctz[q] = (float)sz;
-        cex[q] = (float)se;
+        ctx[q] = (T)sx;
+        cty[q] = (T)sy;
+        ctz[q] = (T)sz;
+        cex[q] = (T)se;
     }
 }
 
 // inverse diagonals of a level from its stored coefficients (0 where a cell has no coupling)
-__global__ void k_mg_dinv(int nx, int ny, int nz, const float* __restrict__ tx, const float* __restrict__ ty,
-                          const float* __restrict__ tz, const float* __restrict__ ex, float* __restrict__ di) {
+template <typename T>
+__global__ void k_mg_dinv(int nx, int ny, int nz, const T* __restrict__ tx, const T* __restrict__ ty,
+                          const T* __restrict__ tz, const T* __restrict__ ex, T* __restrict__ di) {
     const long long n = (long long)nx * ny * nz, pl = (long long)nx * ny;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
         const int i = int(c % nx), j = int((c / nx) % ny), k = int(c / pl);
@@ -140,29 +145,29 @@ __global__ void k_mg_dinv(int nx, int ny, int nz, const float* __restrict__ tx, 
         if (i > 0) s += (double)tx[c - 1];
         if (j > 0) s += (double)ty[c - nx];
         if (k > 0) s += (double)tz[c - pl];
-        di[c] = s > 1e-30 ? (float)(1.0 / s) : 0.0f;
+        di[c] = s > 1e-30 ? (T)(1.0 / s) : T(0);
     }
 }
 
 // weights of the vector entries (before the merge groups): sq of a non-red cell with an unknown, 0
 // of the others; on the compact vectors entries past N/2 belong to group members (-1)
-template <bool COMPACT>
+template <bool COMPACT, typename T>
 __global__ void k_mg_weights(Dims d, long long n, long long nh, const double* __restrict__ sq,
                              const int32_t* __restrict__ root, const uint32_t* __restrict__ red,
-                             const unsigned long long* dmax, float* __restrict__ w) {
+                             const unsigned long long* dmax, T* __restrict__ w) {
     const double g = scalbn(1.0, -mg_exponent(dmax));
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
         if (COMPACT) {
             if (t >= nh) {
-                w[t] = -1.0f;
+                w[t] = T(-1);
                 continue;
             }
             const long long row = t / (d.nx >> 1);
             const int j = int(row % d.ny), k = int(row / d.ny);
             const long long c = 2 * t + 1 - ((j + k) & 1);   // black cell of pair t
-            w[t] = root[c] < 0 ? 0.0f : (float)(sq[c] * g);
+            w[t] = root[c] < 0 ? T(0) : (T)(sq[c] * g);
         } else {
-            w[t] = (root[t] < 0 || is_slave(red, t)) ? 0.0f : (float)(sq[t] * g);
+            w[t] = (root[t] < 0 || is_slave(red, t)) ? T(0) : (T)(sq[t] * g);
         }
     }
 }
@@ -170,17 +175,17 @@ __global__ void k_mg_weights(Dims d, long long n, long long nh, const double* __
 // merge groups: the master's entry and aggregate (rep) and its weight, -1 for the other members; on the
 // compact vectors the aggregates' mask bits of even-parity masters and their entries, four per aggregate
 // (read, and written, only where the bit is set).  Member entries: gref (compact) or the cells
-template <bool COMPACT>
+template <bool COMPACT, typename T>
 __global__ void k_mg_groups(Dims d, int ng, int nx1, int ny1, const int* __restrict__ gptr,
                             const int* __restrict__ gcells, const int* __restrict__ gref,
-                            const double* __restrict__ sq, const unsigned long long* dmax, float* __restrict__ w,
+                            const double* __restrict__ sq, const unsigned long long* dmax, T* __restrict__ w,
                             int2* __restrict__ rep, uint32_t* __restrict__ mask, int* __restrict__ even) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= ng) return;
     const double sg = scalbn(1.0, -mg_exponent(dmax));
     const int u0 = gptr[g], u1 = gptr[g + 1];
     for (int u = u0; u < u1; ++u)
-        w[COMPACT ? gref[u] : gcells[u]] = u == u0 ? (float)(sq[gcells[u]] * sg) : -1.0f;
+        w[COMPACT ? gref[u] : gcells[u]] = u == u0 ? (T)(sq[gcells[u]] * sg) : T(-1);
     int i, j, k;
     cell_ijk(d, gcells[u0], i, j, k);
     const int t = (i >> 1) + nx1 * ((j >> 1) + ny1 * (k >> 1)), u = 2 * (k & 1) + (j & 1);
@@ -200,7 +205,6 @@ template <bool COMPACT>
 struct MgEntries {
     static constexpr int A = COMPACT ? 2 : 1;
     static constexpr int W = COMPACT ? 4 : 8;       // words of a thread
-    using Word = typename std::conditional<COMPACT, float2, float>::type;
     long long at[W];
     bool in[W];
     __device__ __forceinline__ void set(const Dims& d, int I, int J, int K) {
@@ -214,27 +218,30 @@ struct MgEntries {
         }
     }
 };
-__device__ __forceinline__ void mg_get(float (&v)[2], const float* __restrict__ a, long long at, float2) {
+// one word of A values (two floats: an 8-byte word)
+__device__ __forceinline__ void mg_get(float (&v)[2], const float* a, long long at) {
     const float2 x = *reinterpret_cast<const float2*>(a + at);
     v[0] = x.x;
     v[1] = x.y;
 }
-__device__ __forceinline__ void mg_get(float (&v)[1], const float* __restrict__ a, long long at, float) { v[0] = a[at]; }
-__device__ __forceinline__ void mg_put(const float (&v)[2], float* __restrict__ a, long long at) {
+template <typename T>
+__device__ __forceinline__ void mg_get(T (&v)[1], const T* a, long long at) { v[0] = a[at]; }
+__device__ __forceinline__ void mg_put(const float (&v)[2], float* a, long long at) {
     *reinterpret_cast<float2*>(a + at) = make_float2(v[0], v[1]);
 }
-__device__ __forceinline__ void mg_put(const float (&v)[1], float* __restrict__ a, long long at) { a[at] = v[0]; }
+template <typename T>
+__device__ __forceinline__ void mg_put(const T (&v)[1], T* a, long long at) { a[at] = v[0]; }
 
 // alpha = r.z / p.Ap;  r -= alpha q;  r.r;  b_1 = restriction of the new r.  With UPD = false only the
 // restriction (the start of an inner solve, whose r and r.r are there).  Memory-bound (8.6 bytes per
 // cell on the compact vectors: 31 us at 512x256x128 under ncu, 43 with 4-byte words): a thread takes two
 // aggregates along x at a time there (12 independent 8-byte loads), the first ones before it sums p.Ap
 // and divides.
-template <bool COMPACT, bool UPD>
+template <bool COMPACT, bool UPD, typename T>
 __global__ void __launch_bounds__(kNT, 3)
 k_mg_update(const Dims d, const int nx1, const int ny1, const int n1, const long long nh, const long long nvec,
-            float* __restrict__ r, const float* __restrict__ q, const float* __restrict__ w,
-            const uint8_t* __restrict__ mask, const int* __restrict__ even, float* __restrict__ b1, CgScalars* sc,
+            T* __restrict__ r, const T* __restrict__ q, const T* __restrict__ w,
+            const uint8_t* __restrict__ mask, const int* __restrict__ even, T* __restrict__ b1, CgScalars* sc,
             double* __restrict__ partials, unsigned int* __restrict__ counter,
             cudaGraphConditionalHandle handle, int use_handle, const double* __restrict__ pq_part, int npq) {
     using En = MgEntries<COMPACT>;
@@ -246,7 +253,7 @@ k_mg_update(const Dims d, const int nx1, const int ny1, const int n1, const long
     const int stride = gridDim.x * kNT, items = n1 / A, nxa = nx1 / A;
     int t = blockIdx.x * kNT + threadIdx.x;
     En en;
-    float rv[W][A], qv[W][A], wv[W][A];
+    T rv[W][A], qv[W][A], wv[W][A];
     uint32_t mk = 0;
     auto load = [&]() {
         const int tj = t / nxa, K = tj / ny1;
@@ -255,13 +262,13 @@ k_mg_update(const Dims d, const int nx1, const int ny1, const int n1, const long
         for (int e = 0; e < W; ++e) {
 #pragma unroll
             for (int a = 0; a < A; ++a) {
-                rv[e][a] = qv[e][a] = 0.0f;
-                wv[e][a] = -1.0f;
+                rv[e][a] = qv[e][a] = T(0);
+                wv[e][a] = T(-1);
             }
             if (!en.in[e]) continue;
-            mg_get(rv[e], r, en.at[e], typename En::Word());
-            if (UPD) mg_get(qv[e], q, en.at[e], typename En::Word());
-            mg_get(wv[e], w, en.at[e], typename En::Word());
+            mg_get(rv[e], r, en.at[e]);
+            if (UPD) mg_get(qv[e], q, en.at[e]);
+            mg_get(wv[e], w, en.at[e]);
         }
         if (COMPACT) mk = *reinterpret_cast<const uint16_t*>(mask + (long long)A * t);
     };
@@ -288,20 +295,20 @@ k_mg_update(const Dims d, const int nx1, const int ny1, const int n1, const long
         }
         __syncthreads();
     }
-    const float na = UPD ? -(float)s_alpha : 0.0f;
-    AccF2 acc;
+    const T na = UPD ? -(T)s_alpha : T(0);
+    typename AccFor<T>::type acc;
     while (t < items) {
-        float b[A];
+        T b[A];
 #pragma unroll
-        for (int a = 0; a < A; ++a) b[a] = 0.0f;
+        for (int a = 0; a < A; ++a) b[a] = T(0);
 #pragma unroll
         for (int e = 0; e < W; ++e) {
 #pragma unroll
             for (int a = 0; a < A; ++a) {
-                if (UPD) rv[e][a] = __fmaf_rn(na, qv[e][a], rv[e][a]);
-                if (wv[e][a] >= 0.0f) {
+                if (UPD) rv[e][a] = fmav(na, qv[e][a], rv[e][a]);
+                if (wv[e][a] >= T(0)) {
                     if (UPD) acc.add(rv[e][a], rv[e][a]);
-                    b[a] = __fmaf_rn(wv[e][a], rv[e][a], b[a]);
+                    b[a] = fmav(wv[e][a], rv[e][a], b[a]);
                 }
             }
             if (UPD && en.in[e]) mg_put(rv[e], r, en.at[e]);
@@ -310,15 +317,15 @@ k_mg_update(const Dims d, const int nx1, const int ny1, const int n1, const long
             // even-parity masters of these aggregates (rare)
             for (; mk; mk &= mk - 1) {
                 const int f = __ffs(mk) - 1, a = f >> 3, at = even[4 * ((long long)A * t + a) + (f & 7)];
-                float v = r[at];
+                T v = r[at];
                 if (UPD) {
-                    v = __fmaf_rn(na, q[at], v);
+                    v = fmav(na, q[at], v);
                     r[at] = v;
                     acc.add(v, v);
                 }
-                const float s = w[at] * v;
-                b[0] += a == 0 ? s : 0.0f;
-                b[A - 1] += a == A - 1 && A > 1 ? s : 0.0f;
+                const T s = w[at] * v;
+                b[0] += a == 0 ? s : T(0);
+                b[A - 1] += a == A - 1 && A > 1 ? s : T(0);
             }
         }
         mg_put(b, b1, (long long)A * t);
@@ -329,7 +336,7 @@ k_mg_update(const Dims d, const int nx1, const int ny1, const int n1, const long
     // the other even-parity members of merge groups (copies: not in the sums)
     if (COMPACT)
         for (long long c = nh + blockIdx.x * kNT + threadIdx.x; c < nvec; c += stride)
-            if (w[c] < 0.0f) r[c] = __fmaf_rn(na, q[c], r[c]);
+            if (w[c] < T(0)) r[c] = fmav(na, q[c], r[c]);
     double tot;
     if (grid_reduce(acc.value(), partials, counter, sh, &tot)) {
         const bool broke = s_flags != 0;
@@ -352,38 +359,38 @@ k_mg_update(const Dims d, const int nx1, const int ny1, const int n1, const long
 
 // z = r + sq e_1 and r.z = r.r + e_1.b_1; beta of the next direction.  Merge groups: every member
 // takes the master's z (formed here from r: no order between the two loops).
-template <bool COMPACT>
+template <bool COMPACT, typename T>
 __global__ void __launch_bounds__(kNT, 3)
-k_mg_direction(const Dims d, const int nx1, const int ny1, const int n1, const float* __restrict__ r,
-               const float* __restrict__ w, const float* __restrict__ e1, const float* __restrict__ b1,
-               float* __restrict__ z, const int ng, const int2* __restrict__ rep, const int* __restrict__ gptr,
+k_mg_direction(const Dims d, const int nx1, const int ny1, const int n1, const T* __restrict__ r,
+               const T* __restrict__ w, const T* __restrict__ e1, const T* __restrict__ b1,
+               T* __restrict__ z, const int ng, const int2* __restrict__ rep, const int* __restrict__ gptr,
                const int* __restrict__ gidx, CgScalars* sc, double* __restrict__ partials,
                unsigned int* __restrict__ counter, int start) {
     using En = MgEntries<COMPACT>;
     constexpr int A = En::A, W = En::W;
     __shared__ double sh[32];
     grid_dep_wait();
-    AccF2 acc;
+    typename AccFor<T>::type acc;
     const int stride = gridDim.x * kNT, items = n1 / A, nxa = nx1 / A;
     // the groups first, from the last blocks: their chain of loads overlaps the stream
     for (int g = (gridDim.x - 1 - blockIdx.x) * kNT + threadIdx.x; g < ng; g += stride) {
         const int2 m = rep[g];
         const int u0 = gptr[g], u1 = gptr[g + 1];
-        const float v = __fmaf_rn(w[m.x], e1[m.y], r[m.x]);
+        const T v = fmav(w[m.x], e1[m.y], r[m.x]);
         for (int u = u0; u < u1; ++u) z[gidx[u]] = v;
     }
     for (int t = blockIdx.x * kNT + threadIdx.x; t < items; t += stride) {
         const int tj = t / nxa, K = tj / ny1;
         En en;
         en.set(d, (t - tj * nxa) * A, tj - K * ny1, K);
-        float ev[A], bv[A], rv[W][A], wv[W][A];
-        mg_get(ev, e1, (long long)A * t, typename En::Word());
-        mg_get(bv, b1, (long long)A * t, typename En::Word());
+        T ev[A], bv[A], rv[W][A], wv[W][A];
+        mg_get(ev, e1, (long long)A * t);
+        mg_get(bv, b1, (long long)A * t);
 #pragma unroll
         for (int e = 0; e < W; ++e)
             if (en.in[e]) {
-                mg_get(rv[e], r, en.at[e], typename En::Word());
-                mg_get(wv[e], w, en.at[e], typename En::Word());
+                mg_get(rv[e], r, en.at[e]);
+                mg_get(wv[e], w, en.at[e]);
             }
 #pragma unroll
         for (int a = 0; a < A; ++a) acc.add(ev[a], bv[a]);
@@ -391,18 +398,18 @@ k_mg_direction(const Dims d, const int nx1, const int ny1, const int n1, const f
         for (int e = 0; e < W; ++e) {
             if (!en.in[e]) continue;
             bool all = true;
-            float v[A];
+            T v[A];
 #pragma unroll
             for (int a = 0; a < A; ++a) {
-                all &= wv[e][a] >= 0.0f;
-                v[a] = __fmaf_rn(wv[e][a], ev[a], rv[e][a]);
+                all &= wv[e][a] >= T(0);
+                v[a] = fmav(wv[e][a], ev[a], rv[e][a]);
             }
             if (all) {
                 mg_put(v, z, en.at[e]);
             } else {   // a group member beside it: written below
 #pragma unroll
                 for (int a = 0; a < A; ++a)
-                    if (wv[e][a] >= 0.0f) z[en.at[e] + a] = v[a];
+                    if (wv[e][a] >= T(0)) z[en.at[e] + a] = v[a];
             }
         }
     }
@@ -441,14 +448,15 @@ struct MgGeom {
 };
 
 // One cell of a step: its place in the tile, and what its sum over the faces takes.
+template <typename T>
 struct MgCell {
     int at;              // index in the tile; -1: none
     long long c;         // cell; -1 outside the grid
-    float xp, xm, yp, ym, zp, zm;
-    __device__ __forceinline__ void load(const MgGeom& g, const MgCoef& m, int i, int j, int k) {
+    T xp, xm, yp, ym, zp, zm;
+    __device__ __forceinline__ void load(const MgGeom& g, const MgCoef<T>& m, int i, int j, int k) {
         const long long pl = (long long)g.nx * g.ny;
         c = -1;
-        xp = xm = yp = ym = zp = zm = 0.0f;
+        xp = xm = yp = ym = zp = zm = T(0);
         if (i < 0 || i >= g.nx || j < 0 || j >= g.ny || k < 0 || k >= g.nz) return;
         c = i + g.nx * (long long)j + pl * k;
         xp = m.tx[c];                            // 0 for the last cell of a row
@@ -458,32 +466,32 @@ struct MgCell {
         if (j > 0) ym = m.ty[c - g.nx];
         if (k > 0) zm = m.tz[c - pl];
     }
-    __device__ __forceinline__ float sum(const float* xs) const {
-        const float* p = xs + at;
-        float s = xp * p[1];
-        s = __fmaf_rn(xm, p[-1], s);
-        s = __fmaf_rn(yp, p[kPX], s);
-        s = __fmaf_rn(ym, p[-kPX], s);
-        s = __fmaf_rn(zp, p[kPX * kPY], s);
-        return __fmaf_rn(zm, p[-kPX * kPY], s);
+    __device__ __forceinline__ T sum(const T* xs) const {
+        const T* p = xs + at;
+        T s = xp * p[1];
+        s = fmav(xm, p[-1], s);
+        s = fmav(yp, p[kPX], s);
+        s = fmav(ym, p[-kPX], s);
+        s = fmav(zp, p[kPX * kPY], s);
+        return fmav(zm, p[-kPX * kPY], s);
     }
 };
 
 // DOWN (before the next level): red cells from b alone (the first guess is 0), black cells, and the
 // red cells' residual, summed over each aggregate into the next level's b (the black cells' residual
 // is 0).  Else (after it): red cells from b and the next level's x, black cells, red cells; x.
-template <bool DOWN>
+template <bool DOWN, typename T>
 __global__ void __launch_bounds__(kTileThreads, 2)
-k_mg_level(const MgGeom g, const MgCoef m, const float* __restrict__ b, const float* __restrict__ en,
-           float* __restrict__ out) {
-    __shared__ float xs[kPX * kPY * kPZ];
+k_mg_level(const MgGeom g, const MgCoef<T> m, const T* __restrict__ b, const T* __restrict__ en,
+           T* __restrict__ out) {
+    __shared__ T xs[kPX * kPY * kPZ];
     const int t = threadIdx.x;
     const int tb = blockIdx.x, bx = tb % g.tiles_x, by = (tb / g.tiles_x) % g.tiles_y, bz = tb / (g.tiles_x * g.tiles_y);
     const int i0 = bx * kTX, j0 = by * kTY, k0 = bz * kTZ;
     // black cell of the pair (i0 - 1 + 2a, + 1): the sum of its coordinates is odd
-    MgCell bc, rc;
+    MgCell<T> bc, rc;
     bc.at = rc.at = -1;
-    float bd = 0.0f, bb = 0.0f, rd = 0.0f, rb = 0.0f;
+    T bd = T(0), bb = T(0), rd = T(0), rb = T(0);
     if (t < kBlacks) {
         const int a = t % (kTX / 2 + 1), y = (t / (kTX / 2 + 1)) % (kTY + 2), z = t / ((kTX / 2 + 1) * (kTY + 2));
         const int j = j0 - 1 + y, k = k0 - 1 + z, x = 2 * a + ((j + k) & 1);
@@ -502,13 +510,13 @@ k_mg_level(const MgGeom g, const MgCoef m, const float* __restrict__ b, const fl
     }
     int at[2];
     long long hc[2], he[2];
-    float hd[2];
+    T hd[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
         const int u = t + q * kTileThreads;
         at[q] = -1;
         hc[q] = -1;
-        hd[q] = 0.0f;
+        hd[q] = T(0);
         if (u >= kReds) continue;
         const int a = u % (kPX / 2), y = (u / (kPX / 2)) % kPY, z = u / (kPX / 2 * kPY);
         const int j = j0 - 2 + y, k = k0 - 2 + z, x = 2 * a + ((j + k) & 1), i = i0 - 2 + x;
@@ -526,15 +534,15 @@ k_mg_level(const MgGeom g, const MgCoef m, const float* __restrict__ b, const fl
 #pragma unroll
     for (int q = 0; q < 2; ++q)
         if (at[q] >= 0) {
-            float v = 0.0f;
-            if (hc[q] >= 0) v = DOWN ? hd[q] * b[hc[q]] : __fmaf_rn(hd[q], b[hc[q]], en[he[q]]);
+            T v = T(0);
+            if (hc[q] >= 0) v = DOWN ? hd[q] * b[hc[q]] : fmav(hd[q], b[hc[q]], en[he[q]]);
             xs[at[q]] = v;
         }
     __syncthreads();
-    if (bc.at >= 0) xs[bc.at] = bc.c >= 0 ? bd * (bb + bc.sum(xs)) : 0.0f;
+    if (bc.at >= 0) xs[bc.at] = bc.c >= 0 ? bd * (bb + bc.sum(xs)) : T(0);
     __syncthreads();
     if (t >= kCore) return;
-    float s = rc.c >= 0 ? rc.sum(xs) : 0.0f;
+    T s = rc.c >= 0 ? rc.sum(xs) : T(0);
     if (DOWN) {
         s += __shfl_xor_sync(0xffffffffu, s, 1);
         s += __shfl_xor_sync(0xffffffffu, s, 2);
@@ -559,18 +567,18 @@ constexpr int kLargeThreads = 256;
 constexpr long long kLargeCells = 600 * 1000;
 static_assert(kRX / 2 * kRY <= kLargeThreads && kLX / 2 * kLY * 2 == kLargeThreads, "columns per block");
 
-template <bool DOWN, bool INNER>
-__device__ __forceinline__ void large_sweep(const MgGeom& g, const MgCoef& m, const float* __restrict__ b,
-                                            const float* __restrict__ en, float* __restrict__ out, float* xs, int i0,
+template <bool DOWN, bool INNER, typename T>
+__device__ __forceinline__ void large_sweep(const MgGeom& g, const MgCoef<T>& m, const T* __restrict__ b,
+                                            const T* __restrict__ en, T* __restrict__ out, T* xs, int i0,
                                             int j0, int k0) {
     const int t = threadIdx.x, nx = g.nx, pl = g.nx * g.ny;
-    auto face_sum = [&](int c, int i, int j, int k, const float* p) {
-        float s = m.tx[c] * p[1];
-        if (INNER || i > 0) s = __fmaf_rn(m.tx[c - 1], p[-1], s);
-        s = __fmaf_rn(m.ty[c], p[kRX], s);
-        if (INNER || j > 0) s = __fmaf_rn(m.ty[c - nx], p[-kRX], s);
-        s = __fmaf_rn(m.tz[c], p[kRX * kRY], s);
-        if (INNER || k > 0) s = __fmaf_rn(m.tz[c - pl], p[-kRX * kRY], s);
+    auto face_sum = [&](int c, int i, int j, int k, const T* p) {
+        T s = m.tx[c] * p[1];
+        if (INNER || i > 0) s = fmav(m.tx[c - 1], p[-1], s);
+        s = fmav(m.ty[c], p[kRX], s);
+        if (INNER || j > 0) s = fmav(m.ty[c - nx], p[-kRX], s);
+        s = fmav(m.tz[c], p[kRX * kRY], s);
+        if (INNER || k > 0) s = fmav(m.tz[c - pl], p[-kRX * kRY], s);
         return s;
     };
     if (t < kRX / 2 * kRY) {
@@ -579,11 +587,11 @@ __device__ __forceinline__ void large_sweep(const MgGeom& g, const MgCoef& m, co
 #pragma unroll
         for (int z = 0; z < kRZ; ++z) {
             const int k = k0 - 2 + z, par = (j + k) & 1, i = i2 + par;
-            float v = 0.0f;
+            T v = T(0);
             if (INNER || (row && k >= 0 && k < g.nz && i >= 0 && i < nx)) {
                 const int c = i + nx * j + pl * k;
                 v = m.di[c] * b[c];
-                if (!DOWN) v = __fmaf_rn(m.di[c], b[c], en[(i >> 1) + g.mx * ((j >> 1) + g.my * (k >> 1))]);
+                if (!DOWN) v = fmav(m.di[c], b[c], en[(i >> 1) + g.mx * ((j >> 1) + g.my * (k >> 1))]);
             }
             xs[2 * a + par + kRX * (y + kRY * z)] = v;
         }
@@ -595,8 +603,8 @@ __device__ __forceinline__ void large_sweep(const MgGeom& g, const MgCoef& m, co
 #pragma unroll 5
         for (int z = 0; z < kLZ + 2; ++z) {
             const int k = k0 - 1 + z, par = (j + k) & 1, i = i2 + par;
-            float* p = xs + (2 * a + par + 1) + kRX * ((y + 1) + kRY * (z + 1));
-            float v = 0.0f;
+            T* p = xs + (2 * a + par + 1) + kRX * ((y + 1) + kRY * (z + 1));
+            T v = T(0);
             if (INNER || (row && k >= 0 && k < g.nz && i >= 0 && i < nx)) {
                 const int c = i + nx * j + pl * k;
                 v = m.di[c] * (b[c] + face_sum(c, i, j, k, p));
@@ -610,11 +618,11 @@ __device__ __forceinline__ void large_sweep(const MgGeom& g, const MgCoef& m, co
     const int ip = i0 + 2 * a, j = j0 + y;
 #pragma unroll
     for (int z = z0; z < z0 + 4; z += 2) {
-        float s2 = 0.0f;
+        T s2 = T(0);
 #pragma unroll
         for (int dk = 0; dk < 2; ++dk) {
             const int k = k0 + z + dk, par = (j + k) & 1, i = ip + par;
-            const float* p = xs + (2 * a + par + 2) + kRX * ((y + 2) + kRY * (z + dk + 2));
+            const T* p = xs + (2 * a + par + 2) + kRX * ((y + 2) + kRY * (z + dk + 2));
             if (!(INNER || (j < g.ny && k < g.nz && ip < nx))) continue;
             const int c = i + nx * j + pl * k;
             if (DOWN) {
@@ -632,38 +640,40 @@ __device__ __forceinline__ void large_sweep(const MgGeom& g, const MgCoef& m, co
     }
 }
 
-template <bool DOWN>
+template <bool DOWN, typename T>
 __global__ void __launch_bounds__(kLargeThreads, 4)
-k_mg_level_large(const MgGeom g, const MgCoef m, const float* __restrict__ b, const float* __restrict__ en,
-                 float* __restrict__ out) {
-    __shared__ float xs[kRX * kRY * kRZ];
+k_mg_level_large(const MgGeom g, const MgCoef<T> m, const T* __restrict__ b, const T* __restrict__ en,
+                 T* __restrict__ out) {
+    __shared__ T xs[kRX * kRY * kRZ];
     const int tb = blockIdx.x, bx = tb % g.tiles_x, by = (tb / g.tiles_x) % g.tiles_y, bz = tb / (g.tiles_x * g.tiles_y);
     const int i0 = bx * kLX, j0 = by * kLY, k0 = bz * kLZ;
     grid_dep_wait();
     const bool inner = i0 > 2 && i0 + kLX + 2 <= g.nx && j0 > 2 && j0 + kLY + 2 <= g.ny && k0 > 2 && k0 + kLZ + 2 <= g.nz;
     if (inner)
-        large_sweep<DOWN, true>(g, m, b, en, out, xs, i0, j0, k0);
+        large_sweep<DOWN, true, T>(g, m, b, en, out, xs, i0, j0, k0);
     else
-        large_sweep<DOWN, false>(g, m, b, en, out, xs, i0, j0, k0);
+        large_sweep<DOWN, false, T>(g, m, b, en, out, xs, i0, j0, k0);
 }
 
 // The levels of at most kBottomCells cells in one block, a thread per cell, down to a single cell
 // (which is solved) and back.  Level l keeps tx, ty, tz, D^-1, b, x, each of n[l] values.
+template <typename T>
 struct MgBottom {
     int levels;
     int nx[kMaxBottom], ny[kMaxBottom], nz[kMaxBottom];
-    int off[kMaxBottom];                 // first float of the level in shared memory
-    MgCoef m[kMaxBottom];
-    const float* b;
-    float* x;
+    int off[kMaxBottom];                 // first T of the level in shared memory
+    MgCoef<T> m[kMaxBottom];
+    const T* b;
+    T* x;
 };
 
-__global__ void __launch_bounds__(kBottomThreads) k_mg_bottom(const MgBottom a) {
-    __shared__ float sm[kBottomFloats];
+template <typename T>
+__global__ void __launch_bounds__(kBottomThreads) k_mg_bottom(const MgBottom<T> a) {
+    __shared__ T sm[kBottomValues];
     const int t = threadIdx.x;
     for (int l = 0; l < a.levels; ++l) {
         const int n = a.nx[l] * a.ny[l] * a.nz[l];
-        float* p = sm + a.off[l];
+        T* p = sm + a.off[l];
         if (t < n) {
             p[t] = a.m[l].tx[t];
             p[n + t] = a.m[l].ty[t];
@@ -679,26 +689,26 @@ __global__ void __launch_bounds__(kBottomThreads) k_mg_bottom(const MgBottom a) 
     }
     __syncthreads();
     // sum of coefficient times neighbour's x over the faces of cell c
-    auto sum = [&](const float* p, int n, int nx, int ny, int nz, int c, int i, int j, int k) {
+    auto sum = [&](const T* p, int n, int nx, int ny, int nz, int c, int i, int j, int k) {
         const int pl = nx * ny;
-        const float* x = p + 5 * n;
-        float s = 0.0f;
-        if (i < nx - 1) s = __fmaf_rn(p[c], x[c + 1], s);
-        if (i > 0) s = __fmaf_rn(p[c - 1], x[c - 1], s);
-        if (j < ny - 1) s = __fmaf_rn(p[n + c], x[c + nx], s);
-        if (j > 0) s = __fmaf_rn(p[n + c - nx], x[c - nx], s);
-        if (k < nz - 1) s = __fmaf_rn(p[2 * n + c], x[c + pl], s);
-        if (k > 0) s = __fmaf_rn(p[2 * n + c - pl], x[c - pl], s);
+        const T* x = p + 5 * n;
+        T s = T(0);
+        if (i < nx - 1) s = fmav(p[c], x[c + 1], s);
+        if (i > 0) s = fmav(p[c - 1], x[c - 1], s);
+        if (j < ny - 1) s = fmav(p[n + c], x[c + nx], s);
+        if (j > 0) s = fmav(p[n + c - nx], x[c - nx], s);
+        if (k < nz - 1) s = fmav(p[2 * n + c], x[c + pl], s);
+        if (k > 0) s = fmav(p[2 * n + c - pl], x[c - pl], s);
         return s;
     };
     for (int l = 0; l < a.levels; ++l) {
         const int nx = a.nx[l], ny = a.ny[l], nz = a.nz[l], n = nx * ny * nz;
-        float* p = sm + a.off[l];
+        T* p = sm + a.off[l];
         const int r = t / nx, i = t - r * nx, k = r / ny, j = r - k * ny;
         const bool on = t < n, black = ((i + j + k) & 1) != 0;
-        float* x = p + 5 * n;
-        const float d = on ? p[3 * n + t] : 0.0f, b = on ? p[4 * n + t] : 0.0f;
-        if (on) x[t] = black ? 0.0f : d * b;
+        T* x = p + 5 * n;
+        const T d = on ? p[3 * n + t] : T(0), b = on ? p[4 * n + t] : T(0);
+        if (on) x[t] = black ? T(0) : d * b;
         __syncthreads();
         if (l == a.levels - 1) break;
         if (on && black) x[t] = d * (b + sum(p, n, nx, ny, nz, t, i, j, k));
@@ -706,7 +716,7 @@ __global__ void __launch_bounds__(kBottomThreads) k_mg_bottom(const MgBottom a) 
         const int mx = a.nx[l + 1], my = a.ny[l + 1], mz = a.nz[l + 1], mn = mx * my * mz;
         if (t < mn) {
             const int R = t / mx, I = t - R * mx, K = R / my, J = R - K * my;
-            float s = 0.0f;
+            T s = T(0);
             for (int u = 0; u < 4; ++u) {
                 const int dj = u & 1, dk = u >> 1, ii = 2 * I + ((dj + dk) & 1), jj = 2 * J + dj, kk = 2 * K + dk;
                 if (ii < nx && jj < ny && kk < nz) s += sum(p, n, nx, ny, nz, ii + nx * (jj + ny * kk), ii, jj, kk);
@@ -717,13 +727,13 @@ __global__ void __launch_bounds__(kBottomThreads) k_mg_bottom(const MgBottom a) 
     }
     for (int l = a.levels - 2; l >= 0; --l) {
         const int nx = a.nx[l], ny = a.ny[l], nz = a.nz[l], n = nx * ny * nz;
-        float* p = sm + a.off[l];
+        T* p = sm + a.off[l];
         const int r = t / nx, i = t - r * nx, k = r / ny, j = r - k * ny;
         const bool on = t < n, black = ((i + j + k) & 1) != 0;
-        float* x = p + 5 * n;
-        const float d = on ? p[3 * n + t] : 0.0f, b = on ? p[4 * n + t] : 0.0f;
+        T* x = p + 5 * n;
+        const T d = on ? p[3 * n + t] : T(0), b = on ? p[4 * n + t] : T(0);
         const int mx = a.nx[l + 1], my = a.ny[l + 1], mn = mx * my * a.nz[l + 1];
-        if (on && !black) x[t] = __fmaf_rn(d, b, sm[a.off[l + 1] + 5 * mn + (i >> 1) + mx * ((j >> 1) + my * (k >> 1))]);
+        if (on && !black) x[t] = fmav(d, b, sm[a.off[l + 1] + 5 * mn + (i >> 1) + mx * ((j >> 1) + my * (k >> 1))]);
         __syncthreads();
         if (on && black) x[t] = d * (b + sum(p, n, nx, ny, nz, t, i, j, k));
         __syncthreads();
@@ -736,63 +746,171 @@ __global__ void __launch_bounds__(kBottomThreads) k_mg_bottom(const MgBottom a) 
 
 // ---- host --------------------------------------------------------------------------------------
 
-template <bool DOWN>
-void launch_level(vofp_ctx* c, cudaStream_t st, bool pdl, const MgLevel& l, const MgLevel& n) {
+template <typename T, bool DOWN>
+void launch_level(vofp_ctx* c, cudaStream_t st, bool pdl, const MgLevel<T>& l, const MgLevel<T>& n) {
     const bool large = l.n >= kLargeCells;
     const int tx = large ? kLX : kTX, ty = large ? kLY : kTY, tz = large ? kLZ : kTZ;
     const MgGeom g{l.nx, l.ny, l.nz, n.nx, n.ny, n.nz, ceil_div(l.nx, tx), ceil_div(l.ny, ty)};
     const dim3 grid((unsigned)(g.tiles_x * g.tiles_y * ceil_div(l.nz, tz)));
-    const MgCoef m{l.tx, l.ty, l.tz, l.di};
-    const float *b = l.b, *en = n.x;
-    float* out = DOWN ? n.b : l.x;
+    const MgCoef<T> m{l.tx, l.ty, l.tz, l.di};
+    const T *b = l.b, *en = n.x;
+    T* out = DOWN ? n.b : l.x;
     if (large)
-        launch_dep(c, pdl, k_mg_level_large<DOWN>, grid, dim3(kLargeThreads), 0, st, g, m, b, en, out);
+        launch_dep(c, pdl, k_mg_level_large<DOWN, T>, grid, dim3(kLargeThreads), 0, st, g, m, b, en, out);
     else
-        launch_dep(c, pdl, k_mg_level<DOWN>, grid, dim3(kTileThreads), 0, st, g, m, b, en, out);
+        launch_dep(c, pdl, k_mg_level<DOWN, T>, grid, dim3(kTileThreads), 0, st, g, m, b, en, out);
 }
 
-int bottom_level(const vofp_ctx* c) {
+template <typename T>
+int bottom_level(const MgSet<T>& m) {
     int l = 0;
-    while (c->mg[l].n > kBottomCells) ++l;
+    while (m.lv[l].n > kBottomCells) ++l;
     return l;
 }
 
-void vcycle(vofp_ctx* c, cudaStream_t st, bool pdl) {
-    const int lb = bottom_level(c), nl = (int)c->mg.size();
-    for (int l = 0; l < lb; ++l) launch_level<true>(c, st, pdl, c->mg[l], c->mg[l + 1]);
-    MgBottom a{};
+template <typename T>
+void vcycle(vofp_ctx* c, cudaStream_t st, bool pdl, const MgSet<T>& m) {
+    const int lb = bottom_level(m), nl = (int)m.lv.size();
+    for (int l = 0; l < lb; ++l) launch_level<T, true>(c, st, pdl, m.lv[l], m.lv[l + 1]);
+    MgBottom<T> a{};
     a.levels = nl - lb;
     int off = 0;
     for (int l = lb; l < nl; ++l) {
-        const MgLevel& v = c->mg[l];
+        const MgLevel<T>& v = m.lv[l];
         a.nx[l - lb] = v.nx;
         a.ny[l - lb] = v.ny;
         a.nz[l - lb] = v.nz;
         a.off[l - lb] = off;
         off += 6 * (int)v.n;
-        a.m[l - lb] = MgCoef{v.tx, v.ty, v.tz, v.di};
+        a.m[l - lb] = MgCoef<T>{v.tx, v.ty, v.tz, v.di};
     }
-    a.b = c->mg[lb].b;
-    a.x = c->mg[lb].x;
-    launch_dep(c, pdl, k_mg_bottom, dim3(1), dim3(kBottomThreads), 0, st, a);
-    for (int l = lb - 1; l >= 0; --l) launch_level<false>(c, st, pdl, c->mg[l], c->mg[l + 1]);
+    a.b = m.lv[lb].b;
+    a.x = m.lv[lb].x;
+    launch_dep(c, pdl, k_mg_bottom<T>, dim3(1), dim3(kBottomThreads), 0, st, a);
+    for (int l = lb - 1; l >= 0; --l) launch_level<T, false>(c, st, pdl, m.lv[l], m.lv[l + 1]);
 }
 
-template <bool COMPACT>
+template <typename T>
+MgSet<T>& set_of(vofp_ctx* c) {
+    if constexpr (sizeof(T) == 4)
+        return c->mgf;
+    else
+        return c->mgd;
+}
+// the vectors of the iteration: compact or full-grid FP32 ones, full-grid FP64 ones
+template <bool COMPACT, typename T>
+T* vec_r(vofp_ctx* c) {
+    if constexpr (COMPACT)
+        return c->rbc_r;
+    else if constexpr (sizeof(T) == 4)
+        return c->rf;
+    else
+        return c->r;
+}
+template <bool COMPACT, typename T>
+const T* vec_q(vofp_ctx* c) {
+    if constexpr (COMPACT)
+        return c->rbc_q;
+    else if constexpr (sizeof(T) == 4)
+        return c->qf;
+    else
+        return c->q;
+}
+
+template <bool COMPACT, typename T>
 void launch_direction(vofp_ctx* c, cudaStream_t st, bool pdl, int start) {
-    const MgLevel& l = c->mg[0];
-    launch_dep(c, pdl, k_mg_direction<COMPACT>, dim3(grid_fine(l.n / MgEntries<COMPACT>::A)), dim3(kNT), 0, st, c->d, l.nx, l.ny, (int)l.n,
-               (const float*)(COMPACT ? c->rbc_r : c->rf), (const float*)c->mg_w, (const float*)l.x, (const float*)l.b,
-               c->mg_z, c->ngroups, reinterpret_cast<const int2*>(c->mg_rep), (const int*)c->gptr,
+    MgSet<T>& m = set_of<T>(c);
+    const MgLevel<T>& l = m.lv[0];
+    launch_dep(c, pdl, k_mg_direction<COMPACT, T>, dim3(grid_fine(l.n / MgEntries<COMPACT>::A)), dim3(kNT), 0, st, c->d,
+               l.nx, l.ny, (int)l.n, (const T*)vec_r<COMPACT, T>(c), (const T*)m.w, (const T*)l.x, (const T*)l.b, m.z,
+               c->ngroups, reinterpret_cast<const int2*>(m.rep), (const int*)c->gptr,
                (const int*)(COMPACT ? c->rbc_gref : c->gcells), c->sc, c->partials, c->counters, start);
 }
-template <bool COMPACT, bool UPD>
+template <bool COMPACT, bool UPD, typename T>
 void launch_update(vofp_ctx* c, cudaStream_t st, bool pdl, cudaGraphConditionalHandle h, int use_h) {
-    const MgLevel& l = c->mg[0];
+    MgSet<T>& m = set_of<T>(c);
+    const MgLevel<T>& l = m.lv[0];
     const long long nh = COMPACT ? c->rbc_nh : c->d.n, nv = COMPACT ? c->rbc_nh + c->rbc_ne : c->d.n;
-    launch_dep(c, pdl, k_mg_update<COMPACT, UPD>, dim3(grid_fine(l.n / MgEntries<COMPACT>::A)), dim3(kNT), 0, st, c->d, l.nx, l.ny, (int)l.n, nh, nv,
-               COMPACT ? c->rbc_r : c->rf, (const float*)(COMPACT ? c->rbc_q : c->qf), (const float*)c->mg_w,
-               (const uint8_t*)c->mg_mask, (const int*)c->mg_even, l.b, c->sc, c->partials, c->counters, h, use_h, (const double*)(c->partials + kPqBase), COMPACT ? rbc_pq_parts(c) : 0);
+    launch_dep(c, pdl, k_mg_update<COMPACT, UPD, T>, dim3(grid_fine(l.n / MgEntries<COMPACT>::A)), dim3(kNT), 0, st, c->d,
+               l.nx, l.ny, (int)l.n, nh, nv, vec_r<COMPACT, T>(c), vec_q<COMPACT, T>(c), (const T*)m.w,
+               (const uint8_t*)c->mg_mask, (const int*)c->mg_even, l.b, c->sc, c->partials, c->counters, h, use_h,
+               (const double*)(c->partials + kPqBase), COMPACT ? rbc_pq_parts(c) : 0);
+}
+
+// The hierarchy and the weights of the current operator (once per operator and precision).
+template <bool COMPACT, typename T>
+vofp_status build(vofp_ctx* c) {
+    MgSet<T>& m = set_of<T>(c);
+    const Dims d = c->d;
+    cudaStream_t st = c->stream;
+    vofp_status s;
+    if (m.lv.empty()) {
+        std::vector<MgLevel<T>> v;
+        int nx = d.nx, ny = d.ny, nz = d.nz;
+        do {
+            MgLevel<T> l{};
+            l.nx = nx = (nx + 1) / 2;
+            l.ny = ny = (ny + 1) / 2;
+            l.nz = nz = (nz + 1) / 2;
+            l.n = (long long)nx * ny * nz;
+            for (T** p : {&l.tx, &l.ty, &l.tz, &l.di, &l.ex, &l.b, &l.x})
+                if ((s = c->alloc(p, l.n))) return s;
+            v.push_back(l);
+        } while (v.back().n > 1);
+        if (!c->mg_dmax && (s = c->alloc(&c->mg_dmax, 1))) return s;
+        m.lv = v;
+    }
+    const MgLevel<T>& l1 = m.lv[0];
+    if (COMPACT) {
+        if (!c->mg_even &&
+            ((s = c->alloc(&c->mg_mask, (l1.n + 3) / 4)) || (s = c->alloc(&c->mg_even, 4 * l1.n))))
+            return s;
+        VOFP_CUDA_TRY(c, cudaMemsetAsync(c->mg_mask, 0, sizeof(uint32_t) * ((l1.n + 3) / 4), st));
+    }
+    const long long nv = COMPACT ? c->rbc_cap : d.n;
+    if (nv > m.cap) {
+        // entries past the vectors in use stay 0 (the tensor copies read whole boxes)
+        if ((s = c->alloc(&m.w, nv)) || (s = c->alloc(&m.z, nv))) return s;
+        m.cap = nv;
+    }
+    VOFP_CUDA_TRY(c, cudaMemsetAsync(m.z, 0, sizeof(T) * m.cap, st));
+    if (c->ngroups > m.rep_cap) {
+        const long long cap = c->ngroups + c->ngroups / 2 + 64;
+        if ((s = c->alloc(&m.rep, 2 * cap))) return s;
+        m.rep_cap = cap;
+    }
+    VOFP_CUDA_TRY(c, cudaMemsetAsync(c->mg_dmax, 0, sizeof(unsigned long long), st));
+    launch(c, k_mg_max, grid_n(d.n), kNT, st, d.n, (const double*)c->diag, c->mg_dmax);
+    const unsigned long long* dmax = c->mg_dmax;
+    launch(c, k_mg_coarsen_fine<T>, ceil_div(l1.n, kNT), kNT, st, d, l1.nx, l1.ny, l1.nz, (const double*)c->Tx,
+           (const double*)c->Ty, (const double*)c->Tz, (const double*)c->diag, dmax, l1.tx, l1.ty, l1.tz, l1.ex);
+    for (size_t q = 0; q < m.lv.size(); ++q) {
+        const MgLevel<T>& l = m.lv[q];
+        if (q > 0) {
+            const MgLevel<T>& f = m.lv[q - 1];
+            launch(c, k_mg_coarsen<T>, ceil_div(l.n, kNT), kNT, st, f.nx, f.ny, f.nz, (const T*)f.tx, (const T*)f.ty,
+                   (const T*)f.tz, (const T*)f.ex, l.nx, l.ny, l.nz, l.tx, l.ty, l.tz, l.ex);
+        }
+        launch(c, k_mg_dinv<T>, ceil_div(l.n, kNT), kNT, st, l.nx, l.ny, l.nz, (const T*)l.tx, (const T*)l.ty,
+               (const T*)l.tz, (const T*)l.ex, l.di);
+    }
+    const long long n = COMPACT ? c->rbc_nh + c->rbc_ne : d.n;
+    launch(c, k_mg_weights<COMPACT, T>, grid_n(n), kNT, st, d, n, COMPACT ? c->rbc_nh : d.n, (const double*)c->sq,
+           (const int32_t*)c->root, (const uint32_t*)c->red_bits, dmax, m.w);
+    if (c->ngroups > 0)
+        launch(c, k_mg_groups<COMPACT, T>, ceil_div(c->ngroups, kNT), kNT, st, d, c->ngroups, l1.nx, l1.ny,
+               (const int*)c->gptr, (const int*)c->gcells, (const int*)c->rbc_gref, (const double*)c->sq, dmax, m.w,
+               reinterpret_cast<int2*>(m.rep), c->mg_mask, c->mg_even);
+    VOFP_CUDA_TRY(c, cudaGetLastError());
+    m.ok = true;
+    return VOFP_OK;
+}
+
+template <bool COMPACT, typename T>
+void precondition(vofp_ctx* c, cudaStream_t st, bool pdl, int start) {
+    if (start) launch_update<COMPACT, false, T>(c, st, false, (cudaGraphConditionalHandle)0, 0);
+    vcycle<T>(c, st, pdl, set_of<T>(c));
+    launch_direction<COMPACT, T>(c, st, pdl, start);
 }
 
 }  // namespace
@@ -805,106 +923,36 @@ bool mg_wanted(const vofp_ctx* c, double rtol) {
     return use == 2 || (use != 0 && c->d.n >= kMgMinCells && rtol <= kMgMaxRtol);
 }
 
-// The hierarchy and the weights of the current operator (mixed red-black solve; once per operator).
-vofp_status mg_ensure(vofp_ctx* c) {
-    if (c->mg_built) return VOFP_OK;
-    c->mg_built = true;
-    c->mg_ok = false;
-    const Dims d = c->d;
-    cudaStream_t st = c->stream;
-    vofp_status s;
-    if (c->mg.empty()) {
-        std::vector<MgLevel> v;
-        int nx = d.nx, ny = d.ny, nz = d.nz;
-        do {
-            MgLevel l{};
-            l.nx = nx = (nx + 1) / 2;
-            l.ny = ny = (ny + 1) / 2;
-            l.nz = nz = (nz + 1) / 2;
-            l.n = (long long)nx * ny * nz;
-            for (float** p : {&l.tx, &l.ty, &l.tz, &l.di, &l.ex, &l.b, &l.x})
-                if ((s = c->alloc(p, l.n))) return s;
-            v.push_back(l);
-        } while (v.back().n > 1);
-        c->mg = v;
-        if ((s = c->alloc(&c->mg_dmax, 1)) || (s = c->alloc(&c->mg_mask, (v[0].n + 3) / 4)) ||
-            (s = c->alloc(&c->mg_even, 4 * v[0].n)))
-            return s;
-    }
-    const long long nv = c->rbc_ok ? c->rbc_cap : d.n;
-    if (nv > c->mg_cap) {
-        // entries past the vectors in use stay 0 (the tensor copies read whole boxes)
-        if ((s = c->alloc(&c->mg_w, nv)) || (s = c->alloc(&c->mg_z, nv))) return s;
-        c->mg_cap = nv;
-    }
-    VOFP_CUDA_TRY(c, cudaMemsetAsync(c->mg_z, 0, sizeof(float) * c->mg_cap, st));
-    if (c->ngroups > c->mg_rep_cap) {
-        const long long cap = c->ngroups + c->ngroups / 2 + 64;
-        if ((s = c->alloc(&c->mg_rep, 2 * cap))) return s;
-        c->mg_rep_cap = cap;
-    }
-    VOFP_CUDA_TRY(c, cudaMemsetAsync(c->mg_mask, 0, sizeof(uint32_t) * ((c->mg[0].n + 3) / 4), st));
-    VOFP_CUDA_TRY(c, cudaMemsetAsync(c->mg_dmax, 0, sizeof(unsigned long long), st));
-    launch(c, k_mg_max, grid_n(d.n), kNT, st, d.n, (const double*)c->diag, c->mg_dmax);
-    const MgLevel& l1 = c->mg[0];
-    launch(c, k_mg_coarsen_fine, ceil_div(l1.n, kNT), kNT, st, d, l1.nx, l1.ny, l1.nz, (const double*)c->Tx,
-           (const double*)c->Ty, (const double*)c->Tz, (const double*)c->diag, (const unsigned long long*)c->mg_dmax,
-           l1.tx, l1.ty, l1.tz, l1.ex);
-    for (size_t q = 0; q < c->mg.size(); ++q) {
-        const MgLevel& l = c->mg[q];
-        if (q > 0) {
-            const MgLevel& f = c->mg[q - 1];
-            launch(c, k_mg_coarsen, ceil_div(l.n, kNT), kNT, st, f.nx, f.ny, f.nz, (const float*)f.tx, (const float*)f.ty,
-                   (const float*)f.tz, (const float*)f.ex, l.nx, l.ny, l.nz, l.tx, l.ty, l.tz, l.ex);
-        }
-        launch(c, k_mg_dinv, ceil_div(l.n, kNT), kNT, st, l.nx, l.ny, l.nz, (const float*)l.tx, (const float*)l.ty,
-               (const float*)l.tz, (const float*)l.ex, l.di);
-    }
-    const int ng = c->ngroups;
-    if (c->rbc_ok) {
-        const long long n = c->rbc_nh + c->rbc_ne;
-        launch(c, k_mg_weights<true>, grid_n(n), kNT, st, d, n, c->rbc_nh, (const double*)c->sq, (const int32_t*)c->root,
-               (const uint32_t*)c->red_bits, (const unsigned long long*)c->mg_dmax, c->mg_w);
-        if (ng > 0)
-            launch(c, k_mg_groups<true>, ceil_div(ng, kNT), kNT, st, d, ng, l1.nx, l1.ny, (const int*)c->gptr,
-                   (const int*)c->gcells, (const int*)c->rbc_gref, (const double*)c->sq,
-                   (const unsigned long long*)c->mg_dmax, c->mg_w, reinterpret_cast<int2*>(c->mg_rep), c->mg_mask, c->mg_even);
-    } else {
-        launch(c, k_mg_weights<false>, grid_n(d.n), kNT, st, d, d.n, d.n, (const double*)c->sq, (const int32_t*)c->root,
-               (const uint32_t*)c->red_bits, (const unsigned long long*)c->mg_dmax, c->mg_w);
-        if (ng > 0)
-            launch(c, k_mg_groups<false>, ceil_div(ng, kNT), kNT, st, d, ng, l1.nx, l1.ny, (const int*)c->gptr,
-                   (const int*)c->gcells, (const int*)nullptr, (const double*)c->sq,
-                   (const unsigned long long*)c->mg_dmax, c->mg_w, reinterpret_cast<int2*>(c->mg_rep), c->mg_mask, c->mg_even);
-    }
-    VOFP_CUDA_TRY(c, cudaGetLastError());
-    c->mg_ok = true;
-    return VOFP_OK;
+vofp_status mg_ensure(vofp_ctx* c, bool fp64) {
+    bool& built = fp64 ? c->mgd.built : c->mgf.built;
+    if (built) return VOFP_OK;
+    built = true;
+    (fp64 ? c->mgd.ok : c->mgf.ok) = false;
+    return fp64 ? build<false, double>(c) : c->rbc_ok ? build<true, float>(c) : build<false, float>(c);
 }
 
-// b_1 (at the start of an inner solve: from the new residual), the V-cycle, z, r.z and beta
-void mg_precondition(vofp_ctx* c, cudaStream_t st, bool pdl, int start) {
-    if (start) {
-        if (c->rbc_ok)
-            launch_update<true, false>(c, st, false, (cudaGraphConditionalHandle)0, 0);
-        else
-            launch_update<false, false>(c, st, false, (cudaGraphConditionalHandle)0, 0);
-    }
-    vcycle(c, st, pdl);
-    if (c->rbc_ok)
-        launch_direction<true>(c, st, pdl, start);
+// b_1 (at the start of a loop: from the new residual), the V-cycle, z, r.z and beta
+void mg_precondition(vofp_ctx* c, cudaStream_t st, bool fp64, bool pdl, int start) {
+    if (fp64)
+        precondition<false, double>(c, st, pdl, start);
+    else if (c->rbc_ok)
+        precondition<true, float>(c, st, pdl, start);
     else
-        launch_direction<false>(c, st, pdl, start);
+        precondition<false, float>(c, st, pdl, start);
 }
 
 // r -= alpha q, r.r, the inner loop's stop test and b_1
-void mg_update(vofp_ctx* c, cudaStream_t st, bool pdl, cudaGraphConditionalHandle h, int use_h) {
-    if (c->rbc_ok)
-        launch_update<true, true>(c, st, pdl, h, use_h);
+void mg_update(vofp_ctx* c, cudaStream_t st, bool fp64, bool pdl, cudaGraphConditionalHandle h, int use_h) {
+    if (fp64)
+        launch_update<false, true, double>(c, st, pdl, h, use_h);
+    else if (c->rbc_ok)
+        launch_update<true, true, float>(c, st, pdl, h, use_h);
     else
-        launch_update<false, true>(c, st, pdl, h, use_h);
+        launch_update<false, true, float>(c, st, pdl, h, use_h);
 }
 
-int mg_precondition_kernels(const vofp_ctx* c) { return 2 * bottom_level(c) + 2; }
+int mg_precondition_kernels(const vofp_ctx* c, bool fp64) {
+    return 2 * (fp64 ? bottom_level(c->mgd) : bottom_level(c->mgf)) + 2;
+}
 
 }  // namespace vofp

@@ -648,7 +648,7 @@ void launch_main_t(vofp_ctx* c, cudaStream_t st, const float* po, float* pn, boo
     const Dims d = c->d;
     const int nh = d.nx / 2;
     // the direction's source: z with the coarse-grid correction, r without
-    const float* src = c->mg_use ? c->mg_z : c->rbc_r;
+    const float* src = c->mg_use ? c->mgf.z : c->rbc_r;
     const CUtensorMap *mr = tensor_map_f32_x(c, src, nh, G::BWC, G::TH + 4),
                       *mp = tensor_map_f32_x(c, po, nh, G::BWC, G::TH + 4),
                       *mx = tensor_map_f32(c, c->Txf, G::BWF, G::TH + 2),
@@ -713,8 +713,8 @@ void rbc_iteration(vofp_ctx* c, cudaStream_t st, const float* po, float* pn, cud
     launch_main(c, st, po, pn, pdl);
     rbc_aux(c, st, po, pn, pdl);
     if (c->mg_use) {
-        mg_update(c, st, pdl, h, use_h);
-        mg_precondition(c, st, pdl, 0);
+        mg_update(c, st, false, pdl, h, use_h);
+        mg_precondition(c, st, false, pdl, 0);
         return;
     }
     const long long nc = c->rbc_nh + c->rbc_ne;

@@ -653,9 +653,16 @@ void launch_cg_iteration(vofp_ctx* c, cudaStream_t st, V* r, V* po, V* pn, V* xv
                          const V* Tx, const V* Ty, const V* Tz, bool inner, bool rb,
                          cudaGraphConditionalHandle h, int use_h) {
     const uint32_t* bits = rb ? c->excl_bits : c->slave_bits;
-    const bool mg = sizeof(V) == 4 && inner && rb && c->mg_use;
+    constexpr bool fp64 = sizeof(V) == 8;
+    const bool mg = rb && c->mg_use;
     if (rb) {
-        launch_cg_rb<V>(c, st, Tx, Ty, Tz, mg ? reinterpret_cast<const V*>(c->mg_z) : r, po, pn, xv, q);
+        const V* src = r;
+        if constexpr (fp64) {
+            if (mg) src = c->mgd.z;
+        } else {
+            if (mg) src = c->mgf.z;
+        }
+        launch_cg_rb<V>(c, st, Tx, Ty, Tz, src, po, pn, xv, q);
     } else {
         launch_cg_stencil<V>(c, st, Tx, Ty, Tz, r, po, pn, xv, q);
     }
@@ -663,8 +670,10 @@ void launch_cg_iteration(vofp_ctx* c, cudaStream_t st, V* r, V* po, V* pn, V* xv
         launch(c, k_group_patch<V>, ceil_div(c->ngroups, kNT), kNT, st, c->ngroups, c->gptr, c->gcells, c->gcorr, q, pn,
                1, c->sc, c->partials, c->counters);
     if (mg) {
-        mg_update(c, st, c->pdl != 0 && use_h != 0, h, use_h);
-        mg_precondition(c, st, c->pdl != 0 && use_h != 0, 0);
+        // chained launches in the loops' graphs (a refused one is caught when the capture ends)
+        const bool pdl = c->pdl != 0 && use_h != 0;
+        mg_update(c, st, fp64, pdl, h, inner ? use_h : 0);
+        mg_precondition(c, st, fp64, pdl, 0);
         return;
     }
     if (inner)
@@ -780,12 +789,14 @@ void launch_fp64_body(vofp_ctx* c, cudaStream_t st, int U, bool rb, cudaGraphCon
     for (int u = 0; u < U; ++u) {
         double* po = (u % 2 == 0) ? c->p0 : c->p1;
         double* pn = (u % 2 == 0) ? c->p1 : c->p0;
-        launch_cg_iteration<double>(c, st, c->r, po, pn, c->xt, c->q, c->Txs, c->Tys, c->Tzs, false, rb, h, 0);
+        launch_cg_iteration<double>(c, st, c->r, po, pn, c->xt, c->q, c->Txs, c->Tys, c->Tzs, false, rb, h, use_h);
     }
     launch(c, k_cg_check<double>, stream_grid(c->d.n), kNT, st, c->d.n, (const double*)c->r, (const double*)c->sq,
            (const uint32_t*)(rb ? c->excl_bits : c->slave_bits), c->sc, c->partials, c->counters, h, use_h);
 }
-int fp64_body_kernels(const vofp_ctx* c, int U, bool rb) { return U * iteration_kernels(c, rb) + 1; }
+int fp64_body_kernels(const vofp_ctx* c, int U, bool rb) {
+    return U * (iteration_kernels(c, rb) + (rb && c->mg_use ? mg_precondition_kernels(c, true) : 0)) + 1;
+}
 
 // Mixed outer step, first part: FP64 residual of the full system, outer test, inner right-hand side.
 void launch_outer_head(vofp_ctx* c, cudaStream_t st, bool rb, cudaGraphConditionalHandle ho,
@@ -807,7 +818,7 @@ void launch_outer_head(vofp_ctx* c, cudaStream_t st, bool rb, cudaGraphCondition
         else
             launch(c, k_inner_prep, stream_grid(c->d.n), kNT, st, c->d.n, (const double*)c->q,
                    (const uint32_t*)c->excl_bits, c->rf, c->xf, c->pf0, c->sc, c->partials, c->counters);
-        if (c->mg_use) mg_precondition(c, st, c->pdl != 0 && use_h != 0, 1);
+        if (c->mg_use) mg_precondition(c, st, false, c->pdl != 0 && use_h != 0, 1);
     } else {
         launch(c, k_inner_prep, stream_grid(c->d.n), kNT, st, c->d.n, (const double*)c->r,
                (const uint32_t*)c->slave_bits, c->rf, c->xf, c->pf0, c->sc, c->partials, c->counters);
@@ -815,7 +826,7 @@ void launch_outer_head(vofp_ctx* c, cudaStream_t st, bool rb, cudaGraphCondition
 }
 int outer_head_kernels(const vofp_ctx* c, bool rb) {
     const int g = c->ngroups > 0 ? 1 : 0;
-    return 1 + g + 1 + (rb ? 2 + g + (c->mg_use ? 1 + mg_precondition_kernels(c) : 0) : 0) + 1;
+    return 1 + g + 1 + (rb ? 2 + g + (c->mg_use ? 1 + mg_precondition_kernels(c, false) : 0) : 0) + 1;
 }
 void launch_inner_body(vofp_ctx* c, cudaStream_t st, int U, bool rb, cudaGraphConditionalHandle hi, int use_h) {
     if (rb && c->rbc_ok) {
@@ -855,7 +866,7 @@ int outer_tail_kernels(const vofp_ctx* c, bool rb) {
 }
 // kernels of one mixed inner iteration
 int inner_iteration_kernels(const vofp_ctx* c, bool rb) {
-    const int pre = rb && c->mg_use ? mg_precondition_kernels(c) : 0;
+    const int pre = rb && c->mg_use ? mg_precondition_kernels(c, false) : 0;
     if (rb && c->rbc_ok)   // iteration kernel (exception rows inside), fix rows, update
         return 2 + (c->rbc_nf + (c->rbc_gm ? c->ngroups : 0) > 0 ? 1 : 0) + pre;
     return iteration_kernels(c, rb) + pre;
@@ -880,13 +891,25 @@ vofp_status build_graph_fp64(vofp_ctx* c, int U, bool rb) {
     cudaGraphNode_t node;
     vofp_status s = add_while(c, g, &h, &body, nullptr, 0, &node, 1u);
     if (s) return s;
+    c->launch_err = cudaSuccess;
     s = capture_into(c, cs, body, [&]() { launch_fp64_body(c, cs, U, rb, h, 1); });
-    if (s) return s;
-    VOFP_CUDA_TRY(c, cudaGraphInstantiate(&c->graph_fp64, g, 0));
+    cudaError_t ie = c->launch_err;
+    if (!s && ie == cudaSuccess) ie = cudaGraphInstantiate(&c->graph_fp64, g, 0);
     cudaGraphDestroy(g);
     cudaStreamDestroy(cs);
-    c->graph_fp64_key = graph_key(c, U, rb);
     c->launches = launches0;
+    if (s || ie != cudaSuccess) {
+        (void)cudaGetLastError();
+        c->graph_fp64 = nullptr;
+        if (c->pdl && c->mg_use) {   // chained launches refused inside the body: ordinary ones
+            c->pdl = 0;
+            return build_graph_fp64(c, U, rb);
+        }
+        if (s) return s;
+        c->set_error(std::string("cudaGraphInstantiate: ") + cudaGetErrorString(ie));
+        return VOFP_ERR_CUDA;
+    }
+    c->graph_fp64_key = graph_key(c, U, rb);
     return VOFP_OK;
 }
 
@@ -1098,9 +1121,10 @@ vofp_status solve_pass(vofp_ctx* c, const double* b, double* x, const vofp_solve
     if (o->mode == VOFP_MODE_MIXED && o->precond == VOFP_PRECOND_RBSGS && (s = rbc_ensure(c))) return s;
     // and the hierarchy of its coarse-grid correction
     c->mg_use = false;
-    if (o->mode == VOFP_MODE_MIXED && o->precond == VOFP_PRECOND_RBSGS && mg_wanted(c, o->rtol)) {
-        if ((s = mg_ensure(c))) return s;
-        c->mg_use = c->mg_ok;
+    if (o->precond == VOFP_PRECOND_RBSGS && mg_wanted(c, o->rtol)) {
+        const bool fp64 = o->mode != VOFP_MODE_MIXED;
+        if ((s = mg_ensure(c, fp64))) return s;
+        c->mg_use = fp64 ? c->mgd.ok : c->mgf.ok;
     }
     const long long N = c->d.n;
     cudaStream_t st = c->stream;
@@ -1172,6 +1196,8 @@ vofp_status solve_pass(vofp_ctx* c, const double* b, double* x, const vofp_solve
     launch(c, k_init_residual, stream_grid(N), kNT, st, N, rhs_loop, (const double*)c->q, (const double*)c->sq,
            (const uint32_t*)((rb && !mixed) ? c->excl_bits : c->slave_bits), c->r, c->sc, c->partials, c->counters);
     VOFP_CUDA_TRY(c, cudaMemsetAsync(c->p0, 0, sizeof(double) * N, st));
+    // the FP64 loop starts from z as well (the mixed one forms it at every inner start)
+    if (mg && !mixed) mg_precondition(c, st, true, false, 1);
     VOFP_CUDA_TRY(c, cudaMemcpyAsync(&h, c->sc, sizeof(h), cudaMemcpyDeviceToHost, st));
     VOFP_CUDA_TRY(c, cudaStreamSynchronize(st));
     if (!std::isfinite(h.rnorm2) || !std::isfinite(h.ref2) || !std::isfinite(h.rr)) {
@@ -1270,7 +1296,7 @@ vofp_status solve(vofp_ctx* c, const double* b, double* x, const vofp_solve_opts
     const long long max_iter = o->max_iter > 0 ? o->max_iter : 100000;
     if (r == VOFP_ERR_BREAKDOWN && c->mg_use && std::isfinite(acc.rel_residual) && acc.iterations < max_iter) {
         // the coarse-grid correction lost positivity: the plain red-black iteration from the iterate
-        c->mg_ok = false;
+        c->mgf.ok = c->mgd.ok = false;
         vofp_solve_opts o2 = *o;
         o2.x0_zero = 0;
         o2.max_iter = (int)(max_iter - acc.iterations);
