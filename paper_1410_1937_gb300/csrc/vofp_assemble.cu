@@ -687,6 +687,7 @@ vofp_status build_operator(vofp_ctx* c, const double* F, const double* ax, const
     c->built = false;
     c->rbc_built = false;
     c->rbc_ok = false;
+    c->grp_built = false;
     c->mgf.built = c->mgf.ok = false;
     c->mgd.built = c->mgd.ok = false;
     for (int f = 0; f < 6; ++f) c->bc[f] = bc->kind[f];

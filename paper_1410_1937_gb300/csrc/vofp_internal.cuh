@@ -25,14 +25,16 @@ constexpr int kBX = 32;          // stencil tile width (x), one warp
 constexpr int kBY = 8;           // stencil tile height (y)
 constexpr int kRedThreads = 256; // threads of the streaming/reduction kernels
 constexpr int kMaxPartials = 1 << 17;
+// block partials of p.Ap of an iteration's kernels, for the update: in the last quarter of the partials
+// buffer, which no other reduction of a loop uses
+constexpr int kPqBase = 3 * (kMaxPartials / 4);
 
 // Scalars of one CG run, resident in device memory so that the loop needs no host round trip.
 struct CgScalars {
     double rr;          // r.r of the (scaled) residual over the unknowns
     double rr0;         // r.r at the start of the current (inner) solve
-    double pq_raw;      // p.t summed over all cells by the stencil kernel (the colour-compact
-                        // red-black iteration leaves block partials for the update instead)
-    double pq_corr;     // merge-group correction to p.Ap
+    double pq_raw;      // p.Ap where the update takes it from here (the measurement hook; in a loop the
+                        // kernels before the update leave block partials)
     double alpha;       // step of the last completed iteration (used by the next stencil pass)
     double beta;        // direction coefficient for the next stencil pass
     double bnorm2;      // ||b_hat||^2 (unscaled)
@@ -215,6 +217,9 @@ struct vofp_ctx {
     long long rbc_cap = 0;            // allocated compact length
     int rbc_blocks_per_sm = 0;
     int rbc_rpt = 2;                  // rows per thread of the compact iteration kernel (tile 32 x 8 rpt)
+    uint32_t* grp_bits = nullptr;     // every cell of a merge group (Jacobi loops; of the current operator)
+    bool grp_built = false;
+    int pq_blocks = 0;                // blocks of the stencil launched last (partials of p.Ap it leaves)
     int rbc_nblocks = 0;              // iteration kernel blocks and work split (see rbc_split)
     vofp::RbcSplit rbc_split{};
     // coarse-grid correction of the red-black solves (vofp_mg.cu)
@@ -257,7 +262,8 @@ const CUtensorMap* tensor_map_f32_x(vofp_ctx* c, const float* ptr, int nxe, int 
 // TMA-fed fused red-black iteration, FP32 (vofp_rb_tma.cu): preparation and one launch (false
 // when it cannot run on this context; the caller then uses the register-prefetch kernel)
 void prepare_rb_tma(vofp_ctx* c);
-bool launch_cg_rb_tma(vofp_ctx* c, cudaStream_t st, const float* r, const float* po, float* pn, float* xv, float* q);
+bool launch_cg_rb_tma(vofp_ctx* c, cudaStream_t st, const float* r, const float* po, float* pn, float* xv, float* q,
+                      bool pdl);
 // colour-compact red-black inner solve (vofp_rbc.cu)
 vofp_status rbc_ensure(vofp_ctx* c);   // build the compact structures if eligible; sets c->rbc_ok
 void rbc_prep(vofp_ctx* c, cudaStream_t st, const double* rhs);   // inner start from the FP64 reduced rhs
@@ -269,13 +275,13 @@ int rbc_pq_parts(const vofp_ctx* c);   // block partials of p.Ap the compact ite
 bool mg_wanted(const vofp_ctx* c, double rtol);   // whether a red-black solve takes it
 vofp_status mg_ensure(vofp_ctx* c, bool fp64);    // hierarchy of the current operator; sets mgf.ok / mgd.ok
 void mg_precondition(vofp_ctx* c, cudaStream_t st, bool fp64, bool pdl, int start);   // z and beta from r
-void mg_update(vofp_ctx* c, cudaStream_t st, bool fp64, bool pdl, cudaGraphConditionalHandle h, int use_h);
+void mg_update(vofp_ctx* c, cudaStream_t st, bool fp64, bool pdl, cudaGraphConditionalHandle h, int use_h, int npq);
 int mg_precondition_kernels(const vofp_ctx* c, bool fp64);
 void rbc_time_kernel(vofp_ctx* c, cudaStream_t st);               // one iteration kernel launch
 void rbc_time_aux(vofp_ctx* c, cudaStream_t st);                  // the exception and group kernels of one iteration
 template <typename V>
 bool launch_cg_tma(vofp_ctx* c, cudaStream_t st, const V* Tx, const V* Ty, const V* Tz, const V* r, const V* po,
-                   V* pn, V* xv, V* q);
+                   V* pn, V* xv, V* q, bool pdl, bool groups);
 
 vofp_status build_operator(vofp_ctx* c, const double* F, const double* ax, const double* ay,
                            const double* az, const double* vf, const vofp_bc* bc,
@@ -364,7 +370,7 @@ void launch_stencil_apply_unscaled(vofp_ctx* c, const double* x, double* t);
 void launch_stencil_apply_scaled(vofp_ctx* c, const double* x, double* t);
 // merge-group patch after a scaled stencil: q_m = sum t + corr p_m, expanded; p.Ap correction
 template <typename V>
-void launch_group_patch(vofp_ctx* c, V* t, const V* p, bool dot_correction);
+void launch_group_patch(vofp_ctx* c, V* t, const V* p);
 
 // Launch a kernel on stream s and count it.
 template <typename... KArgs, typename... Args>

@@ -12,11 +12,12 @@
 //   stencil   p = r + beta p_old (shared-memory tile with halo), x += alpha p_old,
 //             t = (S A S) p with unit diagonal, p.t       (reads r, p_old, x, Tx, Ty, Tz;
 //                                                           writes p, x, t)
-//   patch     per merge group: q_m = sum_G t + corr_m p_m, written to every cell of G; adds
-//             corr_m p_m^2 to p.Ap                          (O(merged cells))
-//   update    alpha = r.r / p.Ap;  r -= alpha q;  r.r over the unknowns   (reads r, q; writes r)
-// Reductions: block partial sums, reduced in index order by the block that finishes last, so
-// results are bitwise reproducible from run to run.
+//   update    alpha = r.r / p.Ap;  r -= alpha q;  r.r over the unknowns   (reads r, q; writes r);
+//             q_m = sum_G t + corr_m p_m for each merge group  (O(merged cells))
+// (a red-black iteration writes the groups' q by a kernel between the two, k_group_patch).  The kernels of
+// a loop's graph are chained by programmatic dependent launches.
+// Reductions: block partial sums, reduced in a fixed order (p.Ap by every block of the update, the others by
+// the block that finishes last), so results are bitwise reproducible from run to run.
 #pragma once
 #include <type_traits>
 
@@ -76,8 +77,21 @@ __device__ __forceinline__ float fmav(float a, float b, float c) { return __fmaf
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Sum of the first nw (at most 32) warp values in sh. TREE: pairs of pairs, as an FP64 addition has to wait
+// some 60 cycles for the one before (eight in a row: 0.27 us); else in a row.
+template <bool TREE = false>
+__device__ __forceinline__ double sum_warps(const double* sh, int nw) {
+    double s = 0.0;
+    int w = 0;
+    for (; TREE && w + 8 <= nw; w += 8)
+        s += ((sh[w] + sh[w + 1]) + (sh[w + 2] + sh[w + 3])) + ((sh[w + 4] + sh[w + 5]) + (sh[w + 6] + sh[w + 7]));
+    for (; w < nw; ++w) s += sh[w];
+    return s;
+}
+
 // Reduce `part` over the grid; the last block to finish writes the sum (index order) to *out.
 // Returns true in thread 0 of that block.
+template <bool TREE = false>
 __device__ __forceinline__ bool grid_reduce(double part, double* partials, unsigned int* counter,
                                             double* sh, double* total) {
     __shared__ bool is_last;
@@ -90,9 +104,7 @@ __device__ __forceinline__ bool grid_reduce(double part, double* partials, unsig
     if ((tid & 31) == 0) sh[tid >> 5] = v;
     __syncthreads();
     if (tid == 0) {
-        double s = 0.0;
-        for (int w = 0; w < nt / 32; ++w) s += sh[w];
-        partials[b] = s;
+        partials[b] = sum_warps<TREE>(sh, nt / 32);
         __threadfence();
         unsigned int t = atomicAdd(counter, 1u);
         is_last = (t == (unsigned int)(nb - 1));
@@ -107,12 +119,46 @@ __device__ __forceinline__ bool grid_reduce(double part, double* partials, unsig
     if ((tid & 31) == 0) sh[tid >> 5] = s;
     __syncthreads();
     if (tid == 0) {
-        double tot = 0.0;
-        for (int w = 0; w < nt / 32; ++w) tot += sh[w];
-        *total = tot;
+        *total = sum_warps<TREE>(sh, nt / 32);
         *counter = 0u;
     }
     return tid == 0;
+}
+
+// This block's sum of v (fixed order) as its entry of `part`: p.Ap is left as block partials, which the
+// update kernel sums in every block, so that the kernels before it end without a fence, an atomic and a
+// last-block pass (with their launches chained: 128x64x64 FP64 35.0 -> 32.1 us an
+// iteration, 64x48x40 mixed 20.6 -> 16.6).
+template <bool TREE>
+__device__ __forceinline__ void block_partial(double v, double* part, double* sh) {
+    const int nt = blockDim.x * blockDim.y, tid = threadIdx.x + blockDim.x * threadIdx.y;
+    v = warp_sum(v);
+    if ((tid & 31) == 0) sh[tid >> 5] = v;
+    __syncthreads();
+    if (tid == 0) part[blockIdx.x] = sum_warps<TREE>(sh, nt / 32);
+}
+
+// The merge groups of a plain (not red-black) iteration.  A group's row is q_G = sum of its cells' stencil
+// rows + corr_G p_G.  The stencil kernel adds corr_G p_G^2 to p.Ap (p_G formed from r and p_old), and the
+// update takes the groups' r itself: no kernel between the two (mostly latency; FP64 128x64x64 32.1 -> 30.3 us
+// an iteration, 48x48x40 19.3 -> 17.1; mixed 250x123x62 34.5 -> 33.2).
+template <typename V>
+struct GroupList {
+    int n;
+    const int *ptr, *cells;
+    const double* corr;
+};
+// this thread's share of sum corr_G p_G^2
+template <typename V>
+__device__ __forceinline__ double group_corr(const GroupList<V>& gl, V beta, const V* __restrict__ r,
+                                             const V* __restrict__ pold, int tid, int nt) {
+    double s = 0.0;
+    for (int g = blockIdx.x * nt + tid; g < gl.n; g += gridDim.x * nt) {
+        const int m = gl.cells[gl.ptr[g]];
+        const double p = (double)fmav(beta, pold[m], r[m]);
+        s = fma(gl.corr[g] * p, p, s);
+    }
+    return s;
 }
 
 // Fused direction update + stencil + dot (ST_CG), or a plain operator apply.
@@ -134,7 +180,7 @@ __global__ void __launch_bounds__(kBX* kBY, 4)
 k_stencil(const Dims d, const int per_block, const V* __restrict__ Tx, const V* __restrict__ Ty,
           const V* __restrict__ Tz, const double* __restrict__ diag, const V* __restrict__ src,
           const V* __restrict__ pold, V* __restrict__ pnew, V* __restrict__ xv, V* __restrict__ out,
-          CgScalars* __restrict__ sc, double* __restrict__ partials, unsigned int* __restrict__ counter) {
+          const CgScalars* __restrict__ sc, double* __restrict__ pq_part, const GroupList<V> gl) {
     using Acc = typename AccFor<V>::type;
     constexpr bool CG = MODE == ST_CG;
     __shared__ V tile[4][kBY + 2][kBX + 2];
@@ -142,6 +188,7 @@ k_stencil(const Dims d, const int per_block, const V* __restrict__ Tx, const V* 
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + kBX * ty;
     V beta = V(0), alpha = V(0);
     if (CG) {
+        grid_dep_wait();
         beta = (V)sc->beta;
         alpha = (V)sc->alpha;
     }
@@ -267,21 +314,18 @@ k_stencil(const Dims d, const int per_block, const V* __restrict__ Tx, const V* 
             po_cur = po_next;
         }
     }
-    if (CG) {
-        double tot;
-        if (grid_reduce(acc.value(), partials, counter, sh, &tot)) sc->pq_raw = tot;
-    }
+    if (CG) block_partial<true>(acc.value() + group_corr(gl, beta, src, pold, tid, kBX * kBY), pq_part, sh);
 }
 
 template <typename V>
 __global__ void k_group_patch(int ng, const int* __restrict__ gptr, const int* __restrict__ gcells,
                               const double* __restrict__ gcorr, V* __restrict__ t,
-                              const V* __restrict__ p, int dot, CgScalars* sc,
-                              double* __restrict__ partials, unsigned int* __restrict__ counter) {
+                              const V* __restrict__ p, double* __restrict__ pq_part) {
     __shared__ double sh[32];
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    grid_dep_wait();
+    grid_dep_trigger();
     double part = 0.0;
-    if (g < ng) {
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x) {
         const int b = gptr[g], e = gptr[g + 1];
         const int m = gcells[b];
         double s = 0.0;
@@ -289,12 +333,9 @@ __global__ void k_group_patch(int ng, const int* __restrict__ gptr, const int* _
         const double pm = (double)p[m];
         const V qm = (V)(s + gcorr[g] * pm);
         for (int u = b; u < e; ++u) t[gcells[u]] = qm;
-        part = gcorr[g] * pm * pm;
+        part += gcorr[g] * pm * pm;
     }
-    if (dot) {
-        double tot;
-        if (grid_reduce(part, partials, counter, sh, &tot)) sc->pq_corr = tot;
-    }
+    if (pq_part) block_partial<false>(part, pq_part, sh);
 }
 
 __device__ __forceinline__ bool is_slave(const uint32_t* __restrict__ bits, long long c) {
@@ -304,15 +345,21 @@ __device__ __forceinline__ bool is_slave(const uint32_t* __restrict__ bits, long
 // alpha = r.r / p.Ap;  r -= alpha q;  r.r over the unknowns (cells that are not another cell's
 // group member).  The last block stores rr, beta = rr_new / rr_old, alpha, counts the iteration
 // and, for an inner (mixed-precision) loop, ends it when rr <= inner_rtol^2 rr0 or max_iter.
+// KIND: a red-black iteration (its sums in the order of their indices), a Jacobi one, or a Jacobi one with
+// merge groups. In the last `bits` marks every group cell: the vector path leaves those out, and the groups'
+// threads (from the last block on) sum their rows t from q, form q_G and write r to every cell of the group.
 // At most 64 registers (four 256-thread blocks per SM), so that a grid of four blocks per SM is one
 // wave.
-template <typename V, bool INNER>
+enum UpdateKind { UPD_RB = 0, UPD_JACOBI = 1, UPD_JACOBI_GROUPS = 2 };
+template <typename V, bool INNER, int KIND>
 __global__ void __launch_bounds__(kRedThreads, 4)
 k_cg_update(long long n, V* __restrict__ r, const V* __restrict__ q, const uint32_t* __restrict__ bits,
             CgScalars* sc, double* __restrict__ partials, unsigned int* __restrict__ counter,
-            cudaGraphConditionalHandle handle, int use_handle, const double* __restrict__ pq_part, int npq) {
-    __shared__ double sh[32];
-    __shared__ double s_alpha;
+            cudaGraphConditionalHandle handle, int use_handle, const double* __restrict__ pq_part, int npq1,
+            int npq, const GroupList<V> gl, const V* __restrict__ p) {
+    __shared__ double sh[32], sh2[32];
+    __shared__ double s_alpha, s_inv;
+    constexpr bool JACOBI = KIND != UPD_RB, GROUPS = KIND == UPD_JACOBI_GROUPS;
     __shared__ int s_flags;
     grid_dep_wait();
     using Acc = typename AccFor<V>::type;
@@ -339,30 +386,49 @@ k_cg_update(long long n, V* __restrict__ r, const V* __restrict__ q, const uint3
     // their latency overlaps the p.Ap sum and the division
     bool full = vi + (UN - 1) * stride < nv;
     if (full) load();
-    // p.Ap: with npq > 0 the kernels before left their block partials in pq_part and every block
-    // sums them itself, in the same fixed order (no last-block pass in those kernels); else the
-    // scalars hold it
+    // this thread's first group: its row does not depend on alpha either
+    auto group_row = [&](int g) {
+        double s = 0.0;
+        for (int u = gl.ptr[g]; u < gl.ptr[g + 1]; ++u) s += (double)q[gl.cells[u]];
+        return (V)(s + gl.corr[g] * (double)p[gl.cells[gl.ptr[g]]]);
+    };
+    const int g0 = (int)(gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;
+    const V qg0 = GROUPS && g0 < gl.n ? group_row(g0) : V(0);
+    // p.Ap: with npq > 0 the kernels before left their block partials in pq_part (npq1 of them from the
+    // first kernel) and every block sums them itself, in the same fixed order (no last-block pass in those
+    // kernels); else the scalars hold it
     double pq_sum = 0.0;
     if (npq > 0) {
         const int nt = blockDim.x;
         double v = 0.0;
-        for (int i = threadIdx.x; i < npq; i += nt) v += __ldcg(&pq_part[i]);
+        for (int i = threadIdx.x; i < npq1; i += nt) v += __ldcg(&pq_part[i]);
         v = warp_sum(v);
         if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+        if (!JACOBI && npq1 < npq) {
+            v = 0.0;
+            for (int i = npq1 + threadIdx.x; i < npq; i += nt) v += __ldcg(&pq_part[i]);
+            v = warp_sum(v);
+            if ((threadIdx.x & 31) == 0) sh2[threadIdx.x >> 5] = v;
+        }
         __syncthreads();
-        if (threadIdx.x == 0)
-            for (int wi = 0; wi < nt / 32; ++wi) pq_sum += sh[wi];
-        __syncthreads();
+        if (threadIdx.x == 0) {
+            pq_sum = sum_warps<JACOBI>(sh, nt / 32);
+            if (!JACOBI && npq1 < npq) pq_sum += sum_warps(sh2, nt / 32);
+        }
     }
     // the scalar step is computed once per block (FP64 division is slow on this part)
     if (threadIdx.x == 0) {
         const double rr = sc->rr;
-        const double pq = npq > 0 ? pq_sum : sc->pq_raw + sc->pq_corr;
+        const double pq = npq > 0 ? pq_sum : sc->pq_raw;
         // rr == 0: the residual vanished exactly (later unrolled iterations are no-ops)
         const bool ok = sc->status == VOFP_OK && (pq > 0.0) && isfinite(pq) && isfinite(rr) && rr > 0.0;
         const bool broke = !ok && !(rr == 0.0 && sc->status == VOFP_OK);
         s_alpha = ok ? rr / pq : 0.0;
         s_flags = (ok ? 1 : 0) | (broke ? 2 : 0);
+    } else if (JACOBI && threadIdx.x == 32) {
+        // 1 / r.r for beta, beside alpha's division instead of on the chain that ends the kernel
+        const double rr = sc->rr;
+        s_inv = rr > 0.0 ? 1.0 / rr : 0.0;
     }
     __syncthreads();
     const double alpha_d = s_alpha;
@@ -387,11 +453,34 @@ k_cg_update(long long n, V* __restrict__ r, const V* __restrict__ q, const uint3
             if (!(m & 8u)) acc.add(a.w, a.w);
         }
     };
+    // groups are few: nearly every word is stored whole
+    auto put = [&](long long at, const VV& a, uint32_t m) {
+        m &= (1u << VW) - 1u;
+        if (!GROUPS || m == 0u) {
+            rvp[at] = a;
+            return;
+        }
+        V* e = r + at * VW;
+        if constexpr (VW == 2) {
+            if (!(m & 1u)) e[0] = a.x;
+            if (!(m & 2u)) e[1] = a.y;
+        } else {
+            if (!(m & 1u)) e[0] = a.x;
+            if (!(m & 2u)) e[1] = a.y;
+            if (!(m & 4u)) e[2] = a.z;
+            if (!(m & 8u)) e[3] = a.w;
+        }
+    };
+    for (int g = g0; GROUPS && g < gl.n; g += (int)stride) {
+        const V rg = fmav(na, g == g0 ? qg0 : group_row(g), r[gl.cells[gl.ptr[g]]]);
+        for (int u = gl.ptr[g]; u < gl.ptr[g + 1]; ++u) r[gl.cells[u]] = rg;
+        acc.add(rg, rg);
+    }
     while (full) {
 #pragma unroll
         for (int u = 0; u < UN; ++u) {
             upd(rv[u], qv[u], w[u]);
-            rvp[vi + u * stride] = rv[u];
+            put(vi + u * stride, rv[u], w[u]);
         }
         vi += UN * stride;
         full = vi + (UN - 1) * stride < nv;
@@ -401,20 +490,22 @@ k_cg_update(long long n, V* __restrict__ r, const V* __restrict__ q, const uint3
         VV a = rvp[vi];
         const VV b = qvp[vi];
         const long long c0 = vi * VW;
-        upd(a, b, bits[c0 >> 5] >> (c0 & 31));
-        rvp[vi] = a;
+        const uint32_t m = bits[c0 >> 5] >> (c0 & 31);
+        upd(a, b, m);
+        put(vi, a, m);
     }
     for (long long c = nv * VW + blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += stride) {
+        if (GROUPS && is_slave(bits, c)) continue;
         V a = fmav(-alpha, q[c], r[c]);
         r[c] = a;
         if (!is_slave(bits, c)) acc.add(a, a);
     }
     double tot;
-    if (grid_reduce(acc.value(), partials, counter, sh, &tot)) {
+    if (grid_reduce<JACOBI>(acc.value(), partials, counter, sh, &tot)) {
         const double rr = sc->rr;
         sc->rr_prev = rr;
         sc->rr = tot;
-        sc->beta = (rr > 0.0) ? tot / rr : 0.0;
+        sc->beta = JACOBI ? tot * s_inv : (rr > 0.0) ? tot / rr : 0.0;
         sc->alpha = alpha_d;
         sc->iter += 1;
         sc->iter_total += 1;

@@ -35,7 +35,6 @@ namespace vofp {
 namespace {
 
 constexpr int kNT = 256;
-constexpr int kPqBase = 3 * (kMaxPartials / 4);   // the compact iteration's block partials of p.Ap
 // levels of at most kBottomCells cells are taken by one block, a thread per cell
 constexpr int kBottomCells = 512;
 constexpr int kBottomThreads = 512;
@@ -274,19 +273,14 @@ k_mg_update(const Dims d, const int nx1, const int ny1, const int n1, const long
     };
     if (t < items) load();
     if (UPD) {
-        double pq_sum = 0.0;
-        if (npq > 0) {
-            double v = 0.0;
-            for (int i = threadIdx.x; i < npq; i += kNT) v += __ldcg(&pq_part[i]);
-            v = warp_sum(v);
-            if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-            __syncthreads();
-            if (threadIdx.x == 0)
-                for (int wi = 0; wi < kNT / 32; ++wi) pq_sum += sh[wi];
-            __syncthreads();
-        }
+        double pq_sum = 0.0, v = 0.0;
+        for (int i = threadIdx.x; i < npq; i += kNT) v += __ldcg(&pq_part[i]);
+        v = warp_sum(v);
+        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+        __syncthreads();
+        if (threadIdx.x == 0) pq_sum = sum_warps<true>(sh, kNT / 32);
         if (threadIdx.x == 0) {
-            const double rr = sc->rr, rz = sc->rz, pq = npq > 0 ? pq_sum : sc->pq_raw + sc->pq_corr;
+            const double rr = sc->rr, rz = sc->rz, pq = pq_sum;
             // rr == 0: the residual vanished exactly (later unrolled iterations are no-ops)
             const bool ok = sc->status == VOFP_OK && pq > 0.0 && isfinite(pq) && isfinite(rr) && rr > 0.0 && rz > 0.0;
             const bool broke = !ok && !(rr == 0.0 && sc->status == VOFP_OK);
@@ -338,7 +332,7 @@ k_mg_update(const Dims d, const int nx1, const int ny1, const int n1, const long
         for (long long c = nh + blockIdx.x * kNT + threadIdx.x; c < nvec; c += stride)
             if (w[c] < T(0)) r[c] = fmav(na, q[c], r[c]);
     double tot;
-    if (grid_reduce(acc.value(), partials, counter, sh, &tot)) {
+    if (grid_reduce<true>(acc.value(), partials, counter, sh, &tot)) {
         const bool broke = s_flags != 0;
         sc->rr_prev = sc->rr;
         sc->rr = tot;
@@ -414,7 +408,7 @@ k_mg_direction(const Dims d, const int nx1, const int ny1, const int n1, const T
         }
     }
     double tot;
-    if (grid_reduce(acc.value(), partials, counter, sh, &tot)) {
+    if (grid_reduce<true>(acc.value(), partials, counter, sh, &tot)) {
         const double rz = sc->rr + tot;
         sc->rz = rz;
         double beta = sc->rz_prev > 0.0 ? rz / sc->rz_prev : 0.0;
@@ -827,14 +821,14 @@ void launch_direction(vofp_ctx* c, cudaStream_t st, bool pdl, int start) {
                (const int*)(COMPACT ? c->rbc_gref : c->gcells), c->sc, c->partials, c->counters, start);
 }
 template <bool COMPACT, bool UPD, typename T>
-void launch_update(vofp_ctx* c, cudaStream_t st, bool pdl, cudaGraphConditionalHandle h, int use_h) {
+void launch_update(vofp_ctx* c, cudaStream_t st, bool pdl, cudaGraphConditionalHandle h, int use_h, int npq) {
     MgSet<T>& m = set_of<T>(c);
     const MgLevel<T>& l = m.lv[0];
     const long long nh = COMPACT ? c->rbc_nh : c->d.n, nv = COMPACT ? c->rbc_nh + c->rbc_ne : c->d.n;
     launch_dep(c, pdl, k_mg_update<COMPACT, UPD, T>, dim3(grid_fine(l.n / MgEntries<COMPACT>::A)), dim3(kNT), 0, st, c->d,
                l.nx, l.ny, (int)l.n, nh, nv, vec_r<COMPACT, T>(c), vec_q<COMPACT, T>(c), (const T*)m.w,
                (const uint8_t*)c->mg_mask, (const int*)c->mg_even, l.b, c->sc, c->partials, c->counters, h, use_h,
-               (const double*)(c->partials + kPqBase), COMPACT ? rbc_pq_parts(c) : 0);
+               (const double*)(c->partials + kPqBase), npq);
 }
 
 // The hierarchy and the weights of the current operator (once per operator and precision).
@@ -908,7 +902,7 @@ vofp_status build(vofp_ctx* c) {
 
 template <bool COMPACT, typename T>
 void precondition(vofp_ctx* c, cudaStream_t st, bool pdl, int start) {
-    if (start) launch_update<COMPACT, false, T>(c, st, false, (cudaGraphConditionalHandle)0, 0);
+    if (start) launch_update<COMPACT, false, T>(c, st, false, (cudaGraphConditionalHandle)0, 0, 0);
     vcycle<T>(c, st, pdl, set_of<T>(c));
     launch_direction<COMPACT, T>(c, st, pdl, start);
 }
@@ -941,14 +935,14 @@ void mg_precondition(vofp_ctx* c, cudaStream_t st, bool fp64, bool pdl, int star
         precondition<false, float>(c, st, pdl, start);
 }
 
-// r -= alpha q, r.r, the inner loop's stop test and b_1
-void mg_update(vofp_ctx* c, cudaStream_t st, bool fp64, bool pdl, cudaGraphConditionalHandle h, int use_h) {
+// r -= alpha q, r.r, the inner loop's stop test and b_1; npq: block partials of p.Ap
+void mg_update(vofp_ctx* c, cudaStream_t st, bool fp64, bool pdl, cudaGraphConditionalHandle h, int use_h, int npq) {
     if (fp64)
-        launch_update<false, true, double>(c, st, pdl, h, use_h);
+        launch_update<false, true, double>(c, st, pdl, h, use_h, npq);
     else if (c->rbc_ok)
-        launch_update<true, true, float>(c, st, pdl, h, use_h);
+        launch_update<true, true, float>(c, st, pdl, h, use_h, npq);
     else
-        launch_update<false, true, float>(c, st, pdl, h, use_h);
+        launch_update<false, true, float>(c, st, pdl, h, use_h, npq);
 }
 
 int mg_precondition_kernels(const vofp_ctx* c, bool fp64) {

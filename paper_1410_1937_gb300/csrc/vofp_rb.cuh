@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(kBX* kBY, 3)
 k_cg_rb(const Dims d, const int per_block, const V* __restrict__ Tx, const V* __restrict__ Ty,
         const V* __restrict__ Tz, const uint32_t* __restrict__ red, const V* __restrict__ src,
         const V* __restrict__ pold, V* __restrict__ pnew, V* __restrict__ xv, V* __restrict__ out,
-        CgScalars* __restrict__ sc, double* __restrict__ partials, unsigned int* __restrict__ counter) {
+        const CgScalars* __restrict__ sc, double* __restrict__ pq_part) {
     using Acc = typename AccFor<V>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* sm = reinterpret_cast<V*>(smem_raw);
@@ -36,6 +36,7 @@ k_cg_rb(const Dims d, const int per_block, const V* __restrict__ Tx, const V* __
     auto ftile = [&](int kk) -> unsigned char* { return flags + ((kk + 8) & 3) * kPN; };
     __shared__ double sh[32];
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + kBX * ty;
+    grid_dep_wait();
     const V beta = (V)sc->beta, alpha = (V)sc->alpha;
     Acc acc;
     const int tiles_x = (d.nx + kBX - 1) / kBX;
@@ -196,8 +197,7 @@ k_cg_rb(const Dims d, const int per_block, const V* __restrict__ Tx, const V* __
             po = pn_;
         }
     }
-    double tot;
-    if (grid_reduce(acc.value(), partials, counter, sh, &tot)) sc->pq_raw = tot;
+    block_partial<false>(acc.value(), pq_part, sh);
 }
 
 template <typename V>

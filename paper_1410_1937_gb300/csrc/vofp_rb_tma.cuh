@@ -65,7 +65,7 @@ template <int NS, int TH>
 __global__ void __launch_bounds__(kBX* TH, TH == 8 ? 3 : 6)
 k_cg_rb_tma(const __grid_constant__ RbMaps maps, const Dims d, const int per_block, const float* __restrict__ pold,
             float* __restrict__ pnew, float* __restrict__ xv, float* __restrict__ out, CgScalars* __restrict__ sc,
-            double* __restrict__ partials, unsigned int* __restrict__ counter) {
+            double* __restrict__ pq_part) {
     using G = RbGeom<TH>;
     constexpr int PW = G::PW, BW = G::BW, NT = G::NT, PP = G::kPPer;
     extern __shared__ __align__(128) unsigned char rb_smem[];
@@ -75,6 +75,7 @@ k_cg_rb_tma(const __grid_constant__ RbMaps maps, const Dims d, const int per_blo
     uint64_t* bars = reinterpret_cast<uint64_t*>(wring + 3 * G::WN);
     __shared__ double sh[32];
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + kBX * ty;
+    grid_dep_wait();
     const float beta = (float)sc->beta, alpha = (float)sc->alpha;
     AccF2 acc;
     if (tid == 0) {
@@ -317,8 +318,7 @@ k_cg_rb_tma(const __grid_constant__ RbMaps maps, const Dims d, const int per_blo
             if (pending & (1u << s)) mbar_wait_bounded(&bars[s], (phase >> s) & 1u);
         if (tid == 0) atomicCAS(&sc->status, (int)VOFP_OK, (int)VOFP_ERR_DEVICE_TIMEOUT);
     }
-    double tot;
-    if (grid_reduce(acc.value(), partials, counter, sh, &tot)) sc->pq_raw = tot;
+    block_partial<false>(acc.value(), pq_part, sh);
 }
 
 }  // namespace vofp

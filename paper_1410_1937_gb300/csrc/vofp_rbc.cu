@@ -25,9 +25,6 @@ namespace {
 
 constexpr int kNT = 256;
 constexpr int kRbcStages = 3;
-// the iteration kernel's and the fix rows' block partials of p.Ap live in the last quarter of the
-// partials buffer (no other reduction of an inner iteration uses it)
-constexpr int kPqBase = 3 * (kMaxPartials / 4);
 constexpr int kChunk = 2048;            // cells per block of the compaction passes (8 per thread)
 
 int grid_n(long long n) {
@@ -713,7 +710,7 @@ void rbc_iteration(vofp_ctx* c, cudaStream_t st, const float* po, float* pn, cud
     launch_main(c, st, po, pn, pdl);
     rbc_aux(c, st, po, pn, pdl);
     if (c->mg_use) {
-        mg_update(c, st, false, pdl, h, use_h);
+        mg_update(c, st, false, pdl, h, use_h, rbc_pq_parts(c));
         mg_precondition(c, st, false, pdl, 0);
         return;
     }
@@ -721,9 +718,9 @@ void rbc_iteration(vofp_ctx* c, cudaStream_t st, const float* po, float* pn, cud
     // the update: one wave of four 256-thread blocks per SM (its register cap); two waves of eight
     // per SM took 7.5 us more per iteration at 512x256x128
     const int ug = std::min(grid_n(nc / 4 + 1), num_sms() * 4);
-    launch_dep(c, pdl, k_cg_update<float, true>, dim3(ug), dim3(kNT), 0, st, nc, c->rbc_r,
+    launch_dep(c, pdl, k_cg_update<float, true, UPD_RB>, dim3(ug), dim3(kNT), 0, st, nc, c->rbc_r,
                (const float*)c->rbc_q, (const uint32_t*)c->rbc_bits, c->sc, c->partials, c->counters, h, use_h,
-               (const double*)(c->partials + kPqBase), rbc_pq_parts(c));
+               (const double*)(c->partials + kPqBase), rbc_pq_parts(c), rbc_pq_parts(c), GroupList<float>{}, (const float*)nullptr);
 }
 
 void rbc_finish_xf(vofp_ctx* c, cudaStream_t st) {

@@ -69,23 +69,25 @@ void prepare_kernels(vofp_ctx* c) {
 // kernel where its tensor maps can be built, else the register-prefetch kernel.
 template <typename V>
 void launch_cg_stencil(vofp_ctx* c, cudaStream_t st, const V* Tx, const V* Ty, const V* Tz, const V* r,
-                       const V* po, V* pn, V* xv, V* q) {
-    if (launch_cg_tma(c, st, Tx, Ty, Tz, r, po, pn, xv, q)) return;
-    launch(c, k_stencil<V, ST_CG, stencil_pf<V>()>, stencil_grid(c), dim3(kBX, kBY), st, c->d, stencil_per_block(c),
-           Tx, Ty, Tz, (const double*)nullptr, r, po, pn, xv, q, c->sc, c->partials, c->counters);
+                       const V* po, V* pn, V* xv, V* q, bool pdl, bool groups) {
+    if (launch_cg_tma(c, st, Tx, Ty, Tz, r, po, pn, xv, q, pdl, groups)) return;
+    launch_dep(c, pdl, k_stencil<V, ST_CG, stencil_pf<V>()>, stencil_grid(c), dim3(kBX, kBY), 0, st, c->d,
+               stencil_per_block(c), Tx, Ty, Tz, (const double*)nullptr, r, po, pn, xv, q, (const CgScalars*)c->sc,
+               c->partials + kPqBase, GroupList<V>{groups ? c->ngroups : 0, c->gptr, c->gcells, c->gcorr});
+    c->pq_blocks = stencil_blocks(c);
 }
 
 // one fused red-black CG iteration (k_cg_rb)
 template <typename V>
 void launch_cg_rb(vofp_ctx* c, cudaStream_t st, const V* Tx, const V* Ty, const V* Tz, const V* r,
-                  const V* po, V* pn, V* xv, V* q) {
+                  const V* po, V* pn, V* xv, V* q, bool pdl) {
     if constexpr (sizeof(V) == 4) {
-        if (launch_cg_rb_tma(c, st, r, po, pn, xv, q)) return;
+        if (launch_cg_rb_tma(c, st, r, po, pn, xv, q, pdl)) return;
     }
     constexpr size_t smem = cg_rb_smem<V>();
-    launch_smem(c, k_cg_rb<V, stencil_pf<V>()>, dim3(rb_blocks(c)), dim3(kBX, kBY), smem, st, c->d,
-                rb_per_block(c), Tx, Ty, Tz, (const uint32_t*)c->red_bits, r, po, pn, xv, q, c->sc, c->partials,
-                c->counters);
+    launch_dep(c, pdl, k_cg_rb<V, stencil_pf<V>()>, dim3(rb_blocks(c)), dim3(kBX, kBY), smem, st, c->d, rb_per_block(c), Tx,
+               Ty, Tz, (const uint32_t*)c->red_bits, r, po, pn, xv, q, (const CgScalars*)c->sc, c->partials + kPqBase);
+    c->pq_blocks = rb_blocks(c);
 }
 
 // x_t[c] = x0[root(c)] * sq[c] (scaled initial guess, expanded over groups; 0 without unknown)
@@ -212,7 +214,6 @@ __global__ void k_sum_unknowns(long long n, const double* __restrict__ x, const 
 
 __global__ void k_set_pq_inf(CgScalars* sc, int timing) {
     sc->pq_raw = INFINITY;
-    sc->pq_corr = 0.0;
     sc->alpha = 0.0;
     sc->beta = 0.0;
     sc->timing = timing;
@@ -627,24 +628,40 @@ __global__ void k_to_float(long long n, const double* __restrict__ a, float* __r
 
 void launch_stencil_apply_unscaled(vofp_ctx* c, const double* x, double* t) {
     launch(c, k_stencil<double, ST_APPLY_UNSCALED, 1>, stencil_grid(c), dim3(kBX, kBY), c->stream, 
-        c->d, stencil_per_block(c), c->Tx, c->Ty, c->Tz, c->diag, x, nullptr, nullptr, nullptr, t, c->sc, c->partials, c->counters);
+        c->d, stencil_per_block(c), c->Tx, c->Ty, c->Tz, c->diag, x, nullptr, nullptr, nullptr, t, c->sc, nullptr, GroupList<double>{});
 }
 
 void launch_stencil_apply_scaled(vofp_ctx* c, const double* x, double* t) {
     launch(c, k_stencil<double, ST_APPLY_SCALED, 1>, stencil_grid(c), dim3(kBX, kBY), c->stream, 
-        c->d, stencil_per_block(c), c->Txs, c->Tys, c->Tzs, nullptr, x, nullptr, nullptr, nullptr, t, c->sc, c->partials, c->counters);
+        c->d, stencil_per_block(c), c->Txs, c->Tys, c->Tzs, nullptr, x, nullptr, nullptr, nullptr, t, c->sc, nullptr, GroupList<double>{});
 }
 
 template <typename V>
-void launch_group_patch(vofp_ctx* c, V* t, const V* p, bool dot) {
+void launch_group_patch(vofp_ctx* c, V* t, const V* p) {
     if (c->ngroups == 0) return;
     launch(c, k_group_patch<V>, ceil_div(c->ngroups, kNT), kNT, c->stream, c->ngroups, c->gptr, c->gcells, c->gcorr, t, p,
-                                                                        dot ? 1 : 0, c->sc, c->partials, c->counters);
+           (double*)nullptr);
 }
-template void launch_group_patch<double>(vofp_ctx*, double*, const double*, bool);
-template void launch_group_patch<float>(vofp_ctx*, float*, const float*, bool);
+template void launch_group_patch<double>(vofp_ctx*, double*, const double*);
+template void launch_group_patch<float>(vofp_ctx*, float*, const float*);
 
 namespace {
+
+__global__ void k_group_bits(int n, const int* __restrict__ cells, uint32_t* __restrict__ bits) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < n) atomicOr(&bits[cells[t] >> 5], 1u << (cells[t] & 31));
+}
+// bit of every cell of a merge group (once per operator)
+vofp_status ensure_group_bits(vofp_ctx* c) {
+    if (c->ngroups == 0 || c->grp_built) return VOFP_OK;
+    vofp_status s;
+    if (!c->grp_bits && (s = c->alloc(&c->grp_bits, (c->d.n + 31) / 32))) return s;
+    VOFP_CUDA_TRY(c, cudaMemsetAsync(c->grp_bits, 0, sizeof(uint32_t) * ((c->d.n + 31) / 32), c->stream));
+    const int n = (int)(c->n_merged + c->ngroups);   // the groups' cells: merged ones and masters
+    launch(c, k_group_bits, ceil_div(n, kNT), kNT, c->stream, n, (const int*)c->gcells, c->grp_bits);
+    c->grp_built = true;
+    return VOFP_OK;
+}
 
 // one CG iteration on stream st (FP64 or FP32), reading p_old from `po` and writing `pn`; in
 // red-black mode the red half-stencil runs first and the stencil skips red rows
@@ -652,9 +669,11 @@ template <typename V>
 void launch_cg_iteration(vofp_ctx* c, cudaStream_t st, V* r, V* po, V* pn, V* xv, V* q,
                          const V* Tx, const V* Ty, const V* Tz, bool inner, bool rb,
                          cudaGraphConditionalHandle h, int use_h) {
-    const uint32_t* bits = rb ? c->excl_bits : c->slave_bits;
     constexpr bool fp64 = sizeof(V) == 8;
     const bool mg = rb && c->mg_use;
+    // in the loops' graphs the iteration's kernels are chained (a refused launch is caught when the capture
+    // ends): each waits for its predecessor before it reads
+    const bool pdl = c->pdl != 0 && use_h != 0;
     if (rb) {
         const V* src = r;
         if constexpr (fp64) {
@@ -662,32 +681,42 @@ void launch_cg_iteration(vofp_ctx* c, cudaStream_t st, V* r, V* po, V* pn, V* xv
         } else {
             if (mg) src = c->mgf.z;
         }
-        launch_cg_rb<V>(c, st, Tx, Ty, Tz, src, po, pn, xv, q);
+        launch_cg_rb<V>(c, st, Tx, Ty, Tz, src, po, pn, xv, q, pdl);
     } else {
-        launch_cg_stencil<V>(c, st, Tx, Ty, Tz, r, po, pn, xv, q);
+        launch_cg_stencil<V>(c, st, Tx, Ty, Tz, r, po, pn, xv, q, pdl, true);
     }
-    if (c->ngroups > 0)
-        launch(c, k_group_patch<V>, ceil_div(c->ngroups, kNT), kNT, st, c->ngroups, c->gptr, c->gcells, c->gcorr, q, pn,
-               1, c->sc, c->partials, c->counters);
+    double* part = c->partials + kPqBase;
+    int npq = c->pq_blocks;
+    if (rb && c->ngroups > 0) {
+        // as many blocks as the partials' place has room for beside the stencil's
+        const int pb = std::min(ceil_div(c->ngroups, kNT), kMaxPartials / 8);
+        launch_dep(c, pdl, k_group_patch<V>, dim3(pb), dim3(kNT), 0, st, c->ngroups, (const int*)c->gptr,
+                   (const int*)c->gcells, (const double*)c->gcorr, q, (const V*)pn, part + npq);
+        npq += pb;
+    }
     if (mg) {
-        // chained launches in the loops' graphs (a refused one is caught when the capture ends)
-        const bool pdl = c->pdl != 0 && use_h != 0;
-        mg_update(c, st, fp64, pdl, h, inner ? use_h : 0);
+        mg_update(c, st, fp64, pdl, h, inner ? use_h : 0, npq);
         mg_precondition(c, st, fp64, pdl, 0);
         return;
     }
-    if (inner)
-        launch(c, k_cg_update<V, true>, stream_grid(c->d.n / (sizeof(V) == 8 ? 2 : 4) + 1), kNT, st,
-               c->d.n, r, (const V*)q, bits, c->sc, c->partials, c->counters, h, use_h, (const double*)nullptr, 0);
+    const dim3 g(stream_grid(c->d.n / (fp64 ? 2 : 4) + 1));
+    const GroupList<V> gl{rb ? 0 : c->ngroups, c->gptr, c->gcells, c->gcorr};
+    const uint32_t* bits = rb ? c->excl_bits : gl.n > 0 ? c->grp_bits : c->slave_bits;
+    auto update = [&](auto k) {
+        launch_dep(c, pdl, k, g, dim3(kNT), 0, st, c->d.n, r, (const V*)q, bits, c->sc, c->partials, c->counters, h, use_h,
+                   (const double*)part, c->pq_blocks, npq, gl, (const V*)pn);
+    };
+    if (gl.n > 0)
+        inner ? update(k_cg_update<V, true, UPD_JACOBI_GROUPS>) : update(k_cg_update<V, false, UPD_JACOBI_GROUPS>);
+    else if (!rb)
+        inner ? update(k_cg_update<V, true, UPD_JACOBI>) : update(k_cg_update<V, false, UPD_JACOBI>);
     else
-        launch(c, k_cg_update<V, false>, stream_grid(c->d.n / (sizeof(V) == 8 ? 2 : 4) + 1), kNT, st,
-               c->d.n, r, (const V*)q, bits, c->sc, c->partials, c->counters, h, use_h, (const double*)nullptr, 0);
+        inner ? update(k_cg_update<V, true, UPD_RB>) : update(k_cg_update<V, false, UPD_RB>);
 }
 
 // kernels of one iteration (for the launch count of graph executions)
 int iteration_kernels(const vofp_ctx* c, bool rb) {
-    (void)rb;
-    return 2 + (c->ngroups > 0 ? 1 : 0);
+    return 2 + (rb && c->ngroups > 0 ? 1 : 0);
 }
 
 // Mixed precision, red-black: the reduced right-hand side r_S + E_SR r_R of the correction
@@ -803,12 +832,10 @@ void launch_outer_head(vofp_ctx* c, cudaStream_t st, bool rb, cudaGraphCondition
                        cudaGraphConditionalHandle hi, int use_h) {
     launch(c, k_stencil<double, ST_APPLY_SCALED, 1>, stencil_grid(c), dim3(kBX, kBY), st, c->d, stencil_per_block(c),
            (const double*)c->Txs, (const double*)c->Tys, (const double*)c->Tzs, (const double*)nullptr,
-           (const double*)c->xt, (const double*)nullptr, (double*)nullptr, (double*)nullptr, c->q, c->sc, c->partials,
-           c->counters);
+           (const double*)c->xt, (const double*)nullptr, (double*)nullptr, (double*)nullptr, c->q, c->sc, (double*)nullptr, GroupList<double>{});
     if (c->ngroups > 0)
         launch(c, k_group_patch<double>, ceil_div(c->ngroups, kNT), kNT, st, c->ngroups, (const int*)c->gptr,
-               (const int*)c->gcells, (const double*)c->gcorr, c->q, (const double*)c->xt, 0, c->sc, c->partials,
-               c->counters);
+               (const int*)c->gcells, (const double*)c->gcorr, c->q, (const double*)c->xt, (double*)nullptr);
     launch(c, k_outer_residual, stream_grid(c->d.n), kNT, st, c->d.n, (const double*)c->bt, (const double*)c->q,
            (const double*)c->sq, (const uint32_t*)c->slave_bits, c->r, c->sc, c->partials, c->counters, ho, hi, use_h);
     if (rb) {
@@ -901,7 +928,7 @@ vofp_status build_graph_fp64(vofp_ctx* c, int U, bool rb) {
     if (s || ie != cudaSuccess) {
         (void)cudaGetLastError();
         c->graph_fp64 = nullptr;
-        if (c->pdl && c->mg_use) {   // chained launches refused inside the body: ordinary ones
+        if (c->pdl) {   // chained launches refused inside the body: ordinary ones
             c->pdl = 0;
             return build_graph_fp64(c, U, rb);
         }
@@ -1128,6 +1155,7 @@ vofp_status solve_pass(vofp_ctx* c, const double* b, double* x, const vofp_solve
     }
     const long long N = c->d.n;
     cudaStream_t st = c->stream;
+    if (o->precond == VOFP_PRECOND_JACOBI && (s = ensure_group_bits(c))) return s;
     // Default: the FP64 loop checks its true residual every 8 iterations, and so does the mixed
     // solve's inner loop below 2^20 cells; from 2^20 cells on it tests its stop every 64. An inner
     // solve runs on to the end of its unrolled body past its target, and on large systems, where
@@ -1173,12 +1201,12 @@ vofp_status solve_pass(vofp_ctx* c, const double* b, double* x, const vofp_solve
                (const double*)c->Tzs, (const uint32_t*)c->red_bits, (const double*)c->xt, (const double*)nullptr,
                c->p1, 1);
         launch_stencil_apply_scaled(c, c->p1, c->q);
-        launch_group_patch<double>(c, c->q, c->xt, false);
+        launch_group_patch<double>(c, c->q, c->xt);
         rhs_loop = c->work;
         VOFP_CUDA_TRY(c, cudaMemsetAsync(c->p1, 0, sizeof(double) * N, st));
     } else {
         launch_stencil_apply_scaled(c, c->xt, c->q);
-        launch_group_patch<double>(c, c->q, c->xt, false);
+        launch_group_patch<double>(c, c->q, c->xt);
     }
     CgScalars h{};
     h.status = VOFP_OK;
@@ -1389,11 +1417,11 @@ vofp_status solve_fcg(vofp_ctx* c, const double* b, double* x, const vofp_solve_
     auto apply_f = [&](cudaStream_t ss, const float* p, float* q) {
         launch(c, k_stencil<float, ST_APPLY_SCALED, 2>, stencil_grid(c), dim3(kBX, kBY), ss, c->d,
                stencil_per_block(c), (const float*)c->Txf, (const float*)c->Tyf, (const float*)c->Tzf,
-               (const double*)nullptr, p, (const float*)nullptr, (float*)nullptr, (float*)nullptr, q, c->sc,
-               c->partials, c->counters);
+               (const double*)nullptr, p, (const float*)nullptr, (float*)nullptr, (float*)nullptr, q, (const CgScalars*)c->sc,
+               (double*)nullptr, GroupList<float>{});
         if (c->ngroups > 0)
             launch(c, k_group_patch<float>, ceil_div(c->ngroups, kNT), kNT, ss, c->ngroups, (const int*)c->gptr,
-                   (const int*)c->gcells, (const double*)c->gcorr, q, p, 0, c->sc, c->partials, c->counters);
+                   (const int*)c->gcells, (const double*)c->gcorr, q, p, (double*)nullptr);
     };
     // one FCG iteration: direction and step into (p, q), previous direction in (pp, qp)
     auto iteration = [&](cudaStream_t ss, float* p, float* q, const float* pp, const float* qp,
@@ -1464,7 +1492,7 @@ vofp_status solve_fcg(vofp_ctx* c, const double* b, double* x, const vofp_solve_
     for (;;) {
         // FP64 residual of the scaled system and its true (unscaled) norm
         launch_stencil_apply_scaled(c, c->xt, c->q);
-        launch_group_patch<double>(c, c->q, c->xt, false);
+        launch_group_patch<double>(c, c->q, c->xt);
         CgScalars h{};
         h.status = VOFP_OK;
         VOFP_CUDA_TRY(c, cudaMemcpyAsync(c->sc, &h, sizeof(h), cudaMemcpyHostToDevice, st));
@@ -1572,11 +1600,10 @@ vofp_status nn_train_anorm(vofp_ctx* c, vofp_nn* nn, const float* r, const float
                (const int*)c->gcells, z);
     launch(c, k_stencil<float, ST_APPLY_SCALED, 2>, stencil_grid(c), dim3(kBX, kBY), st, c->d, stencil_per_block(c),
            (const float*)c->Txf, (const float*)c->Tyf, (const float*)c->Tzf, (const double*)nullptr, (const float*)z,
-           (const float*)nullptr, (float*)nullptr, (float*)nullptr, c->qf, c->sc, c->partials, c->counters);
+           (const float*)nullptr, (float*)nullptr, (float*)nullptr, c->qf, (const CgScalars*)c->sc, (double*)nullptr, GroupList<float>{});
     if (c->ngroups > 0)
         launch(c, k_group_patch<float>, ceil_div(c->ngroups, kNT), kNT, st, c->ngroups, (const int*)c->gptr,
-               (const int*)c->gcells, (const double*)c->gcorr, c->qf, (const float*)z, 0, c->sc, c->partials,
-               c->counters);
+               (const int*)c->gcells, (const double*)c->gcorr, c->qf, (const float*)z, (double*)nullptr);
     double* sums = c->partials + kMaxPartials - 48;
     launch(c, k_anorm_dots, stream_grid(N), kNT, st, N, (const float*)z, (const float*)c->qf, r, e,
            (const uint32_t*)c->slave_bits, c->partials, c->counters, sums);
@@ -1648,34 +1675,34 @@ vofp_status time_iteration_kernels(vofp_ctx* c, int precision, bool rb, int reps
         const long long nc = c->rbc_nh + c->rbc_ne;
         auto stn = [&]() { rbc_time_kernel(c, st); };
         auto upd = [&]() {
-            launch(c, k_cg_update<float, false>, stream_grid(nc / 4 + 1), kNT, st, nc, c->rbc_r,
+            launch(c, k_cg_update<float, false, UPD_RB>, stream_grid(nc / 4 + 1), kNT, st, nc, c->rbc_r,
                    (const float*)c->rbc_q, (const uint32_t*)c->rbc_bits, c->sc, c->partials, c->counters,
-                   (cudaGraphConditionalHandle)0, 0, (const double*)nullptr, 0);
+                   (cudaGraphConditionalHandle)0, 0, (const double*)nullptr, 0, 0, GroupList<float>{}, (const float*)nullptr);
         };
         auto aux = [&]() { rbc_time_aux(c, st); };
         if ((s = timed(stn, &t1)) || (s = timed(upd, &t2)) || (s = timed(aux, &t3))) return s;
     } else if (precision == 32) {
         auto stn = [&]() {
             if (rb)
-                launch_cg_rb<float>(c, st, c->Txf, c->Tyf, c->Tzf, c->rf, c->pf0, c->pf1, c->xf, c->qf);
+                launch_cg_rb<float>(c, st, c->Txf, c->Tyf, c->Tzf, c->rf, c->pf0, c->pf1, c->xf, c->qf, false);
             else
-                launch_cg_stencil<float>(c, st, c->Txf, c->Tyf, c->Tzf, c->rf, c->pf0, c->pf1, c->xf, c->qf);
+                launch_cg_stencil<float>(c, st, c->Txf, c->Tyf, c->Tzf, c->rf, c->pf0, c->pf1, c->xf, c->qf, false, false);
         };
         auto upd = [&]() {
-            launch(c, k_cg_update<float, false>, stream_grid(N / 4 + 1), kNT, st, N, c->rf, (const float*)c->qf, bits,
-                   c->sc, c->partials, c->counters, (cudaGraphConditionalHandle)0, 0, (const double*)nullptr, 0);
+            launch(c, k_cg_update<float, false, UPD_RB>, stream_grid(N / 4 + 1), kNT, st, N, c->rf, (const float*)c->qf, bits,
+                   c->sc, c->partials, c->counters, (cudaGraphConditionalHandle)0, 0, (const double*)nullptr, 0, 0, GroupList<float>{}, (const float*)nullptr);
         };
         if ((s = timed(stn, &t1)) || (s = timed(upd, &t2))) return s;
     } else {
         auto stn = [&]() {
             if (rb)
-                launch_cg_rb<double>(c, st, c->Txs, c->Tys, c->Tzs, c->r, c->p0, c->p1, c->xt, c->q);
+                launch_cg_rb<double>(c, st, c->Txs, c->Tys, c->Tzs, c->r, c->p0, c->p1, c->xt, c->q, false);
             else
-                launch_cg_stencil<double>(c, st, c->Txs, c->Tys, c->Tzs, c->r, c->p0, c->p1, c->xt, c->q);
+                launch_cg_stencil<double>(c, st, c->Txs, c->Tys, c->Tzs, c->r, c->p0, c->p1, c->xt, c->q, false, false);
         };
         auto upd = [&]() {
-            launch(c, k_cg_update<double, false>, stream_grid(N / 2 + 1), kNT, st, N, c->r, (const double*)c->q, bits,
-                   c->sc, c->partials, c->counters, (cudaGraphConditionalHandle)0, 0, (const double*)nullptr, 0);
+            launch(c, k_cg_update<double, false, UPD_RB>, stream_grid(N / 2 + 1), kNT, st, N, c->r, (const double*)c->q, bits,
+                   c->sc, c->partials, c->counters, (cudaGraphConditionalHandle)0, 0, (const double*)nullptr, 0, 0, GroupList<double>{}, (const double*)nullptr);
         };
         if ((s = timed(stn, &t1)) || (s = timed(upd, &t2))) return s;
     }

@@ -59,7 +59,7 @@ const CUtensorMap* tensor_map(vofp_ctx* c, const V* ptr, int bw, int bh, int nxe
 
 template <typename V, int NS, int CPT>
 bool launch_tma(vofp_ctx* c, cudaStream_t st, const V* Tx, const V* Ty, const V* Tz, const V* r, const V* po,
-                   V* pn, V* xv, V* q, bool column = false) {
+                   V* pn, V* xv, V* q, bool pdl, const GroupList<V>& gl, bool column = false) {
     using G = TmaGeom<V, CPT>;
     const CUtensorMap *mr = tensor_map(c, r, G::kHW, kBY + 2), *mp = tensor_map(c, po, G::kHW, kBY + 2),
                       *mx = tensor_map(c, Tx, G::kHW, kBY), *my = tensor_map(c, Ty, G::TW, kBY + 1),
@@ -77,8 +77,9 @@ bool launch_tma(vofp_ctx* c, cudaStream_t st, const V* Tx, const V* Ty, const V*
     int nb = 1, per = 1;
     const int per_sm = (sizeof(V) == 4 && NS == 6 && CPT == 2) ? c->tma_blocks_deep32 : c->tma_blocks_per_sm[f64];
     plane_split(tiles, c->d.nz, (long long)num_sms() * per_sm, column, &nb, &per);
-    launch_smem(c, k_cg_tma<V, NS, CPT>, dim3(nb), dim3(kBX, kBY), cg_tma_smem<V, NS, CPT>(), st, maps, c->d, per,
-                pn, xv, q, c->sc, c->partials, c->counters);
+    launch_dep(c, pdl, k_cg_tma<V, NS, CPT>, dim3(nb), dim3(kBX, kBY), cg_tma_smem<V, NS, CPT>(), st, maps, c->d, per, pn,
+               xv, q, c->sc, c->partials + kPqBase, gl, r, po);
+    c->pq_blocks = nb;
     return true;
 }
 
@@ -94,12 +95,13 @@ const CUtensorMap* tensor_map_f32_x(vofp_ctx* c, const float* ptr, int nxe, int 
 
 template <typename V>
 bool launch_cg_tma(vofp_ctx* c, cudaStream_t st, const V* Tx, const V* Ty, const V* Tz, const V* r, const V* po,
-                   V* pn, V* xv, V* q) {
+                   V* pn, V* xv, V* q, bool pdl, bool groups) {
+    const GroupList<V> gl{groups ? c->ngroups : 0, c->gptr, c->gcells, c->gcorr};
     if constexpr (sizeof(V) == 8) {
-        return c->tma_ok[1] && launch_tma<double, kTmaStages64, 1>(c, st, Tx, Ty, Tz, r, po, pn, xv, q);
+        return c->tma_ok[1] && launch_tma<double, kTmaStages64, 1>(c, st, Tx, Ty, Tz, r, po, pn, xv, q, pdl, gl);
     } else {
         if (!c->tma_ok[0]) return false;
-        if (c->tma_cpt32 == 1) return launch_tma<float, 6, 1>(c, st, Tx, Ty, Tz, r, po, pn, xv, q);
+        if (c->tma_cpt32 == 1) return launch_tma<float, 6, 1>(c, st, Tx, Ty, Tz, r, po, pn, xv, q, pdl, gl);
         // Column split with six stages when the tile columns fill, without exceeding, one wave of
         // the six-stage kernel (two blocks per SM): every block marches a whole column in step with
         // its neighbours (halo rows from L2, four planes in flight per block; measured 0.096 against
@@ -108,14 +110,14 @@ bool launch_cg_tma(vofp_ctx* c, cudaStream_t st, const V* Tx, const V* Ty, const
         const long long tiles = (long long)ceil_div(c->d.nx, 2 * kBX) * ceil_div(c->d.ny, kBY);
         const long long deep = (long long)num_sms() * c->tma_blocks_deep32;
         if (deep > 0 && tiles <= deep && 2 * tiles > deep)
-            return launch_tma<float, 6, 2>(c, st, Tx, Ty, Tz, r, po, pn, xv, q, true);
-        return launch_tma<float, 4, 2>(c, st, Tx, Ty, Tz, r, po, pn, xv, q, false);
+            return launch_tma<float, 6, 2>(c, st, Tx, Ty, Tz, r, po, pn, xv, q, pdl, gl, true);
+        return launch_tma<float, 4, 2>(c, st, Tx, Ty, Tz, r, po, pn, xv, q, pdl, gl, false);
     }
 }
 template bool launch_cg_tma<float>(vofp_ctx*, cudaStream_t, const float*, const float*, const float*, const float*,
-                                   const float*, float*, float*, float*);
+                                   const float*, float*, float*, float*, bool, bool);
 template bool launch_cg_tma<double>(vofp_ctx*, cudaStream_t, const double*, const double*, const double*,
-                                    const double*, const double*, double*, double*, double*);
+                                    const double*, const double*, double*, double*, double*, bool, bool);
 
 // Opt the TMA stencil kernels into their dynamic shared memory, size their persistent grids and
 // decide per precision whether the tensor maps can be built.

@@ -131,8 +131,8 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
 template <typename V, int NS, int CPT>
 __global__ void __launch_bounds__(kBX* kBY)
 k_cg_tma(const __grid_constant__ CgMaps maps, const Dims d, const int per_block, V* __restrict__ pnew,
-         V* __restrict__ xv, V* __restrict__ out, CgScalars* __restrict__ sc, double* __restrict__ partials,
-         unsigned int* __restrict__ counter) {
+         V* __restrict__ xv, V* __restrict__ out, CgScalars* __restrict__ sc, double* __restrict__ pq_part,
+         const GroupList<V> gl, const V* __restrict__ r, const V* __restrict__ pold) {
     static_assert(CPT == 1 || (CPT == 2 && sizeof(V) == 4), "two cells per thread: FP32 only");
     using G = TmaGeom<V, CPT>;
     using Acc = typename AccFor<V>::type;
@@ -145,13 +145,17 @@ k_cg_tma(const __grid_constant__ CgMaps maps, const Dims d, const int per_block,
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem_raw + NS * G::kStage + 4 * G::kPN * sizeof(V));
     __shared__ double sh[32];
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + kBX * ty;
-    const V beta = (V)sc->beta, alpha = (V)sc->alpha;
     Acc acc;
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) mbar_init(&bars[s], 1);
         fence_mbar_init();
     }
     __syncthreads();
+    // the scalars and vectors come from the kernels before
+    grid_dep_wait();
+    const V beta = (V)sc->beta, alpha = (V)sc->alpha;
+    double corr = 0.0;
+    bool groups_done = false;
     uint32_t phase = 0u, pending = 0u;   // per stage: parity of the next wait; load in flight
     bool bad = false;
     auto stage = [&](int s) -> unsigned char* { return smem_raw + s * G::kStage; };
@@ -231,6 +235,9 @@ k_cg_tma(const __grid_constant__ CgMaps maps, const Dims d, const int per_block,
         if (tid == 0) fence_proxy_async_smem();
         const int last_pre = min(k0 - 2 + NS, k1);
         for (int kk = k0 - 1; kk <= last_pre; ++kk) issue(kk);
+        // the groups' part of p.Ap while the first planes are in flight
+        if (!groups_done) corr = group_corr(gl, beta, r, pold, tid, kBX * kBY);
+        groups_done = true;
         const int oo = ty * TW + xo;          // own index in the Tz / x boxes
         bool ok = wait(k0 - 1);
         form_p(k0 - 1);
@@ -327,8 +334,8 @@ k_cg_tma(const __grid_constant__ CgMaps maps, const Dims d, const int per_block,
             if (pending & (1u << s)) mbar_wait_bounded(&bars[s], (phase >> s) & 1u);
         if (tid == 0) atomicCAS(&sc->status, (int)VOFP_OK, (int)VOFP_ERR_DEVICE_TIMEOUT);
     }
-    double tot;
-    if (grid_reduce(acc.value(), partials, counter, sh, &tot)) sc->pq_raw = tot;
+    if (!groups_done) corr = group_corr(gl, beta, r, pold, tid, kBX * kBY);
+    block_partial<true>(acc.value() + corr, pq_part, sh);
 }
 
 }  // namespace vofp
