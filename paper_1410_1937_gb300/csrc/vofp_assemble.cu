@@ -15,27 +15,140 @@ namespace {
 constexpr int kNT = 256;
 
 
-// rho = rho_g + (rho_l - rho_g) F   (Eq. density with H(phi) = phi)
-__global__ void k_density(Dims d, const double* __restrict__ F, double rl, double rg,
-                          double* __restrict__ rho) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < d.n;
-         c += (long long)gridDim.x * blockDim.x)
-        rho[c] = rg + (rl - rg) * F[c];
+// How the passes below are laid out. FP64 arithmetic bounds them on this part: one FP64 instruction per cell of
+// 512 x 256 x 128 takes 32 us, as long as moving 13 bytes per cell. So a thread takes one (x, y) column over a
+// range of planes (what belongs to a face between two planes is formed once, and row and column indices are
+// formed once), values are compared as integers, an open aperture's factor 1.0 is not multiplied by, and what
+// a density of pure liquid or pure gas gives is looked up. Every value that is formed is formed by the same
+// operations in the same order as by the plain formula.
+struct March {
+    int kc, nch;   // planes per range, ranges
+};
+// ranges of at most 16 planes, fewer where that leaves fewer than two threads per resident one
+March march_of(const Dims& d) {
+    const long long per = d.n / ((long long)num_sms() * 4096);
+    March m;
+    m.kc = (int)std::max(1LL, std::min(16LL, per));
+    m.nch = ceil_div(d.nz, m.kc);
+    return m;
+}
+struct Column {
+    int i, j, k0, k1;
+    long long c;    // first cell
+    bool on;
+};
+__device__ __forceinline__ Column column_of(const Dims& d, const March m) {
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    Column q;
+    q.on = t < d.plane * m.nch;
+    const unsigned int tt = q.on ? (unsigned int)t : 0u, plane = (unsigned int)d.plane, nx = (unsigned int)d.nx;
+    const unsigned int ch = tt / plane, p = tt - ch * plane;
+    q.j = int(p / nx);
+    q.i = int(p - (unsigned int)q.j * nx);
+    q.k0 = (int)ch * m.kc;
+    q.k1 = q.on ? min(q.k0 + m.kc, d.nz) : q.k0;
+    q.c = p + (long long)q.k0 * d.plane;
+    return q;
+}
+__device__ __forceinline__ long long bits_of(double a) { return __double_as_longlong(a); }
+// a > 0.0 (false for NaN)
+__device__ __forceinline__ bool positive(double a) {
+    return (unsigned long long)(bits_of(a) - 1) < 0x7ff0000000000000ull;
+}
+// Whether it holds for every thread of the warp that is here.  The passes branch on this around whole blocks:
+// around one operation the compiler forms a predicated one, which takes its time on the FP64 pipe all the same.
+__device__ __forceinline__ bool whole_warp(bool a) { return __all_sync(__activemask(), a); }
+__device__ __forceinline__ bool is_one(double a) { return bits_of(a) == 0x3ff0000000000000ll; }
+
+__device__ __forceinline__ double density(double F, double rl, double rg) { return rg + (rl - rg) * F; }
+__device__ __forceinline__ double smooth3(double lo, double in, double hi) { return 0.25 * lo + 0.5 * in + 0.25 * hi; }
+// inverse resistance of the face between two cells; the x faces of odd cells in rows of even length take their
+// neighbours the other way round, which decides the last bit of some (operators have always been built so)
+__device__ __forceinline__ double face_inv(double h0, double r0, double h1, double r1) {
+    return 1.0 / (0.5 * __fma_rn(h0, r0, __dmul_rn(h1, r1)));
+}
+__device__ __forceinline__ double face_inv_x(const Dims& d, int i, const double* __restrict__ dx, double r0, double r1) {
+    return (i & 1) && !(d.nx & 1) ? face_inv(dx[i + 1], r1, dx[i], r0) : face_inv(dx[i], r0, dx[i + 1], r1);
 }
 
-// one pass of the (1/4, 1/2, 1/4) filter along `axis` (0 = x, 1 = y, 2 = z); a missing
-// neighbour at a domain wall is replaced by the cell itself (Sec. 2.10)
-__global__ void k_smooth(Dims d, int axis, const double* __restrict__ in, double* __restrict__ out) {
+// Tables of one operator: the density of F = 0 and F = 1 before and after each smoothing pass (pure[phase][pass],
+// 2 x 4), and 1 / ((d_L rho + d_R rho) / 2) of every face between two cells of that final density along each
+// axis ([phase][axis cell], from tab + 8).
+__global__ void k_tables(Dims d, double rl, double rg, int smoothing, const double* __restrict__ dx,
+                         const double* __restrict__ dy, const double* __restrict__ dz, double* __restrict__ tab) {
+    const int len = d.nx + d.ny + d.nz;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < 2 * len; t += gridDim.x * blockDim.x) {
+        const int ph = t >= len, at = t - ph * len;
+        double r[4];
+        r[0] = density(ph ? 1.0 : 0.0, rl, rg);
+        for (int q = 1; q < 4; ++q) r[q] = smoothing ? smooth3(r[q - 1], r[q - 1], r[q - 1]) : r[q - 1];
+        if (at == 0)
+            for (int q = 0; q < 4; ++q) tab[4 * ph + q] = r[q];
+        const double* h = at < d.nx ? dx : at < d.nx + d.ny ? dy : dz;
+        const int o = at < d.nx ? at : at < d.nx + d.ny ? at - d.nx : at - d.nx - d.ny;
+        const int n = at < d.nx ? d.nx : at < d.nx + d.ny ? d.ny : d.nz;
+        tab[8 + t] = o == n - 1 ? 0.0 : at < d.nx ? face_inv_x(d, o, dx, r[3], r[3]) : face_inv(h[o], r[3], h[o + 1], r[3]);
+    }
+}
+
+// rho = rho_g + (rho_l - rho_g) F   (Eq. density with H(phi) = phi)
+__device__ __forceinline__ bool is_pure(double F) { return bits_of(F) == 0 || is_one(F); }
+__device__ __forceinline__ double density_of(double F, double rl, double rg, double r0, double r1) {
+    const double r = is_one(F) ? r1 : r0;
+    return whole_warp(is_pure(F)) ? r : density(F, rl, rg);
+}
+__global__ void k_density(Dims d, const double* __restrict__ F, double rl, double rg, const double* __restrict__ tab,
+                          double* __restrict__ rho) {
+    const double r0 = tab[0], r1 = tab[4];
+    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < d.n;
+         c += (long long)gridDim.x * blockDim.x)
+        rho[c] = density_of(F[c], rl, rg, r0, r1);
+}
+
+// The (1/4, 1/2, 1/4) filter (Sec. 2.10); a missing neighbour at a domain wall is replaced by the cell itself.
+// `pure`: the densities of the pure phases before this pass (stride 4) and after it (one further).
+__device__ __forceinline__ double smooth_of(double lo, double in, double hi, const double* p) {
+    const long long b = bits_of(in);
+    if (bits_of(lo) == b && bits_of(hi) == b) {
+        if (b == bits_of(p[0])) return p[1];
+        if (b == bits_of(p[4])) return p[5];
+    }
+    return smooth3(lo, in, hi);
+}
+// Density and its x pass, then the y and z passes: two sweeps over memory for what four kernels and a copy did
+// (512 x 256 x 128: 390 us -> 127).
+__global__ void k_density_x(Dims d, const double* __restrict__ F, double rl, double rg, const double* __restrict__ tab,
+                            double* __restrict__ out) {
+    const double p0 = tab[1], p1 = tab[5];
+    const unsigned int nx = (unsigned int)d.nx;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < d.n;
          c += (long long)gridDim.x * blockDim.x) {
-        int i, j, k;
-        cell_ijk(d, c, i, j, k);
-        long long st = axis == 0 ? 1 : axis == 1 ? d.nx : d.plane;
-        int pos = axis == 0 ? i : axis == 1 ? j : k;
-        int len = axis == 0 ? d.nx : axis == 1 ? d.ny : d.nz;
-        double lo = pos > 0 ? in[c - st] : in[c];
-        double hi = pos < len - 1 ? in[c + st] : in[c];
-        out[c] = 0.25 * lo + 0.5 * in[c] + 0.25 * hi;
+        const int i = int((unsigned int)c % nx);
+        const double f = F[c], fl = i > 0 ? F[c - 1] : f, fh = i < d.nx - 1 ? F[c + 1] : f;
+        // one pure phase in all three cells, in every thread of the warp
+        if (whole_warp(is_pure(f) && bits_of(fl) == bits_of(f) && bits_of(fh) == bits_of(f))) {
+            out[c] = is_one(f) ? p1 : p0;
+        } else {
+            out[c] = smooth3(density(fl, rl, rg), density(f, rl, rg), density(fh, rl, rg));
+        }
+    }
+}
+__global__ void k_smooth_yz(Dims d, March m, const double* __restrict__ in, const double* __restrict__ tab,
+                            double* __restrict__ out) {
+    const Column q = column_of(d, m);
+    if (!q.on) return;
+    const double py[6] = {tab[1], tab[2], 0.0, 0.0, tab[5], tab[6]}, pz[6] = {tab[2], tab[3], 0.0, 0.0, tab[6], tab[7]};
+    auto row = [&](long long c) {
+        const double v = in[c];
+        return smooth_of(q.j > 0 ? in[c - d.nx] : v, v, q.j < d.ny - 1 ? in[c + d.nx] : v, py);
+    };
+    long long c = q.c;
+    double cur = row(c), lo = q.k0 > 0 ? row(c - d.plane) : cur;
+    for (int k = q.k0; k < q.k1; ++k, c += d.plane) {
+        const double hi = k < d.nz - 1 ? row(c + d.plane) : cur;
+        out[c] = smooth_of(lo, cur, hi, pz);
+        lo = cur;
+        cur = hi;
     }
 }
 
@@ -75,76 +188,157 @@ __global__ void k_activity_step(Dims d, Bc6 bc, const double* __restrict__ ax,
     }
 }
 
-// effective apertures: faces touching a cell without an unknown are closed
-__global__ void k_eff_apertures(Dims d, const double* __restrict__ ax, const double* __restrict__ ay,
-                                const double* __restrict__ az, const uint8_t* __restrict__ ina,
-                                double* __restrict__ axe, double* __restrict__ aye,
-                                double* __restrict__ aze) {
-    const long long nfx = (long long)(d.nx + 1) * d.ny * d.nz;
-    const long long nfy = (long long)d.nx * (d.ny + 1) * d.nz;
-    const long long nfz = (long long)d.nx * d.ny * (d.nz + 1);
-    for (long long f = blockIdx.x * (long long)blockDim.x + threadIdx.x; f < nfx + nfy + nfz;
-         f += (long long)gridDim.x * blockDim.x) {
-        if (f < nfx) {
-            int i = int(f % (d.nx + 1));
-            long long t = f / (d.nx + 1);
-            long long c = i + d.nx * t;   // cell to the right of face i (row t)
-            bool okl = i == 0 || !ina[c - 1];
-            bool okr = i == d.nx || !ina[c];
-            axe[f] = (okl && okr) ? ax[f] : 0.0;
-        } else if (f < nfx + nfy) {
-            long long g = f - nfx;
-            int i = int(g % d.nx);
-            long long t = g / d.nx;
-            int j = int(t % (d.ny + 1));
-            int k = int(t / (d.ny + 1));
-            long long c = i + d.nx * (j + (long long)d.ny * k);
-            bool okl = j == 0 || !ina[c - d.nx];
-            bool okr = j == d.ny || !ina[c];
-            aye[g] = (okl && okr) ? ay[g] : 0.0;
+// One pass over the cells: whether each has an unknown (from its open volume, or from `ina_in` where that has
+// been settled before), the first step of the activity iteration (k_activity_step: `cnt[0]` counts the cells
+// that it would take out; if there are any, the caller settles the activity and runs the pass again), the
+// effective apertures (faces touching a cell without an unknown are closed), the roots, the number of cells
+// without an unknown (cnt[2]) and the list of the small cells.  Those are cells with an unknown and open volume
+// below the threshold; their merge target is the neighbour across the interior face of largest open area
+// (first of -x,+x,-y,+y,-z,+z on ties).  The list's slots come in arrival order (the order is not significant);
+// cnt[1] counts them, and the caller grows the lists and runs again if they overflow.
+// Seven passes of 700 us together before, 300 here (512 x 256 x 128: 1.0 GB, 150 us at copy bandwidth).
+template <int FROM>   // activity from the open volume (0), from `ina_in` (1), every cell active (2)
+__global__ void __launch_bounds__(kNT, 6)
+k_cells(Dims d, March m, Bc6 bc, double thr, const double* __restrict__ vf,
+                        const uint8_t* __restrict__ ina_in, const double* __restrict__ ax,
+                        const double* __restrict__ ay, const double* __restrict__ az, const double* __restrict__ dx,
+                        const double* __restrict__ dy, const double* __restrict__ dz, uint8_t* __restrict__ ina,
+                        int32_t* __restrict__ root, double* __restrict__ axe, double* __restrict__ aye,
+                        double* __restrict__ aze, unsigned int* __restrict__ cnt, long long cap,
+                        long long* __restrict__ cells, long long* __restrict__ targets, double* __restrict__ vfs) {
+    const Column q = column_of(d, m);
+    const int i = q.i, j = q.j;
+    auto active = [&](long long c) { return FROM == 0 ? positive(vf[c]) : FROM == 1 ? !ina_in[c] : true; };
+    const long long tb = positive(thr) ? bits_of(thr) : 0;
+    const bool xl = i == 0, xr = i == d.nx - 1, yl = j == 0, yr = j == d.ny - 1;
+    long long c = q.c;
+    bool am = true, ac = true;
+    double zlo = 0.0;
+    if (q.on) {
+        am = q.k0 == 0 || active(c - d.plane);
+        ac = active(c);
+        zlo = az[c];
+    }
+    unsigned int lost = 0, none = 0;
+    long long fx = fx_idx(d, i, j, q.k0), fy = fy_idx(d, i, j, q.k0);
+    const long long fxs = (long long)(d.nx + 1) * d.ny, fys = (long long)d.nx * (d.ny + 1);
+    for (int k = q.k0; k < q.k1; ++k, c += d.plane, fx += fxs, fy += fys) {
+        const bool zl = k == 0, zr = k == d.nz - 1;
+        const bool axm = xl || active(c - 1), axp = xr || active(c + 1);
+        const bool aym = yl || active(c - d.nx), ayp = yr || active(c + d.nx), azp = zr || active(c + d.plane);
+        const double x0 = ax[fx], x1 = ax[fx + 1], y0 = ay[fy], y1 = ay[fy + d.nx], z0 = zlo, z1 = az[c + d.plane];
+        ina[c] = ac ? 0 : 1;
+        root[c] = ac ? (int32_t)c : -1;
+        axe[fx] = ac && axm ? x0 : 0.0;
+        if (xr) axe[fx + 1] = ac ? x1 : 0.0;
+        aye[fy] = ac && aym ? y0 : 0.0;
+        if (yr) aye[fy + d.nx] = ac ? y1 : 0.0;
+        aze[c] = ac && am ? z0 : 0.0;
+        if (zr) aze[c + d.plane] = ac ? z1 : 0.0;
+        if (ac) {
+            bool open = false;
+            open |= positive(x0) && (xl ? bc.k[0] == VOFP_BC_DIRICHLET : axm);
+            open |= positive(x1) && (xr ? bc.k[1] == VOFP_BC_DIRICHLET : axp);
+            open |= positive(y0) && (yl ? bc.k[2] == VOFP_BC_DIRICHLET : aym);
+            open |= positive(y1) && (yr ? bc.k[3] == VOFP_BC_DIRICHLET : ayp);
+            open |= positive(z0) && (zl ? bc.k[4] == VOFP_BC_DIRICHLET : am);
+            open |= positive(z1) && (zr ? bc.k[5] == VOFP_BC_DIRICHLET : azp);
+            lost += open ? 0u : 1u;
+            if (tb > 0 && bits_of(vf[c]) < tb) {   // both positive
+                double a[6];
+                a[0] = !xl && axm ? x0 * (dz[k] * dy[j]) : 0.0;
+                a[1] = !xr && axp ? x1 * (dz[k] * dy[j]) : 0.0;
+                a[2] = !yl && aym ? y0 * (dz[k] * dx[i]) : 0.0;
+                a[3] = !yr && ayp ? y1 * (dz[k] * dx[i]) : 0.0;
+                a[4] = !zl && am ? z0 * (dy[j] * dx[i]) : 0.0;
+                a[5] = !zr && azp ? z1 * (dy[j] * dx[i]) : 0.0;
+                int best = 0;
+                for (int f = 1; f < 6; ++f)
+                    if (a[f] > a[best]) best = f;
+                if (a[best] > 0.0) {
+                    const long long off[6] = {-1, 1, -(long long)d.nx, (long long)d.nx, -d.plane, d.plane};
+                    const unsigned int slot = atomicAdd(&cnt[1], 1u);
+                    if ((long long)slot < cap) {
+                        cells[slot] = c;
+                        targets[slot] = c + off[best];
+                        vfs[slot] = vf[c];
+                    }
+                }
+            }
         } else {
-            long long g = f - nfx - nfy;
-            long long plane = d.plane;
-            int k = int(g / plane);
-            long long c = g;   // cell above face k has the same in-plane index at layer k
-            bool okl = k == 0 || !ina[c - plane];
-            bool okr = k == d.nz || !ina[c];
-            aze[g] = (okl && okr) ? az[g] : 0.0;
+            ++none;
         }
+        am = ac;
+        ac = azp;
+        zlo = z1;
+    }
+    __syncwarp();
+    lost = __reduce_add_sync(0xffffffffu, lost);
+    none = __reduce_add_sync(0xffffffffu, none);
+    if ((threadIdx.x & 31) == 0) {
+        if (lost) atomicAdd(&cnt[0], lost);
+        if (none) atomicAdd(&cnt[2], none);
     }
 }
 
-// T of each cell's +x, +y, +z face: A_f S_f / ((d_L rho_L + d_R rho_R) / 2); 0 on domain faces
-// T of each cell's +x, +y, +z interior face, and the face's inverse resistance
-// kappa = 1 / ((d_L rho_L + d_R rho_R) / 2) where the face is open (0 where it is closed or on the
-// domain boundary), which the projection of the face velocities uses
-__global__ void k_face_coeffs(Dims d, const double* __restrict__ dx, const double* __restrict__ dy,
+// T of each cell's +x, +y, +z interior face: A_f S_f / ((d_L rho_L + d_R rho_R) / 2), 0 on domain faces, and the
+// face's inverse resistance kappa = 1 / ((d_L rho_L + d_R rho_R) / 2) where the face is open (0 where it is
+// closed or on the domain boundary), which the projection of the face velocities uses.
+// 512 x 256 x 128: 1075 us with three divisions in every cell, 330 with the pure phases' looked up (1.3 GB,
+// 200 us at copy bandwidth).
+__global__ void __launch_bounds__(kNT, 5)
+k_face_coeffs(Dims d, March m, const double* __restrict__ dx, const double* __restrict__ dy,
                               const double* __restrict__ dz, const double* __restrict__ rho,
                               const double* __restrict__ axe, const double* __restrict__ aye,
-                              const double* __restrict__ aze, double* __restrict__ Tx,
+                              const double* __restrict__ aze, const double* __restrict__ tab, double* __restrict__ Tx,
                               double* __restrict__ Ty, double* __restrict__ Tz, double* __restrict__ kx,
                               double* __restrict__ ky, double* __restrict__ kz) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < d.n;
-         c += (long long)gridDim.x * blockDim.x) {
-        int i, j, k;
-        cell_ijk(d, c, i, j, k);
-        const double rc = rho[c];
+    const Column q = column_of(d, m);
+    if (!q.on) return;
+    const int i = q.i, j = q.j;
+    const long long p0 = bits_of(tab[3]), p1 = bits_of(tab[7]);
+    const int len = d.nx + d.ny + d.nz;
+    const double* ti = tab + 8;
+    const double Sz = dy[j] * dx[i];
+    long long c = q.c;
+    double rc = rho[c];
+    const bool fx = i < d.nx - 1, fy = j < d.ny - 1;
+    long long ox = fx_idx(d, i + 1, j, q.k0), oy = fy_idx(d, i, j + 1, q.k0);
+    const long long oxs = (long long)(d.nx + 1) * d.ny, oys = (long long)d.nx * (d.ny + 1);
+    for (int k = q.k0; k < q.k1; ++k, c += d.plane, ox += oxs, oy += oys) {
+        const bool fz = k < d.nz - 1;
+        const double rx = fx ? rho[c + 1] : 0.0, ry = fy ? rho[c + d.nx] : 0.0, rz = fz ? rho[c + d.plane] : 0.0;
+        const double axv = fx ? axe[ox] : 0.0, ayv = fy ? aye[oy] : 0.0,
+                     azv = fz ? aze[c + d.plane] : 0.0;
+        const long long rb = bits_of(rc);
+        const int ph = rb == p0 ? 0 : rb == p1 ? len : -1;   // offset of the phase's tables
         double tx = 0.0, ty = 0.0, tz = 0.0, qx = 0.0, qy = 0.0, qz = 0.0;
-        // one FP64 division per face (the FP64 pipe bounds this kernel): T = (A S) (1 / den)
-        if (i < d.nx - 1) {
-            const double a = axe[fx_idx(d, i + 1, j, k)], inv = 1.0 / (0.5 * (dx[i] * rc + dx[i + 1] * rho[c + 1]));
-            tx = (a * (dz[k] * dy[j])) * inv;
-            qx = a > 0.0 ? inv : 0.0;
-        }
-        if (j < d.ny - 1) {
-            const double a = aye[fy_idx(d, i, j + 1, k)], inv = 1.0 / (0.5 * (dy[j] * rc + dy[j + 1] * rho[c + d.nx]));
-            ty = (a * (dz[k] * dx[i])) * inv;
-            qy = a > 0.0 ? inv : 0.0;
-        }
-        if (k < d.nz - 1) {
-            const double a = aze[fz_idx(d, i, j, k + 1)], inv = 1.0 / (0.5 * (dz[k] * rc + dz[k + 1] * rho[c + d.plane]));
-            tz = (a * (dy[j] * dx[i])) * inv;
-            qz = a > 0.0 ? inv : 0.0;
+        const double dzk = dz[k];
+        // one pure phase across all three faces, open entirely (or on the domain boundary)
+        if (whole_warp(ph >= 0 && (!fx || (bits_of(rx) == rb && is_one(axv))) && (!fy || (bits_of(ry) == rb && is_one(ayv))) &&
+                       (!fz || (bits_of(rz) == rb && is_one(azv))))) {
+            qx = fx ? ti[ph + i] : 0.0;
+            qy = fy ? ti[ph + d.nx + j] : 0.0;
+            qz = fz ? ti[ph + d.nx + d.ny + k] : 0.0;
+            tx = (dzk * dy[j]) * qx;
+            ty = (dzk * dx[i]) * qy;
+            tz = Sz * qz;
+        } else {
+            if (fx) {
+                const double inv = face_inv_x(d, i, dx, rc, rx);
+                tx = (axv * (dzk * dy[j])) * inv;
+                qx = positive(axv) ? inv : 0.0;
+            }
+            if (fy) {
+                const double inv = face_inv(dy[j], rc, dy[j + 1], ry);
+                ty = (ayv * (dzk * dx[i])) * inv;
+                qy = positive(ayv) ? inv : 0.0;
+            }
+            if (fz) {
+                const double inv = face_inv(dzk, rc, dz[k + 1], rz);
+                tz = (azv * Sz) * inv;
+                qz = positive(azv) ? inv : 0.0;
+            }
         }
         Tx[c] = tx;
         Ty[c] = ty;
@@ -152,175 +346,88 @@ __global__ void k_face_coeffs(Dims d, const double* __restrict__ dx, const doubl
         kx[c] = qx;
         ky[c] = qy;
         kz[c] = qz;
+        rc = rz;
     }
 }
 
-// The same two kernels on x-pairs of cells (nx even): a thread takes cells c and c + 1 of one row
-// (c even, so every cell-indexed and y/z-face stream is 16-byte aligned) and moves the
-// structure-of-arrays streams as double2 words; the x-face apertures (rows of nx + 1) stay
-// scalar.  Each cell's arithmetic is that of the scalar kernels, operation for operation.
-__device__ __forceinline__ double2 ld2(const double* __restrict__ p, long long c) {
-    return *reinterpret_cast<const double2*>(p + c);
-}
-__device__ __forceinline__ void st2(double* __restrict__ p, long long c, double a, double b) {
-    *reinterpret_cast<double2*>(p + c) = make_double2(a, b);
-}
-__global__ void k_face_coeffs2(Dims d, const double* __restrict__ dx, const double* __restrict__ dy,
-                               const double* __restrict__ dz, const double* __restrict__ rho,
-                               const double* __restrict__ axe, const double* __restrict__ aye,
-                               const double* __restrict__ aze, double* __restrict__ Tx,
-                               double* __restrict__ Ty, double* __restrict__ Tz, double* __restrict__ kx,
-                               double* __restrict__ ky, double* __restrict__ kz) {
-    const long long npairs = d.n / 2;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < npairs;
-         q += (long long)gridDim.x * blockDim.x) {
-        const long long c = 2 * q;
-        int i, j, k;
-        cell_ijk(d, c, i, j, k);
-        const double2 r2 = ld2(rho, c);
-        const double rc[2] = {r2.x, r2.y};
-        double tx[2] = {0.0, 0.0}, ty[2] = {0.0, 0.0}, tz[2] = {0.0, 0.0};
-        double qx[2] = {0.0, 0.0}, qy[2] = {0.0, 0.0}, qz[2] = {0.0, 0.0};
-        // +x faces: cell c's is interior (i + 1 < nx), cell c + 1's when i + 2 < nx
-        {
-            const double a0 = axe[fx_idx(d, i + 1, j, k)];
-            const double inv0 = 1.0 / (0.5 * (dx[i] * rc[0] + dx[i + 1] * rc[1]));
-            tx[0] = (a0 * (dz[k] * dy[j])) * inv0;
-            qx[0] = a0 > 0.0 ? inv0 : 0.0;
-            if (i + 1 < d.nx - 1) {
-                const double a1 = axe[fx_idx(d, i + 2, j, k)];
-                const double inv1 = 1.0 / (0.5 * (dx[i + 1] * rc[1] + dx[i + 2] * rho[c + 2]));
-                tx[1] = (a1 * (dz[k] * dy[j])) * inv1;
-                qx[1] = a1 > 0.0 ? inv1 : 0.0;
-            }
-        }
-        if (j < d.ny - 1) {
-            const double2 a = ld2(aye, fy_idx(d, i, j + 1, k)), rn = ld2(rho, c + d.nx);
-            const double av[2] = {a.x, a.y}, rv[2] = {rn.x, rn.y};
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const double inv = 1.0 / (0.5 * (dy[j] * rc[e] + dy[j + 1] * rv[e]));
-                ty[e] = (av[e] * (dz[k] * dx[i + e])) * inv;
-                qy[e] = av[e] > 0.0 ? inv : 0.0;
-            }
-        }
-        if (k < d.nz - 1) {
-            const double2 a = ld2(aze, fz_idx(d, i, j, k + 1)), rn = ld2(rho, c + d.plane);
-            const double av[2] = {a.x, a.y}, rv[2] = {rn.x, rn.y};
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const double inv = 1.0 / (0.5 * (dz[k] * rc[e] + dz[k + 1] * rv[e]));
-                tz[e] = (av[e] * (dy[j] * dx[i + e])) * inv;
-                qz[e] = av[e] > 0.0 ? inv : 0.0;
-            }
-        }
-        st2(Tx, c, tx[0], tx[1]);
-        st2(Ty, c, ty[0], ty[1]);
-        st2(Tz, c, tz[0], tz[1]);
-        st2(kx, c, qx[0], qx[1]);
-        st2(ky, c, qy[0], qy[1]);
-        st2(kz, c, qz[0], qz[1]);
+// r = sqrt(d) and 1 / r.  An approximation y of d^-1/2 to 45 bits comes from FP32 arithmetic (a step of third
+// order from rsqrtf, its residual 1 - d y^2 formed without cancellation by fused products, in the manner of
+// Dekker's double-length arithmetic), then one FP64 Newton step each for the root and for its reciprocal:
+// r = g + (d - g g) y / 2 with g = d y, and 1 / r = y + (1 - r y) y.  Both are within 2^-37 of a half unit in the
+// last place, so correctly rounded but for one value in some 2^36.  Five FP64 instructions instead of the
+// twelve of sqrt and the division.  Values that are not normal numbers of moderate size take those.
+__device__ __forceinline__ void sqrt_and_inverse(double d, double& r, double& inv) {
+    const unsigned long long b = (unsigned long long)bits_of(d);
+    const unsigned int e = (unsigned int)(b >> 52);   // sign and exponent
+    if (e - 200u >= 1600u) {
+        r = sqrt(d);
+        inv = 1.0 / r;
+        return;
     }
+    // d = 4^h m, m in [1, 4): m = mh + ml with mh its leading 24 bits
+    const unsigned int odd = (e + 1u) & 1u;                  // e = 1023: even power
+    const int h = ((int)e - 1023 - (int)odd) / 2;            // exact: e - 1023 - odd is even
+    const float mh = __uint_as_float(((127u + odd) << 23) | (unsigned int)((b >> 29) & 0x7fffffu));
+    const float ml = (float)(int)(b & 0x1fffffffu) * __uint_as_float((127u - 52u + odd) << 23);
+    const float y = fminf(fmaxf(rsqrtf(mh), 0.5f), 1.0f);
+    const float p = __fmul_rn(y, y), pe = __fmaf_rn(y, y, -p);
+    const float t = __fmul_rn(mh, p), te = __fmaf_rn(mh, p, -t);
+    const float res = __fsub_rn(__fsub_rn(1.0f, t), __fmaf_rn(ml, p, __fmaf_rn(mh, pe, te)));
+    const float cy = __fmul_rn(y, __fmul_rn(res, __fmaf_rn(0.375f, res, 0.5f)));
+    // y + cy in units of 2^-53 (y in [1/2, 1]; |cy| < 2^-21), scaled by 2^-h
+    const unsigned int yb = __float_as_uint(y);
+    long long yd = ((long long)(yb >> 23) - 127 + 1023 - h) << 52 | (long long)(yb & 0x7fffffu) << 29;
+    yd += __float2int_rn(cy * 9007199254740992.0f);
+    const double yy = __longlong_as_double(yd), hy = __longlong_as_double(yd - (1ll << 52));
+    const double g = __dmul_rn(d, yy);
+    r = __fma_rn(__fma_rn(-g, g, d), hy, g);
+    inv = __fma_rn(__fma_rn(-r, yy, 1.0), yy, yy);
 }
 
-__global__ void k_diag2(Dims d, Bc6 bc, const double* __restrict__ dx, const double* __restrict__ dy,
-                        const double* __restrict__ dz, const double* __restrict__ rho,
-                        const double* __restrict__ axe, const double* __restrict__ aye,
-                        const double* __restrict__ aze, const double* __restrict__ Tx,
-                        const double* __restrict__ Ty, const double* __restrict__ Tz, double* __restrict__ diag) {
-    const long long npairs = d.n / 2;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < npairs;
-         q += (long long)gridDim.x * blockDim.x) {
-        const long long c = 2 * q;
-        int i, j, k;
-        cell_ijk(d, c, i, j, k);
-        const double2 x2 = ld2(Tx, c), y2 = ld2(Ty, c), z2 = ld2(Tz, c), r2 = ld2(rho, c);
-        const double2 ym = j > 0 ? ld2(Ty, c - d.nx) : make_double2(0.0, 0.0);
-        const double2 zm = k > 0 ? ld2(Tz, c - d.plane) : make_double2(0.0, 0.0);
-        const double txs[2] = {x2.x, x2.y}, tys[2] = {y2.x, y2.y}, tzs[2] = {z2.x, z2.y}, rcs[2] = {r2.x, r2.y};
-        const double tym[2] = {ym.x, ym.y}, tzm[2] = {zm.x, zm.y};
-        const double txm[2] = {i > 0 ? Tx[c - 1] : 0.0, x2.x};
-        double out[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int ii = i + e;
-            const double rc = rcs[e];
-            double s = txs[e] + tys[e] + tzs[e];
-            if (ii > 0) s += txm[e];
-            if (j > 0) s += tym[e];
-            if (k > 0) s += tzm[e];
-            if (ii == 0 && bc.k[0] == VOFP_BC_DIRICHLET) s += (axe[fx_idx(d, 0, j, k)] * (dz[k] * dy[j])) / (0.5 * dx[0] * rc);
-            if (ii == d.nx - 1 && bc.k[1] == VOFP_BC_DIRICHLET) s += (axe[fx_idx(d, d.nx, j, k)] * (dz[k] * dy[j])) / (0.5 * dx[ii] * rc);
-            if (j == 0 && bc.k[2] == VOFP_BC_DIRICHLET) s += (aye[fy_idx(d, ii, 0, k)] * (dz[k] * dx[ii])) / (0.5 * dy[0] * rc);
-            if (j == d.ny - 1 && bc.k[3] == VOFP_BC_DIRICHLET) s += (aye[fy_idx(d, ii, d.ny, k)] * (dz[k] * dx[ii])) / (0.5 * dy[j] * rc);
-            if (k == 0 && bc.k[4] == VOFP_BC_DIRICHLET) s += (aze[fz_idx(d, ii, j, 0)] * (dy[j] * dx[ii])) / (0.5 * dz[0] * rc);
-            if (k == d.nz - 1 && bc.k[5] == VOFP_BC_DIRICHLET) s += (aze[fz_idx(d, ii, j, d.nz)] * (dy[j] * dx[ii])) / (0.5 * dz[k] * rc);
-            out[e] = s;
+// Diagonal of the unmerged operator (sum of the six face coefficients plus p = 0 faces) and the symmetric
+// scaling s = diag^-1/2, sq = diag^1/2 (0 without an unknown; the groups' follow in k_scale_groups).
+// FP64 arithmetic bounds it: 650 us as two kernels with sqrt and a division, 355 here (512 x 256 x 128).
+__global__ void __launch_bounds__(kNT, 5)
+k_diag_scale(Dims d, March m, Bc6 bc, const double* __restrict__ dx, const double* __restrict__ dy,
+                             const double* __restrict__ dz, const double* __restrict__ rho,
+                             const double* __restrict__ axe, const double* __restrict__ aye,
+                             const double* __restrict__ aze, const double* __restrict__ Tx,
+                             const double* __restrict__ Ty, const double* __restrict__ Tz,
+                             const uint8_t* __restrict__ ina, double* __restrict__ diag, double* __restrict__ s,
+                             double* __restrict__ sq) {
+    const Column q = column_of(d, m);
+    if (!q.on) return;
+    const int i = q.i, j = q.j;
+    const bool edge = (i == 0 && bc.k[0] == VOFP_BC_DIRICHLET) || (i == d.nx - 1 && bc.k[1] == VOFP_BC_DIRICHLET) ||
+                      (j == 0 && bc.k[2] == VOFP_BC_DIRICHLET) || (j == d.ny - 1 && bc.k[3] == VOFP_BC_DIRICHLET);
+    long long c = q.c;
+    double tzm = q.k0 > 0 ? Tz[c - d.plane] : 0.0;
+    double last = __longlong_as_double(-1ll), r = 0.0, inv = 0.0;   // of the plane before: r and inv of `last`
+    for (int k = q.k0; k < q.k1; ++k, c += d.plane) {
+        const double tx = Tx[c], ty = Ty[c], tz = Tz[c];
+        const double txm = i > 0 ? Tx[c - 1] : 0.0, tym = j > 0 ? Ty[c - d.nx] : 0.0;
+        const bool off = ina[c] != 0;
+        double v = tx + ty + tz;
+        if (i > 0) v += txm;
+        if (j > 0) v += tym;
+        if (k > 0) v += tzm;
+        if (edge || k == 0 || k == d.nz - 1) {
+            const double rc = rho[c];
+            if (i == 0 && bc.k[0] == VOFP_BC_DIRICHLET) v += (axe[fx_idx(d, 0, j, k)] * (dz[k] * dy[j])) / (0.5 * dx[0] * rc);
+            if (i == d.nx - 1 && bc.k[1] == VOFP_BC_DIRICHLET) v += (axe[fx_idx(d, d.nx, j, k)] * (dz[k] * dy[j])) / (0.5 * dx[i] * rc);
+            if (j == 0 && bc.k[2] == VOFP_BC_DIRICHLET) v += (aye[fy_idx(d, i, 0, k)] * (dz[k] * dx[i])) / (0.5 * dy[0] * rc);
+            if (j == d.ny - 1 && bc.k[3] == VOFP_BC_DIRICHLET) v += (aye[fy_idx(d, i, d.ny, k)] * (dz[k] * dx[i])) / (0.5 * dy[j] * rc);
+            if (k == 0 && bc.k[4] == VOFP_BC_DIRICHLET) v += (aze[fz_idx(d, i, j, 0)] * (dy[j] * dx[i])) / (0.5 * dz[0] * rc);
+            if (k == d.nz - 1 && bc.k[5] == VOFP_BC_DIRICHLET) v += (aze[fz_idx(d, i, j, d.nz)] * (dy[j] * dx[i])) / (0.5 * dz[k] * rc);
         }
-        st2(diag, c, out[0], out[1]);
-    }
-}
-
-// diagonal of the unmerged operator: sum of the six face coefficients plus p = 0 faces
-__global__ void k_diag(Dims d, Bc6 bc, const double* __restrict__ dx, const double* __restrict__ dy,
-                       const double* __restrict__ dz, const double* __restrict__ rho,
-                       const double* __restrict__ axe, const double* __restrict__ aye,
-                       const double* __restrict__ aze, const double* __restrict__ Tx,
-                       const double* __restrict__ Ty, const double* __restrict__ Tz,
-                       double* __restrict__ diag) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < d.n;
-         c += (long long)gridDim.x * blockDim.x) {
-        int i, j, k;
-        cell_ijk(d, c, i, j, k);
-        const double rc = rho[c];
-        double s = Tx[c] + Ty[c] + Tz[c];
-        if (i > 0) s += Tx[c - 1];
-        if (j > 0) s += Ty[c - d.nx];
-        if (k > 0) s += Tz[c - d.plane];
-        if (i == 0 && bc.k[0] == VOFP_BC_DIRICHLET) s += (axe[fx_idx(d, 0, j, k)] * (dz[k] * dy[j])) / (0.5 * dx[0] * rc);
-        if (i == d.nx - 1 && bc.k[1] == VOFP_BC_DIRICHLET) s += (axe[fx_idx(d, d.nx, j, k)] * (dz[k] * dy[j])) / (0.5 * dx[i] * rc);
-        if (j == 0 && bc.k[2] == VOFP_BC_DIRICHLET) s += (aye[fy_idx(d, i, 0, k)] * (dz[k] * dx[i])) / (0.5 * dy[0] * rc);
-        if (j == d.ny - 1 && bc.k[3] == VOFP_BC_DIRICHLET) s += (aye[fy_idx(d, i, d.ny, k)] * (dz[k] * dx[i])) / (0.5 * dy[j] * rc);
-        if (k == 0 && bc.k[4] == VOFP_BC_DIRICHLET) s += (aze[fz_idx(d, i, j, 0)] * (dy[j] * dx[i])) / (0.5 * dz[0] * rc);
-        if (k == d.nz - 1 && bc.k[5] == VOFP_BC_DIRICHLET) s += (aze[fz_idx(d, i, j, d.nz)] * (dy[j] * dx[i])) / (0.5 * dz[k] * rc);
-        diag[c] = s;
-    }
-}
-
-// Cells with an unknown and open volume below the threshold: their merge target is the neighbour
-// across the interior face of largest open area (first of -x,+x,-y,+y,-z,+z on ties).
-// Pass 0 counts, pass 1 writes (cell, target) pairs (order of the list is not significant).
-__global__ void k_small_cells(Dims d, double thr, const double* __restrict__ vf,
-                              const uint8_t* __restrict__ ina, const double* __restrict__ dx,
-                              const double* __restrict__ dy, const double* __restrict__ dz,
-                              const double* __restrict__ axe, const double* __restrict__ aye,
-                              const double* __restrict__ aze, unsigned int* count, long long cap,
-                              long long* __restrict__ cells, long long* __restrict__ targets,
-                              double* __restrict__ vfs) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < d.n;
-         c += (long long)gridDim.x * blockDim.x) {
-        if (ina[c] || !(vf[c] < thr)) continue;
-        int i, j, k;
-        cell_ijk(d, c, i, j, k);
-        double a[6];
-        a[0] = i > 0 ? axe[fx_idx(d, i, j, k)] * (dz[k] * dy[j]) : 0.0;
-        a[1] = i < d.nx - 1 ? axe[fx_idx(d, i + 1, j, k)] * (dz[k] * dy[j]) : 0.0;
-        a[2] = j > 0 ? aye[fy_idx(d, i, j, k)] * (dz[k] * dx[i]) : 0.0;
-        a[3] = j < d.ny - 1 ? aye[fy_idx(d, i, j + 1, k)] * (dz[k] * dx[i]) : 0.0;
-        a[4] = k > 0 ? aze[fz_idx(d, i, j, k)] * (dy[j] * dx[i]) : 0.0;
-        a[5] = k < d.nz - 1 ? aze[fz_idx(d, i, j, k + 1)] * (dy[j] * dx[i]) : 0.0;
-        int best = 0;
-        for (int f = 1; f < 6; ++f)
-            if (a[f] > a[best]) best = f;
-        if (!(a[best] > 0.0)) continue;
-        const long long off[6] = {-1, 1, -(long long)d.nx, (long long)d.nx, -d.plane, d.plane};
-        // slots in arrival order; the caller grows the lists and runs again if they overflow
-        const unsigned int slot = atomicAdd(count, 1u);
-        if ((long long)slot < cap) {
-            cells[slot] = c;
-            targets[slot] = c + off[best];
-            vfs[slot] = vf[c];
+        diag[c] = v;
+        if (!off && bits_of(v) != bits_of(last)) {
+            sqrt_and_inverse(v, r, inv);
+            last = v;
         }
+        s[c] = off ? 0.0 : inv;
+        sq[c] = off ? 0.0 : r;
+        tzm = tz;
     }
 }
 
@@ -337,40 +444,10 @@ __global__ void k_small_target_slots(int m, const long long* __restrict__ target
     if (t < m) tslot[t] = slot_of[targets[t]];
 }
 
-__global__ void k_count_u8(long long n, const uint8_t* __restrict__ a, unsigned int* count) {
-    unsigned int local = 0;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
-         c += (long long)gridDim.x * blockDim.x)
-        local += a[c] ? 1u : 0u;
-    for (int o = 16; o > 0; o >>= 1) local += __shfl_xor_sync(0xffffffffu, local, o);
-    if ((threadIdx.x & 31) == 0 && local) atomicAdd(count, local);
-}
-
-__global__ void k_root_init(Dims d, const uint8_t* __restrict__ ina, int32_t* __restrict__ root) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < d.n;
-         c += (long long)gridDim.x * blockDim.x)
-        root[c] = ina[c] ? -1 : (int32_t)c;
-}
-
 __global__ void k_root_scatter(int m, const long long* __restrict__ cells,
                                const long long* __restrict__ roots, int32_t* __restrict__ root) {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < m) root[cells[t]] = (int32_t)roots[t];
-}
-
-__global__ void k_scale_cells(Dims d, const uint8_t* __restrict__ ina, const double* __restrict__ diag,
-                              double* __restrict__ s, double* __restrict__ sq) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < d.n;
-         c += (long long)gridDim.x * blockDim.x) {
-        if (ina[c]) {
-            s[c] = 0.0;
-            sq[c] = 0.0;
-        } else {
-            double r = sqrt(diag[c]);
-            sq[c] = r;
-            s[c] = 1.0 / r;
-        }
-    }
 }
 
 // diag(A_hat) of a merge group = sum over its cells of the diagonal minus the couplings between
@@ -408,76 +485,114 @@ __global__ void k_scale_groups(Dims d, int ng, const int* __restrict__ gptr,
     gcorr[g] = sm * sm * dsum - double(e - b);
 }
 
-__global__ void k_scaled_coeffs(Dims d, const double* __restrict__ s, const double* __restrict__ Tx,
+// (float)a for a >= 0, by integer arithmetic where the result is a normal number: the conversion instruction
+// takes as long as an FP64 operation.
+__device__ __forceinline__ float to_float(double a) {
+    const unsigned long long b = (unsigned long long)bits_of(a);
+    if ((unsigned int)(b >> 52) - 897u < 252u) {
+        const unsigned long long v = b - (896ull << 52);
+        return __uint_as_float((unsigned int)((v + 0x0fffffffull + ((v >> 29) & 1ull)) >> 29));
+    }
+    if (b == 0ull) return 0.0f;
+    float f;
+    asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f) : "d"(a));   // (volatile: not ahead of the branch)
+    return f;
+}
+
+// The scaled operator in FP64 and FP32, and Tzr = Tzf with the sign bit set on red cells (coefficients are >= 0,
+// so the sign carries the red flag through the same tensor copy as the coefficient; -0.0 marks a red cell with a
+// closed face).  512 x 256 x 128: 315 us as two kernels with converting instructions, 215 here.
+__global__ void k_scaled_coeffs(Dims d, March m, const double* __restrict__ s, const double* __restrict__ Tx,
                                 const double* __restrict__ Ty, const double* __restrict__ Tz,
-                                double* __restrict__ Txs, double* __restrict__ Tys,
-                                double* __restrict__ Tzs, float* __restrict__ Txf,
-                                float* __restrict__ Tyf, float* __restrict__ Tzf) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < d.n;
-         c += (long long)gridDim.x * blockDim.x) {
-        int i, j, k;
-        cell_ijk(d, c, i, j, k);
-        const double sc = s[c];
-        double a = i < d.nx - 1 ? sc * Tx[c] * s[c + 1] : 0.0;
-        double b = j < d.ny - 1 ? sc * Ty[c] * s[c + d.nx] : 0.0;
-        double e = k < d.nz - 1 ? sc * Tz[c] * s[c + d.plane] : 0.0;
+                                const uint32_t* __restrict__ red, double* __restrict__ Txs, double* __restrict__ Tys,
+                                double* __restrict__ Tzs, float* __restrict__ Txf, float* __restrict__ Tyf,
+                                float* __restrict__ Tzf, float* __restrict__ Tzr) {
+    const Column q = column_of(d, m);
+    if (!q.on) return;
+    const bool fx = q.i < d.nx - 1, fy = q.j < d.ny - 1;
+    long long c = q.c;
+    double sc = s[c];
+    for (int k = q.k0; k < q.k1; ++k, c += d.plane) {
+        const bool fz = k < d.nz - 1;
+        const double sx = fx ? s[c + 1] : 0.0, sy = fy ? s[c + d.nx] : 0.0, sz = fz ? s[c + d.plane] : 0.0;
+        const double tx = Tx[c], ty = Ty[c], tz = Tz[c];
+        const uint32_t w = red[c >> 5] >> (c & 31);
+        const double a = fx ? sc * tx * sx : 0.0;
+        const double b = fy ? sc * ty * sy : 0.0;
+        const double e = fz ? sc * tz * sz : 0.0;
+        const float ef = to_float(e);
         Txs[c] = a;
         Tys[c] = b;
         Tzs[c] = e;
-        Txf[c] = (float)a;
-        Tyf[c] = (float)b;
-        Tzf[c] = (float)e;
+        Txf[c] = to_float(a);
+        Tyf[c] = to_float(b);
+        Tzf[c] = ef;
+        Tzr[c] = (w & 1u) ? -fabsf(ef) : ef;
+        sc = sz;
     }
 }
 
-__global__ void k_slave_bits(Dims d, const int32_t* __restrict__ root, uint32_t* __restrict__ bits) {
+// Merged cells and red cells as bits.  A red cell has (i+j+k) even, an unknown of its own and no merge group (the
+// groups' cells are taken out by k_group_flags; a count of the red cells goes with both).
+__global__ void k_cell_bits(Dims d, const uint8_t* __restrict__ ina, uint32_t* __restrict__ slave,
+                            uint32_t* __restrict__ red, unsigned int* __restrict__ count) {
     const long long nw = (d.n + 31) / 32;
+    unsigned int mine = 0;
     for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < nw;
          w += (long long)gridDim.x * blockDim.x) {
-        uint32_t v = 0;
-        for (int b = 0; b < 32; ++b) {
-            long long c = w * 32 + b;
-            if (c < d.n && root[c] >= 0 && root[c] != (int32_t)c) v |= (1u << b);
+        const long long c0 = w * 32;
+        const int n = (int)min(32LL, d.n - c0);
+        int i, j, k;
+        cell_ijk(d, c0, i, j, k);
+        uint32_t par = 0u;   // bit b: cell c0 + b has i+j+k even
+        for (int b = 0; b < n;) {
+            const int run = min(n - b, d.nx - i);   // cells left in this row
+            const uint32_t pat = ((i + j + k + b) & 1) == 0 ? 0x55555555u : 0xaaaaaaaau;
+            const uint32_t part = run == 32 ? 0xffffffffu : ((1u << run) - 1u) << b;
+            par |= pat & part;
+            b += run;
+            i = 0;
+            if (++j == d.ny) {
+                j = 0;
+                ++k;
+            }
         }
-        bits[w] = v;
-    }
-}
-
-// red cells: (i+j+k) even, own root, and not the master of a multi-cell group (a master always
-// touches one of its members, so a neighbour whose root is c marks c as a master)
-// Tzr = Tzf with the sign bit set on red cells (coefficients are >= 0, so the sign carries the red
-// flag through the same tensor copy as the coefficient; -0.0 marks a red cell with a closed face)
-__global__ void k_signed_tz(long long n, const float* __restrict__ tz, const uint32_t* __restrict__ red,
-                            float* __restrict__ tzr) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x)
-        tzr[c] = ((red[c >> 5] >> (c & 31)) & 1u) ? -fabsf(tz[c]) : tz[c];
-}
-
-__global__ void k_red_bits(Dims d, const int32_t* __restrict__ root, const uint32_t* __restrict__ slave,
-                           uint32_t* __restrict__ red, uint32_t* __restrict__ excl, unsigned int* count) {
-    const long long nw = (d.n + 31) / 32;
-    for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < nw;
-         w += (long long)gridDim.x * blockDim.x) {
-        uint32_t v = 0;
-        for (int b = 0; b < 32; ++b) {
-            const long long c = w * 32 + b;
-            if (c >= d.n || root[c] != (int32_t)c) continue;
-            int i, j, k;
-            cell_ijk(d, c, i, j, k);
-            if (((i + j + k) & 1) != 0) continue;
-            bool master = false;
-            if (i > 0) master |= root[c - 1] == (int32_t)c;
-            if (i < d.nx - 1) master |= root[c + 1] == (int32_t)c;
-            if (j > 0) master |= root[c - d.nx] == (int32_t)c;
-            if (j < d.ny - 1) master |= root[c + d.nx] == (int32_t)c;
-            if (k > 0) master |= root[c - d.plane] == (int32_t)c;
-            if (k < d.nz - 1) master |= root[c + d.plane] == (int32_t)c;
-            if (!master) v |= (1u << b);
+        uint32_t v = 0u;
+        if (n == 32) {
+            const uint4* p = reinterpret_cast<const uint4*>(ina + c0);
+            const uint4 a = p[0], b = p[1];
+            const uint32_t x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+            // bytes of 0 or 1: their low bits to four neighbouring bits
+#pragma unroll
+            for (int t = 0; t < 8; ++t) v |= (((x[t] & 0x01010101u) * 0x10204080u) >> 28) << (4 * t);
+            v = ~v;
+        } else {
+            for (int b = 0; b < n; ++b) v |= (ina[c0 + b] ? 0u : 1u) << b;
         }
+        v &= par;
+        slave[w] = 0u;
         red[w] = v;
-        excl[w] = v | slave[w];
-        if (v) atomicAdd(count, (unsigned int)__popc(v));
+        mine += __popc(v);
     }
+    __syncwarp();
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if ((threadIdx.x & 31) == 0 && mine) atomicAdd(count, mine);
+}
+__global__ void k_group_flags(int ng, const int* __restrict__ gptr, const int* __restrict__ gcells,
+                              uint32_t* __restrict__ slave, uint32_t* __restrict__ red, unsigned int* __restrict__ count) {
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= ng) return;
+    for (int t = gptr[g]; t < gptr[g + 1]; ++t) {
+        const int c = gcells[t];
+        const uint32_t bit = 1u << (c & 31);
+        if (t > gptr[g]) atomicOr(&slave[c >> 5], bit);
+        if (atomicAnd(&red[c >> 5], ~bit) & bit) atomicSub(count, 1u);
+    }
+}
+__global__ void k_excl_bits(long long nw, const uint32_t* __restrict__ slave, const uint32_t* __restrict__ red,
+                            uint32_t* __restrict__ excl) {
+    for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < nw; w += (long long)gridDim.x * blockDim.x)
+        excl[w] = slave[w] | red[w];
 }
 
 struct Flux6 {
@@ -485,45 +600,78 @@ struct Flux6 {
 };
 
 // b_c = -(1/dt) (sum of outward open-face fluxes + body flux) + prescribed Neumann fluxes
-__global__ void k_rhs(Dims d, Bc6 bc, Flux6 nf, double dt, const double* __restrict__ dx,
+// Fluxes through partly open faces.  Not inlined: the compiler would predicate the products in every cell.
+struct Flux5 {
+    double xm, xp, ym, yp, zp;
+};
+__device__ __noinline__ Flux5 cut_fluxes(double x0, double x1, double y0, double y1, double z1, double Sx, double Sy,
+                                         double Sz, double u0, double u1, double v0, double v1, double w1) {
+    Flux5 f;
+    f.xm = __dmul_rn(x0 * Sx, u0);
+    f.xp = __dmul_rn(x1 * Sx, u1);
+    f.ym = __dmul_rn(y0 * Sy, v0);
+    f.yp = __dmul_rn(y1 * Sy, v1);
+    f.zp = __dmul_rn(z1 * Sz, w1);
+    return f;
+}
+// FP64 arithmetic bounds it: 1057 us with both faces of every direction formed from three factors and a division
+// in every cell, 505 here (512 x 256 x 128; 0.94 GB, 140 us at copy bandwidth).  The division is left out where
+// dt is 1 (HOW 0) and is a multiplication by the exact reciprocal, given as dt, where it is a power of two (1).
+template <int HOW>   // -div (0), -div times dt (1), -div / dt (2)
+__global__ void __launch_bounds__(kNT, 5)
+k_rhs(Dims d, March m, Bc6 bc, Flux6 nf, double dt, const double* __restrict__ dx,
                       const double* __restrict__ dy, const double* __restrict__ dz,
                       const double* __restrict__ axe, const double* __restrict__ aye,
                       const double* __restrict__ aze, const uint8_t* __restrict__ ina,
                       const double* __restrict__ u, const double* __restrict__ v,
                       const double* __restrict__ w, const double* __restrict__ body,
                       double* __restrict__ b) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < d.n;
-         c += (long long)gridDim.x * blockDim.x) {
-        if (ina[c]) {
-            b[c] = 0.0;
-            continue;
+    const Column q = column_of(d, m);
+    if (!q.on) return;
+    const int i = q.i, j = q.j;
+    const bool wall[6] = {i == 0 && bc.k[0] != VOFP_BC_DIRICHLET, i == d.nx - 1 && bc.k[1] != VOFP_BC_DIRICHLET,
+                          j == 0 && bc.k[2] != VOFP_BC_DIRICHLET, j == d.ny - 1 && bc.k[3] != VOFP_BC_DIRICHLET,
+                          bc.k[4] != VOFP_BC_DIRICHLET, bc.k[5] != VOFP_BC_DIRICHLET};
+    const bool edge = (i == 0 && nf.g[0]) || (i == d.nx - 1 && nf.g[1]) || (j == 0 && nf.g[2]) || (j == d.ny - 1 && nf.g[3]);
+    const double Sz = dy[j] * dx[i];
+    long long c = q.c;
+    double fzm = q.k0 == 0 && wall[4] ? 0.0 : aze[c] * Sz * w[c];
+    long long fx = fx_idx(d, i, j, q.k0), fy = fy_idx(d, i, j, q.k0);
+    const long long fxs = (long long)(d.nx + 1) * d.ny, fys = (long long)d.nx * (d.ny + 1);
+    for (int k = q.k0; k < q.k1; ++k, c += d.plane, fx += fxs, fy += fys) {
+        const long long fz = c + d.plane;
+        const double x0 = axe[fx], x1 = axe[fx + 1], y0 = aye[fy], y1 = aye[fy + d.nx], z1 = aze[fz];
+        const double u0 = u[fx], u1 = u[fx + 1], v0 = v[fy], v1 = v[fy + d.nx], w1 = w[fz];
+        const bool off = ina[c] != 0;
+        const double Sx = dz[k] * dy[j], Sy = dz[k] * dx[i];
+        Flux5 f;
+        if (whole_warp(is_one(x0) && is_one(x1) && is_one(y0) && is_one(y1) && is_one(z1))) {
+            f.xm = __dmul_rn(Sx, u0);
+            f.xp = __dmul_rn(Sx, u1);
+            f.ym = __dmul_rn(Sy, v0);
+            f.yp = __dmul_rn(Sy, v1);
+            f.zp = __dmul_rn(Sz, w1);
+        } else {
+            f = cut_fluxes(x0, x1, y0, y1, z1, Sx, Sy, Sz, u0, u1, v0, v1, w1);
         }
-        int i, j, k;
-        cell_ijk(d, c, i, j, k);
-        const double Sx = dz[k] * dy[j], Sy = dz[k] * dx[i], Sz = dy[j] * dx[i];
-        long long f;
-        f = fx_idx(d, i, j, k);
-        double fxm = (i == 0 && bc.k[0] != VOFP_BC_DIRICHLET) ? 0.0 : axe[f] * Sx * u[f];
-        f = fx_idx(d, i + 1, j, k);
-        double fxp = (i == d.nx - 1 && bc.k[1] != VOFP_BC_DIRICHLET) ? 0.0 : axe[f] * Sx * u[f];
-        f = fy_idx(d, i, j, k);
-        double fym = (j == 0 && bc.k[2] != VOFP_BC_DIRICHLET) ? 0.0 : aye[f] * Sy * v[f];
-        f = fy_idx(d, i, j + 1, k);
-        double fyp = (j == d.ny - 1 && bc.k[3] != VOFP_BC_DIRICHLET) ? 0.0 : aye[f] * Sy * v[f];
-        f = fz_idx(d, i, j, k);
-        double fzm = (k == 0 && bc.k[4] != VOFP_BC_DIRICHLET) ? 0.0 : aze[f] * Sz * w[f];
-        f = fz_idx(d, i, j, k + 1);
-        double fzp = (k == d.nz - 1 && bc.k[5] != VOFP_BC_DIRICHLET) ? 0.0 : aze[f] * Sz * w[f];
-        double div = ((fxp - fxm) + (fyp - fym)) + (fzp - fzm);
+        if (wall[0]) f.xm = 0.0;
+        if (wall[1]) f.xp = 0.0;
+        if (wall[2]) f.ym = 0.0;
+        if (wall[3]) f.yp = 0.0;
+        if (k == d.nz - 1 && wall[5]) f.zp = 0.0;
+        double div = __dadd_rn(__dadd_rn(__dsub_rn(f.xp, f.xm), __dsub_rn(f.yp, f.ym)), __dsub_rn(f.zp, fzm));
         if (body) div += body[c];
-        double bb = -div / dt;
-        if (i == 0 && bc.k[0] == VOFP_BC_NEUMANN && nf.g[0]) bb += axe[fx_idx(d, 0, j, k)] * Sx * nf.g[0][j + (long long)d.ny * k];
-        if (i == d.nx - 1 && bc.k[1] == VOFP_BC_NEUMANN && nf.g[1]) bb += axe[fx_idx(d, d.nx, j, k)] * Sx * nf.g[1][j + (long long)d.ny * k];
-        if (j == 0 && bc.k[2] == VOFP_BC_NEUMANN && nf.g[2]) bb += aye[fy_idx(d, i, 0, k)] * Sy * nf.g[2][i + (long long)d.nx * k];
-        if (j == d.ny - 1 && bc.k[3] == VOFP_BC_NEUMANN && nf.g[3]) bb += aye[fy_idx(d, i, d.ny, k)] * Sy * nf.g[3][i + (long long)d.nx * k];
-        if (k == 0 && bc.k[4] == VOFP_BC_NEUMANN && nf.g[4]) bb += aze[fz_idx(d, i, j, 0)] * Sz * nf.g[4][i + (long long)d.nx * j];
-        if (k == d.nz - 1 && bc.k[5] == VOFP_BC_NEUMANN && nf.g[5]) bb += aze[fz_idx(d, i, j, d.nz)] * Sz * nf.g[5][i + (long long)d.nx * j];
-        b[c] = bb;
+        double bb = HOW == 0 ? -div : HOW == 1 ? -div * dt : -div / dt;
+        if (edge || (k == 0 && nf.g[4]) || (k == d.nz - 1 && nf.g[5])) {
+            if (i == 0 && bc.k[0] == VOFP_BC_NEUMANN && nf.g[0]) bb += axe[fx_idx(d, 0, j, k)] * Sx * nf.g[0][j + (long long)d.ny * k];
+            if (i == d.nx - 1 && bc.k[1] == VOFP_BC_NEUMANN && nf.g[1]) bb += axe[fx_idx(d, d.nx, j, k)] * Sx * nf.g[1][j + (long long)d.ny * k];
+            if (j == 0 && bc.k[2] == VOFP_BC_NEUMANN && nf.g[2]) bb += aye[fy_idx(d, i, 0, k)] * Sy * nf.g[2][i + (long long)d.nx * k];
+            if (j == d.ny - 1 && bc.k[3] == VOFP_BC_NEUMANN && nf.g[3]) bb += aye[fy_idx(d, i, d.ny, k)] * Sy * nf.g[3][i + (long long)d.nx * k];
+            if (k == 0 && bc.k[4] == VOFP_BC_NEUMANN && nf.g[4]) bb += aze[fz_idx(d, i, j, 0)] * Sz * nf.g[4][i + (long long)d.nx * j];
+            if (k == d.nz - 1 && bc.k[5] == VOFP_BC_NEUMANN && nf.g[5]) bb += aze[fz_idx(d, i, j, d.nz)] * Sz * nf.g[5][i + (long long)d.nx * j];
+        }
+        b[c] = off ? 0.0 : bb;
+        fzm = f.zp;
     }
 }
 
@@ -678,7 +826,8 @@ vofp_status build_operator(vofp_ctx* c, const double* F, const double* ax, const
             (s = c->alloc(&c->ky, N)) || (s = c->alloc(&c->kz, N)) ||
             (s = c->alloc(&c->slave_bits, (N + 31) / 32)) || (s = c->alloc(&c->root, N)) ||
             (s = c->alloc(&c->red_bits, (N + 31) / 32)) || (s = c->alloc(&c->excl_bits, (N + 31) / 32)) ||
-            (s = c->alloc(&c->inactive, N)) || (s = c->alloc(&c->work, N)) ||
+            (s = c->alloc(&c->inactive, N)) ||
+            (s = c->alloc(&c->tab, 8 + 2 * ((long long)d.nx + d.ny + d.nz))) || (s = c->alloc(&c->work, N)) ||
             (s = c->alloc(&c->partials, kMaxPartials)) || (s = c->alloc(&c->counters, 64)) ||
             (s = c->alloc(&c->sc, 4)))
             return s;
@@ -699,43 +848,56 @@ vofp_status build_operator(vofp_ctx* c, const double* F, const double* ax, const
         c->dirichlet |= bc->kind[f] == VOFP_BC_DIRICHLET;
     }
     const int gN = grid_for(N);
+    const March m3 = march_of(d);
+    const int gM = (int)ceil_div(d.plane * m3.nch, kNT);
 
-    // density (Eq. density), optional smoothing (Sec. 2.10); rho lives in Txs during assembly
-    double* rho = c->Txs;
-    double* tmp = c->Tys;
-    launch(c, k_density, gN, kNT, st, d, F, phys->rho_liquid, phys->rho_gas, rho);
+    // density (Eq. density), optional smoothing (Sec. 2.10, through Txs)
+    launch(c, k_tables, ceil_div(2 * (d.nx + d.ny + d.nz), kNT), kNT, st, d, phys->rho_liquid, phys->rho_gas,
+           phys->density_smoothing ? 1 : 0, (const double*)c->dx, (const double*)c->dy, (const double*)c->dz, c->tab);
     if (phys->density_smoothing) {
-        for (int axis = 0; axis < 3; ++axis) {
-            launch(c, k_smooth, gN, kNT, st, d, axis, rho, tmp);
-            std::swap(rho, tmp);
+        launch(c, k_density_x, gN, kNT, st, d, F, phys->rho_liquid, phys->rho_gas, (const double*)c->tab, c->Txs);
+        launch(c, k_smooth_yz, gM, kNT, st, d, m3, (const double*)c->Txs, (const double*)c->tab, c->rho);
+    } else {
+        launch(c, k_density, gN, kNT, st, d, F, phys->rho_liquid, phys->rho_gas, (const double*)c->tab, c->rho);
+    }
+    // activity, effective apertures and small cells; the activity is iterated to a fixed point, which it
+    // nearly always is at the start
+    unsigned int* cnt = c->counters + 32;
+    unsigned int hc[3] = {0, 0, 0};   // cells that lose their unknown, small cells, cells without one
+    const double thr = vf ? phys->merge_threshold : 0.0;
+    const uint8_t* settled = nullptr;
+    for (int attempt = 0; attempt < 3; ++attempt) {
+        VOFP_CUDA_TRY(c, cudaMemsetAsync(cnt, 0, sizeof(hc), st));
+        launch(c, settled ? k_cells<1> : vf ? k_cells<0> : k_cells<2>, gM, kNT, st, d, m3, b6, thr, vf, settled, ax, ay, az,
+               c->dx, c->dy, c->dz, c->inactive, c->root, c->axe, c->aye, c->aze, cnt, c->small_cap, c->small_cells,
+               c->small_targets, c->small_vf);
+        VOFP_CUDA_TRY(c, cudaMemcpyAsync(hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost, st));
+        VOFP_CUDA_TRY(c, cudaStreamSynchronize(st));
+        const bool settle = !settled && hc[0] > 0, grow = (long long)hc[1] > c->small_cap;
+        if (!settle && !grow) break;
+        if (settle) {
+            uint8_t* ina_a = reinterpret_cast<uint8_t*>(c->work);
+            uint8_t* ina_b = ina_a + N;
+            launch(c, k_activity_init, gN, kNT, st, d, vf, ina_a);
+            for (int pass = 0; pass < 100000; ++pass) {
+                VOFP_CUDA_TRY(c, cudaMemsetAsync(cnt, 0, sizeof(unsigned int), st));
+                launch(c, k_activity_step, gN, kNT, st, d, b6, ax, ay, az, ina_a, ina_b, cnt);
+                unsigned int h = 0;
+                VOFP_CUDA_TRY(c, cudaMemcpyAsync(&h, cnt, sizeof(h), cudaMemcpyDeviceToHost, st));
+                VOFP_CUDA_TRY(c, cudaStreamSynchronize(st));
+                std::swap(ina_a, ina_b);
+                if (h == 0) break;
+            }
+            settled = ina_a;
         }
+        if (grow && attempt < 2 && (s = grow_small(c, (long long)hc[1] + hc[1] / 2 + 1024))) return s;
     }
-    VOFP_CUDA_TRY(c, cudaMemcpyAsync(c->rho, rho, sizeof(double) * N, cudaMemcpyDeviceToDevice, st));
-    // activity, iterated to a fixed point
-    uint8_t* ina_a = c->inactive;
-    uint8_t* ina_b = reinterpret_cast<uint8_t*>(c->work);
-    launch(c, k_activity_init, gN, kNT, st, d, vf, ina_a);
-    unsigned int* changed = c->counters + 32;
-    for (int pass = 0; pass < 100000; ++pass) {
-        VOFP_CUDA_TRY(c, cudaMemsetAsync(changed, 0, sizeof(unsigned int), st));
-        launch(c, k_activity_step, gN, kNT, st, d, b6, ax, ay, az, ina_a, ina_b, changed);
-        unsigned int h = 0;
-        VOFP_CUDA_TRY(c, cudaMemcpyAsync(&h, changed, sizeof(h), cudaMemcpyDeviceToHost, st));
-        VOFP_CUDA_TRY(c, cudaStreamSynchronize(st));
-        std::swap(ina_a, ina_b);
-        if (h == 0) break;
+    const unsigned int m = hc[1];
+    if ((long long)m > c->small_cap) {
+        c->set_error("small-cell count changed between two passes over the same input");
+        return VOFP_ERR_CUDA;
     }
-    if (ina_a != c->inactive)
-        VOFP_CUDA_TRY(c, cudaMemcpyAsync(c->inactive, ina_a, N, cudaMemcpyDeviceToDevice, st));
-    {
-        unsigned int* ninact = c->counters + 34;
-        VOFP_CUDA_TRY(c, cudaMemsetAsync(ninact, 0, sizeof(unsigned int), st));
-        launch(c, k_count_u8, gN, kNT, st, d.n, c->inactive, ninact);
-        unsigned int h = 0;
-        VOFP_CUDA_TRY(c, cudaMemcpyAsync(&h, ninact, sizeof(h), cudaMemcpyDeviceToHost, st));
-        VOFP_CUDA_TRY(c, cudaStreamSynchronize(st));
-        c->n_inactive = h;
-    }
+    c->n_inactive = hc[2];
     // prescribed Neumann fluxes are copied so the caller's arrays need not outlive this call
     for (int f = 0; f < 6; ++f) {
         const long long nb = f < 2 ? (long long)d.ny * d.nz : f < 4 ? (long long)d.nx * d.nz : (long long)d.nx * d.ny;
@@ -748,63 +910,41 @@ vofp_status build_operator(vofp_ctx* c, const double* F, const double* ax, const
             c->has_nflux[f] = false;
         }
     }
-    launch(c, k_eff_apertures, grid_for(nfx + nfy + nfz), kNT, st, d, ax, ay, az, c->inactive, c->axe, c->aye, c->aze);
-    if (d.nx % 2 == 0) {
-        // x-pairs of cells, 16-byte words on the cell and y/z-face streams
-        const int gP = grid_for(d.n / 2);
-        launch(c, k_face_coeffs2, gP, kNT, st, d, c->dx, c->dy, c->dz, rho, c->axe, c->aye, c->aze, c->Tx, c->Ty,
-               c->Tz, c->kx, c->ky, c->kz);
-        launch(c, k_diag2, gP, kNT, st, d, b6, c->dx, c->dy, c->dz, rho, c->axe, c->aye, c->aze, c->Tx, c->Ty, c->Tz,
-               c->diag);
-    } else {
-        launch(c, k_face_coeffs, gN, kNT, st, d, c->dx, c->dy, c->dz, rho, c->axe, c->aye, c->aze, c->Tx, c->Ty,
-               c->Tz, c->kx, c->ky, c->kz);
-        launch(c, k_diag, gN, kNT, st, d, b6, c->dx, c->dy, c->dz, rho, c->axe, c->aye, c->aze, c->Tx, c->Ty, c->Tz,
-               c->diag);
-    }
-
     // merge map (Sec. 2.3): small cells listed on the device, chains resolved on the host
     std::vector<long long> cells, targets, roots;
     std::vector<double> vfs;
     std::vector<int32_t> tslot;
-    unsigned int* cnt = c->counters + 33;
-    if (vf && phys->merge_threshold > 0.0) {
-        unsigned int m = 0;
-        for (int attempt = 0; attempt < 2; ++attempt) {
-            VOFP_CUDA_TRY(c, cudaMemsetAsync(cnt, 0, sizeof(unsigned int), st));
-            launch(c, k_small_cells, gN, kNT, st, d, phys->merge_threshold, vf, c->inactive, c->dx, c->dy, c->dz,
-                   c->axe, c->aye, c->aze, cnt, c->small_cap, c->small_cells, c->small_targets, c->small_vf);
-            VOFP_CUDA_TRY(c, cudaMemcpyAsync(&m, cnt, sizeof(m), cudaMemcpyDeviceToHost, st));
-            VOFP_CUDA_TRY(c, cudaStreamSynchronize(st));
-            if ((long long)m <= c->small_cap) break;
-            if ((s = grow_small(c, (long long)m + m / 2 + 1024))) return s;
-        }
-        if ((long long)m > c->small_cap) {
-            c->set_error("small-cell count changed between two passes over the same input");
-            return VOFP_ERR_CUDA;
-        }
-        if (m > 0) {
-            // root[] serves as the cell -> slot map here; k_root_init below rewrites it
-            VOFP_CUDA_TRY(c, cudaMemsetAsync(c->root, 0xff, sizeof(int32_t) * N, st));
-            launch(c, k_small_slots, ceil_div(m, kNT), kNT, st, (int)m, (const long long*)c->small_cells, c->root);
-            launch(c, k_small_target_slots, ceil_div(m, kNT), kNT, st, (int)m, (const long long*)c->small_targets,
-                   (const int32_t*)c->root, c->small_tslot);
-            cells.resize(m);
-            targets.resize(m);
-            vfs.resize(m);
-            tslot.resize(m);
-            VOFP_CUDA_TRY(c, cudaMemcpyAsync(cells.data(), c->small_cells, sizeof(long long) * m,
-                                             cudaMemcpyDeviceToHost, st));
-            VOFP_CUDA_TRY(c, cudaMemcpyAsync(targets.data(), c->small_targets, sizeof(long long) * m,
-                                             cudaMemcpyDeviceToHost, st));
-            VOFP_CUDA_TRY(c, cudaMemcpyAsync(vfs.data(), c->small_vf, sizeof(double) * m, cudaMemcpyDeviceToHost, st));
-            VOFP_CUDA_TRY(c, cudaMemcpyAsync(tslot.data(), c->small_tslot, sizeof(int32_t) * m,
-                                             cudaMemcpyDeviceToHost, st));
-            VOFP_CUDA_TRY(c, cudaStreamSynchronize(st));
-        }
+    if (m > 0) {
+        // the slots are mapped through Txs, which is not in use here
+        int32_t* slot_of = reinterpret_cast<int32_t*>(c->Txs);
+        VOFP_CUDA_TRY(c, cudaMemsetAsync(slot_of, 0xff, sizeof(int32_t) * N, st));
+        launch(c, k_small_slots, ceil_div(m, kNT), kNT, st, (int)m, (const long long*)c->small_cells, slot_of);
+        launch(c, k_small_target_slots, ceil_div(m, kNT), kNT, st, (int)m, (const long long*)c->small_targets,
+               (const int32_t*)slot_of, c->small_tslot);
+        cells.resize(m);
+        targets.resize(m);
+        vfs.resize(m);
+        tslot.resize(m);
+        VOFP_CUDA_TRY(c, cudaMemcpyAsync(cells.data(), c->small_cells, sizeof(long long) * m,
+                                         cudaMemcpyDeviceToHost, st));
+        VOFP_CUDA_TRY(c, cudaMemcpyAsync(targets.data(), c->small_targets, sizeof(long long) * m,
+                                         cudaMemcpyDeviceToHost, st));
+        VOFP_CUDA_TRY(c, cudaMemcpyAsync(vfs.data(), c->small_vf, sizeof(double) * m, cudaMemcpyDeviceToHost, st));
+        VOFP_CUDA_TRY(c, cudaMemcpyAsync(tslot.data(), c->small_tslot, sizeof(int32_t) * m,
+                                         cudaMemcpyDeviceToHost, st));
+        VOFP_CUDA_TRY(c, cudaStreamSynchronize(st));
     }
+    // the coefficients, the diagonal and its scaling do not need the merge map: the device forms them while the
+    // host resolves it
+    unsigned int* nred = c->counters + 35;
+    VOFP_CUDA_TRY(c, cudaMemsetAsync(nred, 0, sizeof(unsigned int), st));
+    launch(c, k_face_coeffs, gM, kNT, st, d, m3, c->dx, c->dy, c->dz, c->rho, c->axe, c->aye, c->aze, c->tab, c->Tx, c->Ty,
+           c->Tz, c->kx, c->ky, c->kz);
+    launch(c, k_diag_scale, gM, kNT, st, d, m3, b6, c->dx, c->dy, c->dz, c->rho, c->axe, c->aye, c->aze, c->Tx, c->Ty,
+           c->Tz, c->inactive, c->diag, c->s, c->sq);
+    launch(c, k_cell_bits, grid_for((N + 31) / 32), kNT, st, d, (const uint8_t*)c->inactive, c->slave_bits, c->red_bits,
+           nred);
     resolve_roots(cells, targets, vfs, tslot, roots);
-    launch(c, k_root_init, gN, kNT, st, d, c->inactive, c->root);
     // groups: cells whose root differs from themselves, plus the roots
     std::vector<std::pair<long long, long long>> members;   // (root, cell)
     for (size_t t = 0; t < cells.size(); ++t)
@@ -841,26 +981,22 @@ vofp_status build_operator(vofp_ctx* c, const double* F, const double* ax, const
         launch(c, k_root_scatter, ceil_div((long long)mc.size(), kNT), kNT, st, (int)mc.size(),
                (const long long*)c->small_cells, (const long long*)c->small_targets, c->root);
     }
-    // symmetric scaling s = diag(A_hat)^-1/2 per group
-    launch(c, k_scale_cells, gN, kNT, st, d, c->inactive, c->diag, c->s, c->sq);
-    if (c->ngroups > 0)
+    // the groups' scale s = diag(A_hat)^-1/2 and flags
+    if (c->ngroups > 0) {
         launch(c, k_scale_groups, ceil_div(c->ngroups, kNT), kNT, st, d, c->ngroups, c->gptr, c->gcells, c->root, c->diag,
                                                                   c->Tx, c->Ty, c->Tz, c->s, c->sq, c->gcorr);
-    launch(c, k_scaled_coeffs, gN, kNT, st, d, c->s, c->Tx, c->Ty, c->Tz, c->Txs, c->Tys, c->Tzs, c->Txf, c->Tyf, c->Tzf);
-    launch(c, k_slave_bits, grid_for((N + 31) / 32), kNT, st, d, c->root, c->slave_bits);
-    {
-        unsigned int* nred = c->counters + 35;
-        VOFP_CUDA_TRY(c, cudaMemsetAsync(nred, 0, sizeof(unsigned int), st));
-        launch(c, k_red_bits, grid_for((N + 31) / 32), kNT, st, d, (const int32_t*)c->root,
-               (const uint32_t*)c->slave_bits, c->red_bits, c->excl_bits, nred);
-        launch(c, k_signed_tz, gN, kNT, st, d.n, (const float*)c->Tzf, (const uint32_t*)c->red_bits, c->Tzr);
-        unsigned int h = 0;
-        VOFP_CUDA_TRY(c, cudaMemcpyAsync(&h, nred, sizeof(h), cudaMemcpyDeviceToHost, st));
-        VOFP_CUDA_TRY(c, cudaStreamSynchronize(st));
-        c->n_red = h;
+        launch(c, k_group_flags, ceil_div(c->ngroups, kNT), kNT, st, c->ngroups, (const int*)c->gptr,
+               (const int*)c->gcells, c->slave_bits, c->red_bits, nred);
     }
+    launch(c, k_excl_bits, grid_for((N + 31) / 32), kNT, st, (N + 31) / 32, (const uint32_t*)c->slave_bits,
+           (const uint32_t*)c->red_bits, c->excl_bits);
+    launch(c, k_scaled_coeffs, gM, kNT, st, d, m3, (const double*)c->s, (const double*)c->Tx, (const double*)c->Ty,
+           (const double*)c->Tz, (const uint32_t*)c->red_bits, c->Txs, c->Tys, c->Tzs, c->Txf, c->Tyf, c->Tzf, c->Tzr);
+    unsigned int hred = 0;
+    VOFP_CUDA_TRY(c, cudaMemcpyAsync(&hred, nred, sizeof(hred), cudaMemcpyDeviceToHost, st));
     VOFP_CUDA_TRY(c, cudaGetLastError());
     VOFP_CUDA_TRY(c, cudaStreamSynchronize(st));
+    c->n_red = hred;
     c->built = true;
     return VOFP_OK;
 }
@@ -872,8 +1008,12 @@ vofp_status rhs(vofp_ctx* c, const double* u, const double* v, const double* w, 
     for (int f = 0; f < 6; ++f) b6.k[f] = c->bc[f];
     Flux6 nf{};
     for (int f = 0; f < 6; ++f) nf.g[f] = c->has_nflux[f] ? c->nflux[f] : nullptr;
-    launch(c, k_rhs, grid_for(d.n), kNT, c->stream, d, b6, nf, c->phys.dt, c->dx, c->dy, c->dz, c->axe, c->aye,
-                                                c->aze, c->inactive, u, v, w, body, b);
+    const March m = march_of(d);
+    const double dt = c->phys.dt;
+    int e = 0;
+    const bool pow2 = std::isnormal(dt) && std::fabs(std::frexp(dt, &e)) == 0.5 && std::isnormal(1.0 / dt);
+    launch(c, dt == 1.0 ? k_rhs<0> : pow2 ? k_rhs<1> : k_rhs<2>, ceil_div(d.plane * m.nch, kNT), kNT, c->stream, d, m, b6, nf,
+           pow2 ? 1.0 / dt : dt, c->dx, c->dy, c->dz, c->axe, c->aye, c->aze, c->inactive, u, v, w, body, b);
     VOFP_CUDA_TRY(c, cudaGetLastError());
     return VOFP_OK;
 }

@@ -136,6 +136,7 @@ struct vofp_ctx {
     uint32_t* excl_bits = nullptr;
     long long n_red = 0;
     int32_t* root = nullptr;          // group root per cell, -1 without unknown
+    double* tab = nullptr;                                // pure phases' densities and face factors (k_tables)
     uint8_t* inactive = nullptr;
     // merge groups with more than one cell: cells of group g are gcells[gptr[g] .. gptr[g+1]),
     // master first; gcorr[g] = s_m^2 * sum of the cells' diagonals - |G|
