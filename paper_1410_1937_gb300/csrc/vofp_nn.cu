@@ -53,9 +53,18 @@ __host__ __device__ __forceinline__ long long aidx(long long v, int c, long long
 // channel group.  The three z taps are columns of one instruction: input plane p times the
 // weights of the three z taps (N = 3 NOUT) gives in one MMA the contributions of p to output
 // planes p+1, p and p-1, which sit in consecutive TMEM column blocks (block j: z tap j, output
-// p+1-j).  Output plane o therefore owns columns NOUT (S + 1 - (o - z0)) of a segment of S planes
-// starting at z0 (descending in o), with one block above and two below for the contributions that
-// fall outside the segment.  Each input plane is read by 9 taps x (Cin/16) MMAs and released.
+// p+1-j).  The column blocks are a ring of NB, taken in descending order by consecutive output planes;
+// where the three wrap around its end an instruction is issued in two pieces, and the first and last
+// planes of a segment take only the blocks of outputs that exist.  Each input plane is read by
+// 9 taps x (Cin/16) MMAs and released, each finished output plane is read back and its columns released.
+//
+// Blocks are persistent: each keeps its weights and takes segments of z columns in turn, all blocks
+// neighbouring ones at a time (halo rows through L2).  What bounds it is issuing: an instruction reads the 128
+// rows of A (4 KB) from shared memory, some 40 cycles whatever N up to 48, and one thread of a diverged warp
+// needs 100 and more to form its operands.  So the whole warp forms them in uniform registers, the taps are
+// unrolled, and four blocks share an SM where tensor memory and shared memory allow it.  512 x 256 x 128:
+// 16 -> 16 channels 544 us with a block per segment of twelve planes and a single issuing thread, 424 persistent,
+// 337 with uniform operands, 277 unrolled; 48 -> 16 938 -> 698; 96 -> 32 at half resolution 736 -> 507.
 constexpr int kTileX = 8, kTileY = 16, kBoxX = kTileX + 2, kBoxY = kTileY + 2;
 constexpr int kGroupBytes = kBoxX * kBoxY * 16;   // one channel group of one halo'd plane
 constexpr int kConvThreads = 192;                 // warp 0 copies, warp 1 issues MMAs, 2..5 store
@@ -69,22 +78,23 @@ template <int CIN, int NOUT, int R>
 struct ConvCfg {
     static_assert(CIN % 16 == 0 && NOUT % 16 == 0 && 3 * NOUT <= 256, "shape");
     static constexpr int KCH = CIN / 8;                               // input channel groups
-    // output planes per segment: the accumulators of S + 4 planes (S outputs and the blocks that
-    // fall outside the segment) in TMEM; two blocks per SM for 16 output channels, one otherwise
-    static constexpr int S = NOUT == 16 ? 12 : (NOUT == 32 ? 12 : (NOUT == 48 ? 6 : 4));
-    static constexpr uint32_t TCOLS = pow2_at_least((uint32_t)NOUT * (S + 4));
+    // column blocks of the accumulator ring: three in use by the plane at hand, the others being read back;
+    // four blocks per SM for 16 output channels, two or one (where shared memory allows one) otherwise
+    static constexpr int NB = NOUT == 48 ? (CIN == 16 ? 5 : 10) : NOUT == 16 ? (CIN <= 32 ? 8 : CIN / 3) : NOUT == 32 && CIN == 64 ? 16 : 8;
+    static constexpr uint32_t TCOLS = pow2_at_least((uint32_t)NOUT * NB);
+    static constexpr int MINB = TCOLS == 128 ? 4 : TCOLS == 256 ? 2 : 1;   // blocks per SM by tensor memory
     static constexpr uint32_t PLANE = (uint32_t)KCH * kGroupBytes;    // bytes of one ring slot
     static constexpr uint32_t WBYTES = 27u * CIN * NOUT * 2u;         // this block's weights
     static constexpr uint32_t WTAP = (uint32_t)KCH * 3 * NOUT * 16;   // weights of one (y, x) tap
     static constexpr size_t oW = 0;
     static constexpr size_t oRing = al128(WBYTES);
     static constexpr size_t oBar = oRing + al128((size_t)R * PLANE);
-    static constexpr size_t oBias = oBar + 8 * (2 * R + S + 1) + 8;
+    static constexpr size_t oBias = oBar + 8 * (2 * R + 2 * NB + 1) + 8;
     static constexpr size_t SMEM_USED = al128(oBias + 4 * NOUT) + 128;   // + alignment slack
     // requested shared memory: at least enough to keep the blocks per SM within what tensor memory
     // holds (512 columns per SM), so that no block waits inside its TMEM allocation
-    static constexpr size_t SMEM = TCOLS == 512 ? (SMEM_USED > 120 * 1024 ? SMEM_USED : 120 * 1024)
-                                 : TCOLS == 256 ? (SMEM_USED > 80 * 1024 ? SMEM_USED : 80 * 1024) : SMEM_USED;
+    static constexpr size_t SMEM_MIN = TCOLS == 512 ? 120 * 1024 : TCOLS == 256 ? 80 * 1024 : 48 * 1024;
+    static constexpr size_t SMEM = SMEM_USED > SMEM_MIN ? SMEM_USED : SMEM_MIN;
     static_assert(SMEM <= 232448, "shared memory per block");
     static_assert(TCOLS <= 512, "tensor memory");
 };
@@ -92,7 +102,8 @@ struct ConvCfg {
 struct ConvArgs {
     int nx, ny, nz;
     int tiles_x, tiles_y;
-    int seg, nseg;            // planes per z segment (<= S), segments
+    int seg, nseg;            // planes per z segment, segments
+    int nsplit;               // blocks of output channels
     long long V;              // voxels of the level
     const float* bias;        // per output channel (null: none)
     int relu;
@@ -102,40 +113,50 @@ struct ConvArgs {
     int* err;                 // set to 1 when a bounded wait runs out
 };
 
-// Block order: x tiles fastest, then y tiles, z segments, output-channel splits (neighbouring
-// blocks share halo rows through L2).
+// Segments in the order x tiles fastest, then y tiles, z segments.  Block b takes output-channel split
+// b % nsplit and the segments b / nsplit, + gridDim / nsplit, ...
+struct ConvSeg {
+    int x0, y0, z0, nout;   // output planes z0 .. z0 + nout - 1
+};
+__device__ __forceinline__ ConvSeg conv_seg(const ConvArgs& a, int u) {
+    ConvSeg g;
+    const int t = u / a.tiles_x;
+    g.x0 = (u - t * a.tiles_x) * kTileX;
+    const int sg = t / a.tiles_y;
+    g.y0 = (t - sg * a.tiles_y) * kTileY;
+    g.z0 = sg * a.seg;
+    g.nout = min(a.nz, g.z0 + a.seg) - g.z0;
+    return g;
+}
+
 template <int CIN, int NOUT, int R>
-__global__ void __launch_bounds__(kConvThreads, 1)
+__global__ void __launch_bounds__(kConvThreads, (ConvCfg<CIN, NOUT, R>::MINB))
 k_conv3_umma(const __grid_constant__ CUtensorMap in_map, const ConvArgs a) {
     using G = ConvCfg<CIN, NOUT, R>;
-    constexpr int S = G::S;
+    constexpr int NB = G::NB;
     extern __shared__ unsigned char smraw[];
     unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smraw) + 127) & ~uintptr_t(127));
     unsigned char* wsm = sm + G::oW;
     unsigned char* ring = sm + G::oRing;
     uint64_t* full = reinterpret_cast<uint64_t*>(sm + G::oBar);
     uint64_t* empty = full + R;
-    uint64_t* accf = empty + R;   // one per output plane of the segment
-    uint64_t* wbar = accf + S;
+    uint64_t* accf = empty + R;   // per column block: output plane complete, read back
+    uint64_t* acce = accf + NB;
+    uint64_t* wbar = acce + NB;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(wbar + 1);
     float* bsm = reinterpret_cast<float*>(sm + G::oBias);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    int b = blockIdx.x;
-    const int tx = b % a.tiles_x;
-    b /= a.tiles_x;
-    const int ty = b % a.tiles_y;
-    b /= a.tiles_y;
-    const int sg = b % a.nseg, split = b / a.nseg;
-    const int x0 = tx * kTileX, y0 = ty * kTileY;
-    const int z0 = sg * a.seg;
-    const int nout = min(a.nz, z0 + a.seg) - z0;   // output planes of this block (1 .. S)
-    const int nin = nout + 2;                       // input planes z0-1 .. z0+nout
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const int split = blockIdx.x % a.nsplit, u0 = blockIdx.x / a.nsplit, du = gridDim.x / a.nsplit;
+    const int units = a.tiles_x * a.tiles_y * a.nseg;
     if (tid == 0) {
         for (int i = 0; i < R; ++i) {
             mbar_init(&full[i], 1);
             mbar_init(&empty[i], 1);
         }
-        for (int i = 0; i < S; ++i) mbar_init(&accf[i], 1);
+        for (int i = 0; i < NB; ++i) {
+            mbar_init(&accf[i], 1);
+            mbar_init(&acce[i], 4);
+        }
         mbar_init(wbar, 1);
         fence_mbar_init();
     }
@@ -153,103 +174,141 @@ k_conv3_umma(const __grid_constant__ CUtensorMap in_map, const ConvArgs a) {
             mbar_expect_tx(wbar, G::WBYTES);
             umma::bulk_load(wsm, reinterpret_cast<const unsigned char*>(a.wblob) + (size_t)split * G::WBYTES,
                             G::WBYTES, wbar);
-            int issued = 0;
-            for (int lp = 0; lp < nin; ++lp) {
-                const int s = lp % R;
-                if (lp >= R && !mbar_wait_bounded(&empty[s], (uint32_t)((lp / R) - 1) & 1u)) {
-                    fail = true;
-                    break;
+            int ip = 0;   // input planes so far
+            for (int u = u0; u < units && !fail; u += du) {
+                const ConvSeg g = conv_seg(a, u);
+                for (int lp = 0; lp < g.nout + 2; ++lp, ++ip) {
+                    const int s = ip % R;
+                    if (ip >= R && !mbar_wait_bounded(&empty[s], (uint32_t)((ip / R) - 1) & 1u)) {
+                        fail = true;
+                        break;
+                    }
+                    mbar_expect_tx(&full[s], G::PLANE);
+                    umma::tma_load_5d(ring + (size_t)s * G::PLANE, &in_map, &full[s], 0, g.x0 - 1, g.y0 - 1,
+                                      g.z0 - 1 + lp, 0);
                 }
-                mbar_expect_tx(&full[s], G::PLANE);
-                umma::tma_load_5d(ring + (size_t)s * G::PLANE, &in_map, &full[s], 0, x0 - 1, y0 - 1, z0 - 1 + lp, 0);
-                ++issued;
             }
             // every copy issued must have landed before the block may leave
-            for (int lp = max(0, issued - R); lp < issued; ++lp)
-                if (!mbar_wait_bounded(&full[lp % R], (uint32_t)(lp / R) & 1u)) fail = true;
+            for (int p = max(0, ip - R); p < ip; ++p)
+                if (!mbar_wait_bounded(&full[p % R], (uint32_t)(p / R) & 1u)) fail = true;
             if (!mbar_wait_bounded(wbar, 0)) fail = true;
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t id1 = umma::idesc_bf16(128, NOUT), id2 = umma::idesc_bf16(128, 2 * NOUT),
-                               id3 = umma::idesc_bf16(128, 3 * NOUT);
-            const uint32_t wbase = umma::saddr(wsm), rbase = umma::saddr(ring);
-            if (!mbar_wait_bounded(wbar, 0)) fail = true;
-            for (int lp = 0; lp < nin && !fail; ++lp) {
-                const int s = lp % R;
-                if (!mbar_wait_bounded(&full[s], (uint32_t)(lp / R) & 1u)) {
+        // the whole warp follows (its operands are uniform), one lane issues
+        const bool lead = lane == 0;
+        const uint32_t wbase = umma::saddr(wsm), rbase = umma::saddr(ring);
+        fail = !__all_sync(0xffffffffu, mbar_wait_bounded(wbar, 0));
+        int ip = 0, ob = 0;   // input planes and output planes before this segment's
+        for (int u = u0; u < units && !fail; u += du) {
+            const ConvSeg g = conv_seg(a, u);
+            for (int lp = 0; lp < g.nout + 2; ++lp, ++ip) {
+                const int s = ip % R;
+                const bool fresh = lp < g.nout;   // output plane lp is begun
+                // output planes hi, hi - 1, ... (n of them) are z taps j0, j0 + 1, ...
+                const int hi = min(lp, g.nout - 1), n = hi - max(lp - 2, 0) + 1, j0 = lp - hi;
+                const int q = (ob + hi) % NB;
+                bool ok = mbar_wait_bounded(&full[s], (uint32_t)(ip / R) & 1u);
+                if (fresh && ob + hi >= NB) ok = ok && mbar_wait_bounded(&acce[q], (uint32_t)((ob + hi) / NB - 1) & 1u);
+                if (!__all_sync(0xffffffffu, ok)) {
                     fail = true;
                     break;
                 }
                 umma::fence_after_sync();
-                // input plane z0-1+lp: block j of the result is output plane z0+lp-j
-                const uint32_t d = tmem + (uint32_t)(NOUT * (S + 1 - lp));
-                const uint32_t slot = rbase + (uint32_t)s * G::PLANE;
-#pragma unroll 1
-                for (int t = 0; t < 9; ++t) {
-                    const int dy = t / 3, dx = t % 3;
-                    const uint32_t abase = slot + (uint32_t)(dy * kBoxX + dx) * 16u;
-                    const uint32_t bbase = wbase + (uint32_t)t * G::WTAP;
+                const int c0 = NB - 1 - q, n1 = min(n, NB - c0);   // column blocks c0 .. and, wrapped, 0 ..
+                const uint32_t d = tmem + (uint32_t)(NOUT * c0);
+                const uint32_t id1 = umma::idesc_bf16(128, 0) | (uint32_t)(n1 * NOUT / 8) << 17,
+                               id2 = umma::idesc_bf16(128, 0) | (uint32_t)((n - n1) * NOUT / 8) << 17;
+                const uint64_t ad0 = umma::smem_desc(rbase + (uint32_t)s * G::PLANE, kGroupBytes, kBoxX * 16);
+                const uint64_t bd0 = umma::smem_desc(wbase + (uint32_t)(j0 * (NOUT / 8) * 128), 3 * NOUT * 16, 128);
+                constexpr uint32_t kBlk = (NOUT / 8) * 128;   // bytes from one z tap's weights to the next
+                // instruction x: (y, x) tap x / (CIN / 16), 16 input channels from 16 (x % (CIN / 16)) on
+                auto adesc = [&](int x) {
+                    const int t = x / (CIN / 16), ks = x % (CIN / 16);
+                    return ad0 + (uint32_t)((t / 3) * kBoxX + t % 3 + (2 * ks * kGroupBytes >> 4));
+                };
+                auto bdesc = [&](int x) {
+                    const int t = x / (CIN / 16), ks = x % (CIN / 16);
+                    return bd0 + ((uint32_t)t * G::WTAP + 2u * ks * (3 * NOUT * 16) >> 4);
+                };
+                if (fresh) {
+                    // the first block starts its output plane afresh; the others add to planes that earlier
+                    // input planes began
+                    umma::mma_bf16_if(lead, d, ad0, bd0, umma::idesc_bf16(128, NOUT), 0u);
+                    for (int e = 1; e < n; ++e)
+                        umma::mma_bf16_if(lead, tmem + (uint32_t)(NOUT * ((c0 + e) % NB)), ad0, bd0 + (e * kBlk >> 4),
+                                          umma::idesc_bf16(128, NOUT), 1u);
+                } else {
+                    umma::mma_bf16_if(lead, d, ad0, bd0, id1, 1u);
+                    if (n1 < n) umma::mma_bf16_if(lead, tmem, ad0, bd0 + (n1 * kBlk >> 4), id2, 1u);
+                }
+                if (n1 == n) {
 #pragma unroll
-                    for (int ks = 0; ks < CIN / 16; ++ks) {
-                        const uint64_t ad = umma::smem_desc(abase + 2u * ks * kGroupBytes, kGroupBytes, kBoxX * 16);
-                        const uint32_t bk = bbase + 2u * ks * (3 * NOUT * 16);
-                        if (t == 0 && ks == 0) {
-                            // block 0 starts output plane z0+lp afresh; blocks 1, 2 add to planes
-                            // that earlier input planes began
-                            umma::mma_bf16(d, ad, umma::smem_desc(bk, 3 * NOUT * 16, 128), id1, 0u);
-                            umma::mma_bf16(d + NOUT, ad, umma::smem_desc(bk + (NOUT / 8) * 128, 3 * NOUT * 16, 128),
-                                           id2, 1u);
-                        } else {
-                            umma::mma_bf16(d, ad, umma::smem_desc(bk, 3 * NOUT * 16, 128), id3, 1u);
-                        }
+                    for (int x = 1; x < 9 * (CIN / 16); ++x) umma::mma_bf16_if(lead, d, adesc(x), bdesc(x), id1, 1u);
+                } else {
+#pragma unroll
+                    for (int x = 1; x < 9 * (CIN / 16); ++x) {
+                        umma::mma_bf16_if(lead, d, adesc(x), bdesc(x), id1, 1u);
+                        umma::mma_bf16_if(lead, tmem, adesc(x), bdesc(x) + (n1 * kBlk >> 4), id2, 1u);
                     }
                 }
-                umma::commit(&empty[s]);                     // the plane's slot may be refilled
-                if (lp >= 2) umma::commit(&accf[lp - 2]);    // output plane z0+lp-2 is complete
+                if (lead) umma::commit(&empty[s]);                              // the plane's slot may be refilled
+                if (lead && lp >= 2) umma::commit(&accf[(ob + lp - 2) % NB]);     // output plane lp - 2 is complete
             }
+            ob += g.nout;
+        }
+        if (lead && fail && ip > 0) {   // the instructions issued must have ended before the tensor memory is freed
+            umma::commit(wbar);
+            mbar_wait_bounded(wbar, 1);
         }
     } else {
         // epilogue: TMEM lane quadrant (warp % 4) of the 128 rows; row m = voxel (m % 8, m / 8)
         const int q = warp & 3;
         const int m = q * 32 + lane;
-        const int xi = x0 + (m & 7), yi = y0 + (m >> 3);
-        const bool inside = xi < a.nx && yi < a.ny;
-        for (int lz = 0; lz < nout; ++lz) {
-            if (!fail && !mbar_wait_bounded(&accf[lz], 0u)) fail = true;
-            if (__any_sync(0xffffffffu, fail)) {
-                fail = true;
-                break;
-            }
-            umma::fence_after_sync();
-            const uint32_t col = (uint32_t)(NOUT * (S + 1 - lz));
-            float v[NOUT];
+        int o = 0;   // output planes so far
+        for (int u = u0; u < units && !fail; u += du) {
+            const ConvSeg g = conv_seg(a, u);
+            const int xi = g.x0 + (m & 7), yi = g.y0 + (m >> 3);
+            const bool inside = xi < a.nx && yi < a.ny;
+            for (int lz = 0; lz < g.nout; ++lz, ++o) {
+                const int qb = o % NB;
+                if (!mbar_wait_bounded(&accf[qb], (uint32_t)(o / NB) & 1u)) fail = true;
+                if (__any_sync(0xffffffffu, fail)) {
+                    fail = true;
+                    break;
+                }
+                umma::fence_after_sync();
+                const uint32_t col = (uint32_t)(NOUT * (NB - 1 - qb));
+                float v[NOUT];
 #pragma unroll
-            for (int c0 = 0; c0 < NOUT; c0 += 16) {
-                uint32_t r[16];
-                umma::tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + col + c0, r);
-                umma::tmem_wait_ld();
+                for (int c0 = 0; c0 < NOUT; c0 += 16) {
+                    uint32_t r[16];
+                    umma::tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + col + c0, r);
+                    umma::tmem_wait_ld();
 #pragma unroll
-                for (int j = 0; j < 16; ++j) v[c0 + j] = __uint_as_float(r[j]);
-            }
-            if (inside) {
-                const long long vox = ((long long)(z0 + lz) * a.ny + yi) * a.nx + xi;
+                    for (int j = 0; j < 16; ++j) v[c0 + j] = __uint_as_float(r[j]);
+                }
+                umma::fence_before_sync();
+                __syncwarp();
+                if (lane == 0) umma::mbar_arrive(&acce[qb]);   // the columns may be used again
+                if (inside) {
+                    const long long vox = ((long long)(g.z0 + lz) * a.ny + yi) * a.nx + xi;
 #pragma unroll
-                for (int oc = 0; oc < NOUT / 8; ++oc) {
-                    uint32_t w4[4];
+                    for (int oc = 0; oc < NOUT / 8; ++oc) {
+                        uint32_t w4[4];
 #pragma unroll
-                    for (int h = 0; h < 4; ++h) {
-                        float lo = v[oc * 8 + 2 * h] + bsm[oc * 8 + 2 * h];
-                        float hi = v[oc * 8 + 2 * h + 1] + bsm[oc * 8 + 2 * h + 1];
-                        if (a.relu) {
-                            lo = fmaxf(lo, 0.f);
-                            hi = fmaxf(hi, 0.f);
+                        for (int h = 0; h < 4; ++h) {
+                            float lo = v[oc * 8 + 2 * h] + bsm[oc * 8 + 2 * h];
+                            float hi = v[oc * 8 + 2 * h + 1] + bsm[oc * 8 + 2 * h + 1];
+                            if (a.relu) {
+                                lo = fmaxf(lo, 0.f);
+                                hi = fmaxf(hi, 0.f);
+                            }
+                            const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
+                            w4[h] = *reinterpret_cast<const uint32_t*>(&p);
                         }
-                        const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
-                        w4[h] = *reinterpret_cast<const uint32_t*>(&p);
+                        const long long grp = a.out_chunk0 + (long long)split * (NOUT / 8) + oc;
+                        *reinterpret_cast<uint4*>(a.out + (grp * a.V + vox) * 8) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
                     }
-                    const long long grp = a.out_chunk0 + (long long)split * (NOUT / 8) + oc;
-                    *reinterpret_cast<uint4*>(a.out + (grp * a.V + vox) * 8) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
                 }
             }
         }
@@ -380,7 +439,7 @@ k_conv3_wgrad_umma(const __grid_constant__ CUtensorMap x_map, const __grid_const
     uint64_t* empty = full + R;
     uint64_t* done = empty + R;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     int b = blockIdx.x;
     const int chunk = b % a.nchunks;
     b /= a.nchunks;
@@ -426,56 +485,56 @@ k_conv3_wgrad_umma(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 if (!mbar_wait_bounded(&full[i % R], (uint32_t)(i / R) & 1u)) fail = true;
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t id = G::XN ? umma::idesc_bf16_mn(M, 24) : umma::idesc_bf16_mn(M, NCO);
-            const uint32_t xbase = umma::saddr(xs), dbase = umma::saddr(ds);
-            for (int i = 0; i < nitems && !fail; ++i) {
-                const int s = i % R;
-                if (!mbar_wait_bounded(&full[s], (uint32_t)(i / R) & 1u)) {
-                    fail = true;
-                    break;
-                }
-                umma::fence_after_sync();
-                const uint32_t xslot = xbase + (uint32_t)s * G::XSLOT, dslot = dbase + (uint32_t)s * G::DSLOT;
-                // K steps outermost: consecutive instructions go to the nine taps' separate
-                // accumulators
-#pragma unroll 1
-                for (int ks = 0; ks < kTileY / 2 && G::XN; ++ks) {
-                    // K = tile rows 2 ks and 2 ks + 1: gradient box rows one box row (10 voxels)
-                    // apart, the three shifts 16 bytes apart; input box at x offset 2, shifted by
-                    // the y tap
-#pragma unroll
-                    for (int ty = 0; ty < 3; ++ty) {
-                        const uint64_t ad =
-                            umma::smem_desc(xslot + (uint32_t)(((2 * ks + ty) * kBoxX + 2) * 16), kBoxX * 16, kGroupBytes);
-#pragma unroll
-                        for (int cg = 0; cg < G::DG; ++cg) {
-                            const uint64_t bd =
-                                umma::smem_desc(dslot + (uint32_t)(cg * G::DGB + ks * 2 * G::DW * 16), G::DW * 16, 16);
-                            umma::mma_bf16(tmem + (uint32_t)((ty * G::DG + cg) * 24), ad, bd, id,
-                                           (i > 0 || ks > 0) ? 1u : 0u);
-                        }
-                    }
-                }
-#pragma unroll 1
-                for (int ks = 0; ks < kTileY / 2 && !G::XN; ++ks) {
-                    // K = tile rows 2 ks and 2 ks + 1 (8 voxels each): gradient tile rows one tile row
-                    // apart, channel groups one group plane apart
-                    const uint64_t bd = umma::smem_desc(dslot + (uint32_t)(ks * 2 * kTileX * 16), kTileX * 16, G::DGB);
-#pragma unroll
-                    for (int t = 0; t < 9; ++t) {
-                        const int ty = t / 3, tx = t % 3;
-                        // input box rows shifted by the tap, one box row (kBoxX voxels) apart; M
-                        // groups (plane, channel group) one box plane apart
-                        const uint64_t ad =
-                            umma::smem_desc(xslot + (uint32_t)(((2 * ks + ty) * kBoxX + tx) * 16), kBoxX * 16, kGroupBytes);
-                        umma::mma_bf16(tmem + (uint32_t)(t * NCO), ad, bd, id, (i > 0 || ks > 0) ? 1u : 0u);
-                    }
-                }
-                umma::commit(&empty[s]);   // the slot may be refilled
+        // the whole warp follows (its operands are uniform), one lane issues
+        const bool lead = lane == 0;
+        constexpr uint32_t id = G::XN ? umma::idesc_bf16_mn(M, 24) : umma::idesc_bf16_mn(M, NCO);
+        const uint32_t xbase = umma::saddr(xs), dbase = umma::saddr(ds);
+        for (int i = 0; i < nitems && !fail; ++i) {
+            const int s = i % R;
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full[s], (uint32_t)(i / R) & 1u))) {
+                fail = true;
+                break;
             }
-            umma::commit(done);            // every MMA issued has completed
+            umma::fence_after_sync();
+            const uint32_t xslot = xbase + (uint32_t)s * G::XSLOT, dslot = dbase + (uint32_t)s * G::DSLOT;
+            // K steps outermost: consecutive instructions go to the nine taps' separate
+            // accumulators
+#pragma unroll 1
+            for (int ks = 0; ks < kTileY / 2 && G::XN; ++ks) {
+                // K = tile rows 2 ks and 2 ks + 1: gradient box rows one box row (10 voxels)
+                // apart, the three shifts 16 bytes apart; input box at x offset 2, shifted by
+                // the y tap
+#pragma unroll
+                for (int ty = 0; ty < 3; ++ty) {
+                    const uint64_t ad =
+                        umma::smem_desc(xslot + (uint32_t)(((2 * ks + ty) * kBoxX + 2) * 16), kBoxX * 16, kGroupBytes);
+#pragma unroll
+                    for (int cg = 0; cg < G::DG; ++cg) {
+                        const uint64_t bd =
+                            umma::smem_desc(dslot + (uint32_t)(cg * G::DGB + ks * 2 * G::DW * 16), G::DW * 16, 16);
+                        umma::mma_bf16_if(lead, tmem + (uint32_t)((ty * G::DG + cg) * 24), ad, bd, id,
+                                       (i > 0 || ks > 0) ? 1u : 0u);
+                    }
+                }
+            }
+#pragma unroll 1
+            for (int ks = 0; ks < kTileY / 2 && !G::XN; ++ks) {
+                // K = tile rows 2 ks and 2 ks + 1 (8 voxels each): gradient tile rows one tile row
+                // apart, channel groups one group plane apart
+                const uint64_t bd = umma::smem_desc(dslot + (uint32_t)(ks * 2 * kTileX * 16), kTileX * 16, G::DGB);
+#pragma unroll
+                for (int t = 0; t < 9; ++t) {
+                    const int ty = t / 3, tx = t % 3;
+                    // input box rows shifted by the tap, one box row (kBoxX voxels) apart; M
+                    // groups (plane, channel group) one box plane apart
+                    const uint64_t ad =
+                        umma::smem_desc(xslot + (uint32_t)(((2 * ks + ty) * kBoxX + tx) * 16), kBoxX * 16, kGroupBytes);
+                    umma::mma_bf16_if(lead, tmem + (uint32_t)(t * NCO), ad, bd, id, (i > 0 || ks > 0) ? 1u : 0u);
+                }
+            }
+            if (lead) umma::commit(&empty[s]);   // the slot may be refilled
         }
+        if (lead) umma::commit(done);            // every MMA issued has completed
     } else {
         // epilogue: warp quarter q of the TMEM lanes; accumulator row of this lane (M = 64: the
         // first 16 lanes of each quarter), its group plane m (channel group m / 3, z tap m % 3)
@@ -1005,23 +1064,37 @@ template <int CIN, int NOUT, int R>
 vofp_status conv_umma(vofp_nn* n, const CUtensorMap* map, ConvArgs a, int nsplit) {
     using G = ConvCfg<CIN, NOUT, R>;
     auto kern = k_conv3_umma<CIN, NOUT, R>;
-    static int occ = -1;   // resident blocks per SM (per instantiation; one device per process)
-    if (occ < 0) {
+    static bool ready = false;   // (per instantiation; one device per process)
+    if (!ready) {
+        int occ = 0;
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kConvThreads, G::SMEM) != cudaSuccess || occ < 1) {
-            occ = -1;
             n->err = "tensor-core convolution: shared memory opt-in failed";
             return VOFP_ERR_CUDA;
         }
+        ready = true;
     }
-    // z segments of at most S planes (the accumulators one block keeps in tensor memory), equal
-    // in length; each re-reads a 2-plane halo
-    const long long cols = (long long)a.tiles_x * a.tiles_y * nsplit;
-    const int nseg = (a.nz + G::S - 1) / G::S;
-    a.seg = (a.nz + nseg - 1) / nseg;
+    // blocks per SM: what tensor memory and shared memory (228 KB, 1 KB of it per block reserved) hold. (The
+    // occupancy query answers 1 for a kernel that allocates tensor memory.)
+    const int occ = std::min(G::MINB, (int)(228 * 1024 / (G::SMEM + 1024)));
+    // z segments: of the lengths (even, so that a pooled plane stays in one), the one with the fewest planes
+    // in the longest-working block, a segment counting three more (two halo planes and its start)
+    const int slots = std::max(1, num_sms() * occ / nsplit);
+    const long long cols = (long long)a.tiles_x * a.tiles_y;
+    long long best = -1;
+    for (int q = 1; q <= a.nz; ++q) {
+        const int len = std::max(2, ((a.nz + q - 1) / q + 1) / 2 * 2);
+        const long long units = cols * ((a.nz + len - 1) / len), cost = (units + slots - 1) / slots * (len + 3);
+        if (best < 0 || cost < best) {
+            best = cost;
+            a.seg = len;
+        }
+        if (len == 2) break;
+    }
     a.nseg = (a.nz + a.seg - 1) / a.seg;
+    a.nsplit = nsplit;
     a.err = n->derr;
-    const long long blocks = cols * a.nseg;
+    const long long blocks = std::min((long long)slots, cols * a.nseg) * nsplit;
     kern<<<(unsigned)blocks, kConvThreads, G::SMEM, n->stream>>>(*map, a);
     return cudaGetLastError() == cudaSuccess ? VOFP_OK : VOFP_ERR_CUDA;
 }
