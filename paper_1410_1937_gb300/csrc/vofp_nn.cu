@@ -47,6 +47,31 @@ __host__ __device__ __forceinline__ long long aidx(long long v, int c, long long
     return ((long long)(c >> 3) * V + v) * 8 + (c & 7);
 }
 
+// two neighbouring records with the same value, a whole 32-byte sector in one store
+__device__ __forceinline__ void store_twice(uint4* p, const uint4& v) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(p)), "r"(v.x), "r"(v.y),
+                 "r"(v.z), "r"(v.w)
+                 : "memory");
+}
+// eight channels of a voxel record
+__device__ __forceinline__ void unpack8(const uint4& u, float (&f)[8]) {
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        f[2 * h] = __uint_as_float(w[h] << 16);
+        f[2 * h + 1] = __uint_as_float(w[h] & 0xFFFF0000u);
+    }
+}
+__device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
+    uint32_t w[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        const __nv_bfloat162 p = __floats2bfloat162_rn(f[2 * h], f[2 * h + 1]);
+        w[h] = *reinterpret_cast<const uint32_t*>(&p);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // ---- 3x3x3 convolution on the tensor cores ---------------------------------------------------
 // Tile of one block: 8 voxels along x (one core-matrix row group) by 16 along y (M = 128 rows,
 // row m = voxel (m % 8, m / 8)); its input box is 10 x 18 voxels (one-voxel halo) of every input
@@ -99,7 +124,19 @@ struct ConvCfg {
     static_assert(TCOLS <= 512, "tensor memory");
 };
 
+// What the epilogue does with a finished plane besides storing it: the tensors that are only another layer's
+// pooled, upsampled or output form of it are written from registers, from the stored (rounded) values. As passes
+// of their own they took 640 us of a 3.22 ms forward pass at 512 x 256 x 128; it takes 2.77 ms so (2.89 with the
+// upsampled records stored by 16 bytes, half a sector, at a time).
+enum ConvThen { THEN_NOTHING = 0, THEN_UPSAMPLE = 1, THEN_POOL = 2, THEN_HEAD = 3 };
+struct ConvTail {
+    bf16* dst = nullptr;                  // upsampled (2nx, 2ny, 2nz) or pooled (nx/2, ny/2, nz/2) tensor
+    // output layer: out = mask (b + w . h) scale
+    const float *w = nullptr, *b = nullptr, *scale = nullptr, *mask = nullptr;
+    float* head = nullptr;
+};
 struct ConvArgs {
+    ConvTail tail;
     int nx, ny, nz;
     int tiles_x, tiles_y;
     int seg, nseg;            // planes per z segment, segments
@@ -129,7 +166,7 @@ __device__ __forceinline__ ConvSeg conv_seg(const ConvArgs& a, int u) {
     return g;
 }
 
-template <int CIN, int NOUT, int R>
+template <int CIN, int NOUT, int R, int THEN>
 __global__ void __launch_bounds__(kConvThreads, (ConvCfg<CIN, NOUT, R>::MINB))
 k_conv3_umma(const __grid_constant__ CUtensorMap in_map, const ConvArgs a) {
     using G = ConvCfg<CIN, NOUT, R>;
@@ -265,6 +302,15 @@ k_conv3_umma(const __grid_constant__ CUtensorMap in_map, const ConvArgs a) {
         const int q = warp & 3;
         const int m = q * 32 + lane;
         int o = 0;   // output planes so far
+        float below[THEN == THEN_POOL ? NOUT : 1];   // x and y sums of the even plane of a pair
+        (void)below;
+        float hw[THEN == THEN_HEAD ? NOUT : 1], hb = 0.f, hscale = 0.f;
+        if constexpr (THEN == THEN_HEAD) {
+#pragma unroll
+            for (int e = 0; e < NOUT; ++e) hw[e] = a.tail.w[e];
+            hb = a.tail.b[0];
+            hscale = a.tail.scale[0];
+        }
         for (int u = u0; u < units && !fail; u += du) {
             const ConvSeg g = conv_seg(a, u);
             const int xi = g.x0 + (m & 7), yi = g.y0 + (m >> 3);
@@ -290,25 +336,69 @@ k_conv3_umma(const __grid_constant__ CUtensorMap in_map, const ConvArgs a) {
                 umma::fence_before_sync();
                 __syncwarp();
                 if (lane == 0) umma::mbar_arrive(&acce[qb]);   // the columns may be used again
-                if (inside) {
-                    const long long vox = ((long long)(g.z0 + lz) * a.ny + yi) * a.nx + xi;
+                const long long vox = ((long long)(g.z0 + lz) * a.ny + yi) * a.nx + xi;
+                float hs = hb;
 #pragma unroll
-                    for (int oc = 0; oc < NOUT / 8; ++oc) {
-                        uint32_t w4[4];
+                for (int oc = 0; oc < NOUT / 8; ++oc) {
+                    uint32_t w4[4];
+                    const float* vv = v + oc * 8;
 #pragma unroll
-                        for (int h = 0; h < 4; ++h) {
-                            float lo = v[oc * 8 + 2 * h] + bsm[oc * 8 + 2 * h];
-                            float hi = v[oc * 8 + 2 * h + 1] + bsm[oc * 8 + 2 * h + 1];
-                            if (a.relu) {
-                                lo = fmaxf(lo, 0.f);
-                                hi = fmaxf(hi, 0.f);
-                            }
-                            const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
-                            w4[h] = *reinterpret_cast<const uint32_t*>(&p);
+                    for (int h = 0; h < 4; ++h) {
+                        float lo = vv[2 * h] + bsm[oc * 8 + 2 * h];
+                        float hi = vv[2 * h + 1] + bsm[oc * 8 + 2 * h + 1];
+                        if (a.relu) {
+                            lo = fmaxf(lo, 0.f);
+                            hi = fmaxf(hi, 0.f);
                         }
-                        const long long grp = a.out_chunk0 + (long long)split * (NOUT / 8) + oc;
-                        *reinterpret_cast<uint4*>(a.out + (grp * a.V + vox) * 8) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+                        const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
+                        w4[h] = *reinterpret_cast<const uint32_t*>(&p);
                     }
+                    const uint4 rec = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+                    const long long grp = a.out_chunk0 + (long long)split * (NOUT / 8) + oc;
+                    if (inside) *reinterpret_cast<uint4*>(a.out + (grp * a.V + vox) * 8) = rec;
+                    if constexpr (THEN == THEN_UPSAMPLE) {
+                        // the voxel's eight children
+                        if (inside) {
+                            bf16* to = a.tail.dst + ((long long)split * (NOUT / 8) + oc) * a.V * 64;
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                const long long row = (long long)(2 * (g.z0 + lz) + (c >> 1)) * 2 * a.ny + 2 * yi + (c & 1);
+                                uint4* p = reinterpret_cast<uint4*>(to + (row * 2 * a.nx + 2 * xi) * 8);
+                                store_twice(p, rec);
+                            }
+                        }
+                    }
+                    if constexpr (THEN == THEN_POOL) {
+                        // the mean of the stored values: x pairs are neighbouring lanes, y pairs eight apart
+                        float f[8];
+                        unpack8(rec, f);
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            f[e] += __shfl_xor_sync(0xffffffffu, f[e], 1);
+                            f[e] += __shfl_xor_sync(0xffffffffu, f[e], 8);
+                        }
+                        if (lz & 1) {
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) f[e] = (below[oc * 8 + e] + f[e]) * 0.125f;
+                            if (inside && (lane & 9) == 0) {
+                                const long long Vc = a.V / 8;
+                                const long long to = ((long long)((g.z0 + lz) >> 1) * (a.ny / 2) + (yi >> 1)) * (a.nx / 2) + (xi >> 1);
+                                *reinterpret_cast<uint4*>(a.tail.dst + (((long long)split * (NOUT / 8) + oc) * Vc + to) * 8) = pack8(f);
+                            }
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) below[oc * 8 + e] = f[e];
+                        }
+                    }
+                    if constexpr (THEN == THEN_HEAD) {
+                        float f[8];
+                        unpack8(rec, f);
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) hs = fmaf(hw[oc * 8 + e], f[e], hs);
+                    }
+                }
+                if constexpr (THEN == THEN_HEAD) {
+                    if (inside) a.tail.head[vox] = a.tail.mask[vox] * hs * hscale;
                 }
             }
         }
@@ -588,14 +678,6 @@ __global__ void k_relu_bwd(bf16* __restrict__ dy, const bf16* __restrict__ y, lo
         if (!(__bfloat162float(y[i]) > 0.f)) dy[i] = zero;
 }
 
-__device__ __forceinline__ void unpack8(const uint4& u, float (&f)[8]) {
-    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-        f[2 * h] = __uint_as_float(w[h] << 16);
-        f[2 * h + 1] = __uint_as_float(w[h] & 0xFFFF0000u);
-    }
-}
 // db[8 g + j] += sum over voxels of dy[v][8 g + j] (channel group g = blockIdx.y): one 16-byte
 // word (the group's 8 channels of a voxel) per thread and voxel, eight sums per thread, reduced
 // over the warp by shuffles and over the block in shared memory
@@ -626,43 +708,10 @@ __global__ void __launch_bounds__(256) k_bias_grad(const bf16* __restrict__ dy, 
     }
 }
 
-__device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
-    uint32_t w[4];
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-        const __nv_bfloat162 p = __floats2bfloat162_rn(f[2 * h], f[2 * h + 1]);
-        w[h] = *reinterpret_cast<const uint32_t*>(&p);
-    }
-    return make_uint4(w[0], w[1], w[2], w[3]);
-}
 __device__ __forceinline__ long long parent_voxel(long long v, int nx, int ny) {
     const int x = int(v % nx), y = int((v / nx) % ny);
     const long long z = v / ((long long)nx * ny);
     return ((z / 2) * (ny / 2) + y / 2) * (nx / 2) + x / 2;
-}
-
-// 2x2x2 average pooling of `groups` channel groups: (nx,ny,nz) -> (nx/2,ny/2,nz/2)
-__global__ void k_pool(const bf16* __restrict__ in, bf16* __restrict__ out, int nx, int ny, int nz, int groups) {
-    const int hx = nx / 2, hy = ny / 2, hz = nz / 2;
-    const long long Vf = (long long)nx * ny * nz, Vc = (long long)hx * hy * hz;
-    const uint4* src = reinterpret_cast<const uint4*>(in);
-    uint4* dst = reinterpret_cast<uint4*>(out);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < Vc * groups; i += (long long)gridDim.x * blockDim.x) {
-        const int k = int(i / Vc);
-        const long long v = i % Vc;
-        const int x = int(v % hx), y = int((v / hx) % hy), z = int(v / ((long long)hx * hy));
-        float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int q = 0; q < 8; ++q) {
-            const int xx = 2 * x + (q & 1), yy = 2 * y + ((q >> 1) & 1), zz = 2 * z + (q >> 2);
-            float f[8];
-            unpack8(src[k * Vf + ((long long)zz * ny + yy) * nx + xx], f);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) s[e] += f[e];
-        }
-#pragma unroll
-        for (int e = 0; e < 8; ++e) s[e] *= 0.125f;
-        dst[k * Vc + v] = pack8(s);
-    }
 }
 
 // gradient of the pooling, added into din (din += dout(parent) / 8), `groups` channel groups
@@ -680,17 +729,6 @@ __global__ void k_pool_bwd(const bf16* __restrict__ dout, bf16* __restrict__ din
 #pragma unroll
         for (int e = 0; e < 8; ++e) d[e] = accumulate ? d[e] + 0.125f * g[e] : 0.125f * g[e];
         dst[i] = pack8(d);
-    }
-}
-
-// nearest upsampling of `groups` coarse channel groups into the first groups of a fine tensor
-__global__ void k_upsample(const bf16* __restrict__ coarse, bf16* __restrict__ fine, int nx, int ny, int nz, int groups) {
-    const long long Vf = (long long)nx * ny * nz, Vc = Vf / 8;
-    const uint4* src = reinterpret_cast<const uint4*>(coarse);
-    uint4* dst = reinterpret_cast<uint4*>(fine);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < Vf * groups; i += (long long)gridDim.x * blockDim.x) {
-        const int k = int(i / Vf);
-        dst[i] = src[k * Vc + parent_voxel(i % Vf, nx, ny)];
     }
 }
 
@@ -895,22 +933,6 @@ __global__ void k_pack_input_dev(const bf16* __restrict__ geo, const float* __re
         x4[v] = u;
     }
 }
-__global__ void k_head_dev(const bf16* __restrict__ h, const float* __restrict__ w, const float* __restrict__ b,
-                           const float* scal, const float* __restrict__ mask, float* __restrict__ out, long long nv) {
-    const float scale = scal[2];
-    const uint4* h4 = reinterpret_cast<const uint4*>(h);
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nv; v += (long long)gridDim.x * blockDim.x) {
-        float f0[8], f1[8];
-        unpack8(h4[v], f0);
-        unpack8(h4[nv + v], f1);
-        float s = b[0];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) s = fmaf(w[c], f0[c], s);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) s = fmaf(w[8 + c], f1[c], s);
-        out[v] = mask[v] * s * scale;
-    }
-}
 __global__ void k_head_bwd_dev(const bf16* __restrict__ h, const float* __restrict__ w, const float* __restrict__ out,
                                const float* __restrict__ target, const float* __restrict__ mask, float* scal,
                                bf16* __restrict__ dh, float* __restrict__ dw, float* __restrict__ db, long long nv) {
@@ -1060,10 +1082,10 @@ vofp_status wgrad_umma(vofp_nn* n, const CUtensorMap* xm, const CUtensorMap* dm,
     return cudaGetLastError() == cudaSuccess ? VOFP_OK : VOFP_ERR_CUDA;
 }
 
-template <int CIN, int NOUT, int R>
+template <int CIN, int NOUT, int R, int THEN = THEN_NOTHING>
 vofp_status conv_umma(vofp_nn* n, const CUtensorMap* map, ConvArgs a, int nsplit) {
     using G = ConvCfg<CIN, NOUT, R>;
-    auto kern = k_conv3_umma<CIN, NOUT, R>;
+    auto kern = k_conv3_umma<CIN, NOUT, R, THEN>;
     static bool ready = false;   // (per instantiation; one device per process)
     if (!ready) {
         int occ = 0;
@@ -1103,7 +1125,8 @@ vofp_status conv_umma(vofp_nn* n, const CUtensorMap* map, ConvArgs a, int nsplit
 // channels in blocks of nout): the layer's forward weights, or its data-gradient weights (taps
 // mirrored, channels transposed; no bias, no ReLU).
 vofp_status conv(vofp_nn* n, const bf16* in, int cin, const bf16* blob, int cout, int nout, const float* bias,
-                 bool relu, bf16* out, int out_chunk0, int nx, int ny, int nz) {
+                 bool relu, bf16* out, int out_chunk0, int nx, int ny, int nz, int then = THEN_NOTHING,
+                 const ConvTail& tail = ConvTail()) {
     const CUtensorMap* map = act_map(n, in, nx, ny, nz, cin / 8);
     if (!map) {
         n->err = "tensor map of an activation could not be built";
@@ -1121,8 +1144,14 @@ vofp_status conv(vofp_nn* n, const bf16* in, int cin, const bf16* blob, int cout
     a.wblob = blob;
     a.out = out;
     a.out_chunk0 = out_chunk0;
+    a.tail = tail;
     const int ns = cout / nout;
-    switch (cin * 1000 + nout) {
+    switch (then * 1000000 + cin * 1000 + nout) {
+        case THEN_UPSAMPLE * 1000000 + 32032: return conv_umma<32, 32, 4, THEN_UPSAMPLE>(n, map, a, ns);
+        case THEN_UPSAMPLE * 1000000 + 64032: return conv_umma<64, 32, 4, THEN_UPSAMPLE>(n, map, a, ns);
+        case THEN_POOL * 1000000 + 16016: return conv_umma<16, 16, 4, THEN_POOL>(n, map, a, ns);
+        case THEN_POOL * 1000000 + 32032: return conv_umma<32, 32, 4, THEN_POOL>(n, map, a, ns);
+        case THEN_HEAD * 1000000 + 16016: return conv_umma<16, 16, 4, THEN_HEAD>(n, map, a, ns);
         case 16016: return conv_umma<16, 16, 4>(n, map, a, ns);
         case 16032: return conv_umma<16, 32, 4>(n, map, a, ns);
         case 16048: return conv_umma<16, 48, 4>(n, map, a, ns);
@@ -1137,8 +1166,9 @@ vofp_status conv(vofp_nn* n, const bf16* in, int cin, const bf16* blob, int cout
     }
 }
 
-vofp_status conv_fwd(vofp_nn* n, const Layer& l, const bf16* in, bf16* out, int out_chunk0, int nx, int ny, int nz) {
-    return conv(n, in, l.cin, l.blob_f, l.cout, l.nout_f, l.b, true, out, out_chunk0, nx, ny, nz);
+vofp_status conv_fwd(vofp_nn* n, const Layer& l, const bf16* in, bf16* out, int out_chunk0, int nx, int ny, int nz,
+                     int then = THEN_NOTHING, const ConvTail& tail = ConvTail()) {
+    return conv(n, in, l.cin, l.blob_f, l.cout, l.nout_f, l.b, true, out, out_chunk0, nx, ny, nz, then, tail);
 }
 
 // weight and bias gradients of one layer from its input x and the gradient dy of its output
@@ -1203,21 +1233,29 @@ vofp_status forward(vofp_nn* n, const float* r) {
     k_pack_input_dev<<<gs(n->V1), 256, 0, st>>>(n->geo, r, n->scal, n->x0, n->V1);
     auto& L = n->L;
     vofp_status s;
-    if ((s = conv_fwd(n, L[0], n->x0, n->a1, 0, X, Y, Z)) || (s = conv_fwd(n, L[1], n->a1, n->c1, 4, X, Y, Z)))
+    // pooled, upsampled and output tensors come with the convolution before them
+    auto to = [](bf16* dst) {
+        ConvTail t;
+        t.dst = dst;
+        return t;
+    };
+    ConvTail head;
+    head.w = n->hw;
+    head.b = n->hb;
+    head.scale = n->scal + 2;
+    head.mask = n->mask;
+    head.head = n->out;
+    if ((s = conv_fwd(n, L[0], n->x0, n->a1, 0, X, Y, Z)) ||
+        (s = conv_fwd(n, L[1], n->a1, n->c1, 4, X, Y, Z, THEN_POOL, to(n->p1))) ||
+        (s = conv_fwd(n, L[2], n->p1, n->a2, 0, X2, Y2, Z2)) ||
+        (s = conv_fwd(n, L[3], n->a2, n->c2, 8, X2, Y2, Z2, THEN_POOL, to(n->p2))) ||
+        (s = conv_fwd(n, L[4], n->p2, n->a3, 0, X4, Y4, Z4)) ||
+        (s = conv_fwd(n, L[5], n->a3, n->b3, 0, X4, Y4, Z4, THEN_UPSAMPLE, to(n->c2))) ||
+        (s = conv_fwd(n, L[6], n->c2, n->d2a, 0, X2, Y2, Z2)) ||
+        (s = conv_fwd(n, L[7], n->d2a, n->d2b, 0, X2, Y2, Z2, THEN_UPSAMPLE, to(n->c1))) ||
+        (s = conv_fwd(n, L[8], n->c1, n->d1a, 0, X, Y, Z)) ||
+        (s = conv_fwd(n, L[9], n->d1a, n->d1b, 0, X, Y, Z, THEN_HEAD, head)))
         return s;
-    k_pool<<<gs(n->V2 * 2), 256, 0, st>>>(n->s1, n->p1, X, Y, Z, 2);
-    if ((s = conv_fwd(n, L[2], n->p1, n->a2, 0, X2, Y2, Z2)) || (s = conv_fwd(n, L[3], n->a2, n->c2, 8, X2, Y2, Z2)))
-        return s;
-    k_pool<<<gs(n->V3 * 4), 256, 0, st>>>(n->s2, n->p2, X2, Y2, Z2, 4);
-    if ((s = conv_fwd(n, L[4], n->p2, n->a3, 0, X4, Y4, Z4)) || (s = conv_fwd(n, L[5], n->a3, n->b3, 0, X4, Y4, Z4)))
-        return s;
-    k_upsample<<<gs(n->V2 * 8), 256, 0, st>>>(n->b3, n->c2, X2, Y2, Z2, 8);
-    if ((s = conv_fwd(n, L[6], n->c2, n->d2a, 0, X2, Y2, Z2)) || (s = conv_fwd(n, L[7], n->d2a, n->d2b, 0, X2, Y2, Z2)))
-        return s;
-    k_upsample<<<gs(n->V1 * 4), 256, 0, st>>>(n->d2b, n->c1, X, Y, Z, 4);
-    if ((s = conv_fwd(n, L[8], n->c1, n->d1a, 0, X, Y, Z)) || (s = conv_fwd(n, L[9], n->d1a, n->d1b, 0, X, Y, Z)))
-        return s;
-    k_head_dev<<<gs(n->V1), 256, 0, st>>>(n->d1b, n->hw, n->hb, n->scal, n->mask, n->out, n->V1);
     return check_err(n);
 }
 
@@ -1385,8 +1423,8 @@ vofp_status forward_on(vofp_nn* n, cudaStream_t st, const float* r) {
     return s;
 }
 float* output(vofp_nn* n) { return n->out; }
-// rms, its finish, input packing, ten convolutions, two poolings, two upsamplings, output layer
-int forward_kernels(const vofp_nn*) { return 18; }
+// rms, its finish, input packing, ten convolutions
+int forward_kernels(const vofp_nn*) { return 13; }
 vofp_status read_device_error(vofp_nn* n) { return read_err(n); }
 vofp_status train_from_grad_on(vofp_nn* n, cudaStream_t st, const float* dz, float lr, int update) {
     const cudaStream_t own = n->stream;
