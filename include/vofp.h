@@ -132,7 +132,7 @@ typedef struct {
  *               The network's steps continue while the inner residual norm falls at least to
  *               stag_ratio of its value stag_window iterations before; otherwise (or on a
  *               breakdown) the solve hands over to VOFP_MODE_MIXED (precond as given) from the
- *               current iterate.  A network application costs about as much as 30-40 iterations
+ *               current iterate.  A network application costs about as much as 25 iterations
  *               of the mixed red-black solve, so the defaults (window 2, ratio 0.6) keep it only
  *               while it beats those.
  *   stag_window, stag_ratio  the hand-over test above (0 selects the defaults; window <= 63). */
