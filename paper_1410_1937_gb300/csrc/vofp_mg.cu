@@ -21,8 +21,8 @@
 //
 // Merge groups: the group's unknown is present at every member cell of the expanded vectors.  Its
 // master represents it in the restriction (weight sq); the other members, small cells whose own
-// aggregate may have next to no coupling, carry weight -1: left out of the sums and given the
-// master's z.  On the compact vectors an even-parity master sits after the N/2 pairs; a mask byte per
+// aggregate may have next to no coupling, carry weight -1 like the red cells of the full-grid vectors:
+// left out of the sums, and given the master's z.  On the compact vectors an even-parity master sits after the N/2 pairs; a mask byte per
 // aggregate says which of its four even cells are such masters.
 //
 // Everything is gathered (no floating-point atomics), so a solve is bitwise reproducible.
@@ -148,8 +148,10 @@ __global__ void k_mg_dinv(int nx, int ny, int nz, const T* __restrict__ tx, cons
     }
 }
 
-// weights of the vector entries (before the merge groups): sq of a non-red cell with an unknown, 0
-// of the others; on the compact vectors entries past N/2 belong to group members (-1)
+// weights of the vector entries (before the merge groups): sq of a non-red cell with an unknown, 0 of one
+// without, -1 (in no sum; z stays 0) of a red one: the iteration kernel writes no row there, so q holds
+// whatever the passes before the loop left, and with a starting pressure those are rounding errors that r
+// gathers in every iteration.  On the compact vectors entries past N/2 belong to group members (-1)
 template <bool COMPACT, typename T>
 __global__ void k_mg_weights(Dims d, long long n, long long nh, const double* __restrict__ sq,
                              const int32_t* __restrict__ root, const uint32_t* __restrict__ red,
@@ -166,7 +168,7 @@ __global__ void k_mg_weights(Dims d, long long n, long long nh, const double* __
             const long long c = 2 * t + 1 - ((j + k) & 1);   // black cell of pair t
             w[t] = root[c] < 0 ? T(0) : (T)(sq[c] * g);
         } else {
-            w[t] = (root[t] < 0 || is_slave(red, t)) ? T(0) : (T)(sq[t] * g);
+            w[t] = is_slave(red, t) ? T(-1) : root[t] < 0 ? T(0) : (T)(sq[t] * g);
         }
     }
 }
