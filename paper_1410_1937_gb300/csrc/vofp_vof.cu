@@ -54,6 +54,8 @@ int grid_cells(long long n) {
 
 // ---- fluid volume below a plane in a box -------------------------------------------------------
 
+__device__ __forceinline__ uint32_t high_abs(double v) { return (uint32_t)__double2hiint(v) & 0x7fffffffu; }
+
 __device__ __forceinline__ void sort3(double& a, double& b, double& c) {
     if (a > b) { const double t = a; a = b; b = t; }
     if (b > c) { const double t = b; b = c; c = t; }
@@ -61,7 +63,9 @@ __device__ __forceinline__ void sort3(double& a, double& b, double& c) {
 }
 
 // fraction of the unit cube in {a.y <= alpha} (any signs), region by region in forms that divide by the
-// smallest component only where the region's width is that component
+// smallest component only where the region's width is that component.  a is of the size of the gradient of
+// phi: where products of two components would leave the range of FP64 (fractions of 1e-162 all around), a and
+// alpha are scaled by a power of two first, which changes nothing else
 __device__ double cube_fraction(double a1, double a2, double a3, double alpha) {
     // reflect negative components (y -> 1 - y)
     if (a1 < 0.0) alpha -= a1;
@@ -73,7 +77,14 @@ __device__ double cube_fraction(double a1, double a2, double a3, double alpha) {
     if (alpha >= s) return 1.0;
     sort3(c1, c2, c3);
     const bool flip = alpha > 0.5 * s;
-    const double b = flip ? s - alpha : alpha;
+    double b = flip ? s - alpha : alpha;
+    if ((high_abs(c3) >> 20) - 723u >= 600u) {   // c3 outside 2^-300 .. 2^300
+        const int e = isfinite(c3) ? -ilogb(c3) : 0;
+        c1 = scalbn(c1, e);
+        c2 = scalbn(c2, e);
+        c3 = scalbn(c3, e);
+        b = scalbn(b, e);
+    }
     double num, den = c2 * c3;   // f = num / den
     if (b < c1) {
         num = (b * (b / c1)) * (b / 6.0);
@@ -151,8 +162,6 @@ __device__ __forceinline__ double span(const double* __restrict__ w, int i, int 
     const double wp = i > 0 ? w[i - 1] : w[i], wn = i < n - 1 ? w[i + 1] : w[i];
     return 0.5 * wp + w[i] + 0.5 * wn;
 }
-
-__device__ __forceinline__ uint32_t high_abs(double v) { return (uint32_t)__double2hiint(v) & 0x7fffffffu; }
 
 // Per axis: 1 / width, -1/16 over the distance of a cell's two neighbours' centres, and the high word of 0.49 width / dt, the least of a cell and its two neighbours: a
 // velocity whose high word is below it moves less than half a donor cell (false for NaN)
