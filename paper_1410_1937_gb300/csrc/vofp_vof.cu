@@ -62,10 +62,31 @@ __device__ __forceinline__ void sort3(double& a, double& b, double& c) {
     if (a > b) { const double t = a; a = b; b = t; }
 }
 
-// fraction of the unit cube in {a.y <= alpha} (any signs), region by region in forms that divide by the
-// smallest component only where the region's width is that component.  a is of the size of the gradient of
-// phi: where products of two components would leave the range of FP64 (fractions of 1e-162 all around), a and
-// alpha are scaled by a power of two first, which changes nothing else
+// Fraction of the unit cube in {c.y <= b} for 0 <= c1 <= c2 <= c3 and 0 < b <= (c1 + c2 + c3) / 2 as a quotient,
+// region by region in forms that divide by the smallest component only where the region's width is that component.
+__device__ __forceinline__ double region_fraction(double c1, double c2, double c3, double b, double& den) {
+    den = c2 * c3;
+    if (b < c1) return (b * (b / c1)) * (b / 6.0);
+    if (b < c2) return 0.5 * fma(b, b - c1, c1 * c1 * (1.0 / 3.0));
+    const double c12 = c1 + c2, p1 = fma(3.0 * b, b - c1, c1 * c1), e2 = b - c2;
+    if (b < fmin(c12, c3)) return fma(-e2 * (e2 / c1), e2, p1) * (1.0 / 6.0);
+    if (c3 < c12) {
+        const double e3 = b - c3;
+        return fma(-e3 * (e3 / c1), e3, fma(-e2 * (e2 / c1), e2, p1)) * (1.0 / 6.0);
+    }
+    den = 2.0 * c3;
+    return 2.0 * b - c12;
+}
+// the same where the denominator would leave the range of FP64: scaled by a power of two, which changes nothing else
+__device__ __noinline__ double scaled_fraction(double c1, double c2, double c3, double b) {
+    const int e = isfinite(c3) ? -ilogb(c3) : 0;
+    double den;
+    const double num = region_fraction(scalbn(c1, e), scalbn(c2, e), scalbn(c3, e), scalbn(b, e), den);
+    return num / den;
+}
+
+// fraction of the unit cube in {a.y <= alpha} (any signs).  a is of the size of the gradient of phi, which is
+// 1e-162 and less where all fractions around are.
 __device__ double cube_fraction(double a1, double a2, double a3, double alpha) {
     // reflect negative components (y -> 1 - y)
     if (a1 < 0.0) alpha -= a1;
@@ -77,32 +98,11 @@ __device__ double cube_fraction(double a1, double a2, double a3, double alpha) {
     if (alpha >= s) return 1.0;
     sort3(c1, c2, c3);
     const bool flip = alpha > 0.5 * s;
-    double b = flip ? s - alpha : alpha;
-    if ((high_abs(c3) >> 20) - 723u >= 600u) {   // c3 outside 2^-300 .. 2^300
-        const int e = isfinite(c3) ? -ilogb(c3) : 0;
-        c1 = scalbn(c1, e);
-        c2 = scalbn(c2, e);
-        c3 = scalbn(c3, e);
-        b = scalbn(b, e);
-    }
-    double num, den = c2 * c3;   // f = num / den
-    if (b < c1) {
-        num = (b * (b / c1)) * (b / 6.0);
-    } else if (b < c2) {
-        num = 0.5 * fma(b, b - c1, c1 * c1 * (1.0 / 3.0));
-    } else {
-        const double c12 = c1 + c2, p1 = fma(3.0 * b, b - c1, c1 * c1), e2 = b - c2;
-        if (b < fmin(c12, c3)) {
-            num = fma(-e2 * (e2 / c1), e2, p1) * (1.0 / 6.0);
-        } else if (c3 < c12) {
-            const double e3 = b - c3;
-            num = fma(-e3 * (e3 / c1), e3, fma(-e2 * (e2 / c1), e2, p1)) * (1.0 / 6.0);
-        } else {
-            num = 2.0 * b - c12;
-            den = 2.0 * c3;
-        }
-    }
-    const double f = num / den;
+    const double b = flip ? s - alpha : alpha;
+    double den;
+    const double num = region_fraction(c1, c2, c3, b, den);
+    // outside 2^-900 .. 2^900
+    const double f = (high_abs(den) >> 20) - 123u >= 1800u ? scaled_fraction(c1, c2, c3, b) : num / den;
     return flip ? 1.0 - f : f;
 }
 
@@ -155,6 +155,32 @@ struct CubeFrac {
         return flip ? T(1) - f : f;
     }
 };
+
+// The root b of volume(b) = pc for a fraction pc below rounding, a_i and their sum unscaled: in FP64 and from
+// below, as the volume is at most that of each region's formula with the other faces left out and, for a small
+// fraction, near one of the three.  (In line it cost k_vof_plic 8 of 159 us at 512x256x128, as a call 3.)
+__device__ __noinline__ double vanishing_root(double a1, double a2, double a3, double sum, double pc) {
+    if (sum < 0x1p-1000) {   // its reciprocal would overflow
+        a1 *= 0x1p200;
+        a2 *= 0x1p200;
+        a3 *= 0x1p200;
+        sum *= 0x1p200;
+    }
+    const double is = 1.0 / sum;
+    const CubeFrac<double> f(a1 * is, a2 * is, a3 * is);
+    double lo = 0.0, hi = 1.0, dv;
+    double b = fmax(cbrt(6.0 * f.c1 * f.c2 * f.c3 * pc), fmax(sqrt(2.0 * f.c2 * f.c3 * pc), f.c3 * pc));
+    for (int it = 0; it < 100; ++it) {
+        const double res = f(b, &dv) - pc;
+        if (res == 0.0) break;
+        if (res < 0.0) lo = b;
+        else hi = b;
+        const double nb = dv > 0.0 ? b - res / dv : 2.0;
+        if (fabs(nb - b) <= 1e-9 * b) return nb;
+        b = nb > lo && nb < hi ? nb : 0.5 * (lo + hi);
+    }
+    return b;
+}
 
 // ---- per-call tables and the interface list -----------------------------------------------------
 
@@ -291,48 +317,53 @@ k_vof_plic(Dims d, const double* __restrict__ dx, const double* __restrict__ dy,
         const double sum = (a1 + a2) + a3;
         double alpha = 0.0;
         if (sum > 0.0) {
-            const double is = 1.0 / sum;
-            a1 *= is;
-            a2 *= is;
-            a3 *= is;
-            // FP32 first (its result only starts the FP64 search)
-            double b = pc;
-            {
-                const CubeFrac<float> f((float)a1, (float)a2, (float)a3);
-                const float p = (float)pc;
-                float lo = 0.0f, hi = 1.0f, x = p;
-                for (int it = 0; it < 24; ++it) {
-                    float dv;
-                    const float res = f(x, &dv) - p;
-                    if (res == 0.0f) break;
-                    if (res < 0.0f) lo = x;
-                    else hi = x;
-                    float nx = dv > 0.0f ? x - res / dv : 0.5f * (lo + hi);
-                    if (!(nx > lo && nx < hi)) nx = 0.5f * (lo + hi);
-                    const float step = fabsf(nx - x);
-                    x = nx;
-                    if (step <= 2e-7f * x) break;
+            double b;
+            if (high_abs(pc) < 0x3a200000u) {   // 2^-93: the FP32 quotient below would lose its residual
+                b = vanishing_root(a1, a2, a3, sum, pc);
+            } else {
+                const double is = 1.0 / sum;
+                a1 *= is;
+                a2 *= is;
+                a3 *= is;
+                // FP32 first (its result only starts the FP64 search)
+                b = pc;
+                {
+                    const CubeFrac<float> f((float)a1, (float)a2, (float)a3);
+                    const float p = (float)pc;
+                    float lo = 0.0f, hi = 1.0f, x = p;
+                    for (int it = 0; it < 24; ++it) {
+                        float dv;
+                        const float res = f(x, &dv) - p;
+                        if (res == 0.0f) break;
+                        if (res < 0.0f) lo = x;
+                        else hi = x;
+                        float nx = dv > 0.0f ? x - res / dv : 0.5f * (lo + hi);
+                        if (!(nx > lo && nx < hi)) nx = 0.5f * (lo + hi);
+                        const float step = fabsf(nx - x);
+                        x = nx;
+                        if (step <= 2e-7f * x) break;
+                    }
+                    if (x > 0.0f && x < 1.0f) b = (double)x;
                 }
-                if (x > 0.0f && x < 1.0f) b = (double)x;
-            }
-            const CubeFrac<double> f(a1, a2, a3);
-            double lo = 0.0, hi = 1.0;
-            for (int it = 0; it < 100; ++it) {
-                double dv;
-                const double res = f(b, &dv) - pc;
-                if (res == 0.0) break;
-                if (res < 0.0) lo = b;
-                else hi = b;
-                // the quotient in FP32: a Newton step is right to 1e-7 of itself, and as an error of e becomes
-                // one of about e^2 / min(b, 1 - b), one of at most 1e-9 of that leaves an error below its
-                // rounding and ends the search; a step that leaves the bracket becomes a bisection
-                const double step = dv > 0.0 ? (double)((float)res / (float)dv) : 2.0;
-                const double nb = b - step;
-                if (fabs(step) <= 1e-9 * fmin(b, 1.0 - b)) {
-                    b = nb;
-                    break;
+                const CubeFrac<double> f(a1, a2, a3);
+                double lo = 0.0, hi = 1.0;
+                for (int it = 0; it < 100; ++it) {
+                    double dv;
+                    const double res = f(b, &dv) - pc;
+                    if (res == 0.0) break;
+                    if (res < 0.0) lo = b;
+                    else hi = b;
+                    // the quotient in FP32: a Newton step is right to 1e-7 of itself, and as an error of e becomes
+                    // one of about e^2 / min(b, 1 - b), one of at most 1e-9 of that leaves an error below its
+                    // rounding and ends the search; a step that leaves the bracket becomes a bisection
+                    const double step = dv > 0.0 ? (double)((float)res / (float)dv) : 2.0;
+                    const double nb = b - step;
+                    if (fabs(step) <= 1e-9 * fmin(b, 1.0 - b)) {
+                        b = nb;
+                        break;
+                    }
+                    b = nb > lo && nb < hi ? nb : 0.5 * (lo + hi);
                 }
-                b = nb > lo && nb < hi ? nb : 0.5 * (lo + hi);
             }
             alpha = lo0 + b * sum;
         }
