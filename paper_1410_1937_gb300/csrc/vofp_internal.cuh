@@ -226,7 +226,7 @@ struct vofp_ctx {
     // coarse-grid correction of the red-black solves (vofp_mg.cu)
     vofp::MgSet<float> mgf;           // mixed mode
     vofp::MgSet<double> mgd;          // FP64 mode
-    bool mg_use = false;              // in use in the current solve
+    bool mg_use = false;              // in use in the current solve (set by each; means nothing outside one)
     uint32_t* mg_mask = nullptr;      // per aggregate (a byte): its even cells that are group masters
     int* mg_even = nullptr;           // their entries, four per aggregate
     unsigned long long* mg_dmax = nullptr;

@@ -639,13 +639,12 @@ void rbc_prep(vofp_ctx* c, cudaStream_t st, const double* rhs) {
 }
 
 namespace {
+// src: the direction's source, z with the coarse-grid correction, r without
 template <int RPT>
-void launch_main_t(vofp_ctx* c, cudaStream_t st, const float* po, float* pn, bool pdl) {
+void launch_main_t(vofp_ctx* c, cudaStream_t st, const float* src, const float* po, float* pn, bool pdl) {
     using G = RbcGeomT<RPT>;
     const Dims d = c->d;
     const int nh = d.nx / 2;
-    // the direction's source: z with the coarse-grid correction, r without
-    const float* src = c->mg_use ? c->mgf.z : c->rbc_r;
     const CUtensorMap *mr = tensor_map_f32_x(c, src, nh, G::BWC, G::TH + 4),
                       *mp = tensor_map_f32_x(c, po, nh, G::BWC, G::TH + 4),
                       *mx = tensor_map_f32(c, c->Txf, G::BWF, G::TH + 2),
@@ -667,11 +666,11 @@ void launch_main_t(vofp_ctx* c, cudaStream_t st, const float* po, float* pn, boo
                cg_rbc_smem<kRbcStages, RPT>(), st, maps, d, c->rbc_split, ex, po, pn, c->rbc_x, c->rbc_q,
                c->sc, c->partials + kPqBase);
 }
-void launch_main(vofp_ctx* c, cudaStream_t st, const float* po, float* pn, bool pdl) {
+void launch_main(vofp_ctx* c, cudaStream_t st, const float* src, const float* po, float* pn, bool pdl) {
     if (c->rbc_rpt == 1)
-        launch_main_t<1>(c, st, po, pn, pdl);
+        launch_main_t<1>(c, st, src, po, pn, pdl);
     else
-        launch_main_t<2>(c, st, po, pn, pdl);
+        launch_main_t<2>(c, st, src, po, pn, pdl);
 }
 }  // namespace
 
@@ -707,7 +706,7 @@ void rbc_iteration(vofp_ctx* c, cudaStream_t st, const float* po, float* pn, cud
     // only, 388.2 ms without the chaining, measured with a separate exception kernel). The
     // host-driven loop launches them as ordinary kernels.
     const bool pdl = c->pdl != 0 && use_h != 0;
-    launch_main(c, st, po, pn, pdl);
+    launch_main(c, st, c->mg_use ? c->mgf.z : c->rbc_r, po, pn, pdl);
     rbc_aux(c, st, po, pn, pdl);
     if (c->mg_use) {
         mg_update(c, st, false, pdl, h, use_h, rbc_pq_parts(c));
@@ -731,8 +730,8 @@ void rbc_finish_xf(vofp_ctx* c, cudaStream_t st) {
                (const float*)c->rbc_x, (const float*)c->rbc_p0, c->xf, (const CgScalars*)c->sc);
 }
 
-// timed as ordinary launches, one kernel after the other
-void rbc_time_kernel(vofp_ctx* c, cudaStream_t st) { launch_main(c, st, c->rbc_p0, c->rbc_p1, false); }
+// timed as ordinary launches, one kernel after the other (from r, whatever the last solve iterated on)
+void rbc_time_kernel(vofp_ctx* c, cudaStream_t st) { launch_main(c, st, c->rbc_r, c->rbc_p0, c->rbc_p1, false); }
 void rbc_time_aux(vofp_ctx* c, cudaStream_t st) { rbc_aux(c, st, c->rbc_p0, c->rbc_p1, false); }
 
 }  // namespace vofp
