@@ -105,7 +105,9 @@ typedef struct {
  *               (Eisenstat's form); both modes, and the bench default in mixed mode).  From 2^16
  *               cells and for rtol <= 1e-7 its CG also has a coarse-grid correction: an additive
  *               V-cycle on 2x2x2 aggregates smoothed by red-black Gauss-Seidel (in the precision
- *               of the iteration's vectors).
+ *               of the iteration's vectors).  It takes 10 to 12 bytes per cell in mixed mode and 24 in
+ *               FP64 mode, allocated on the first such solve and kept by the context; an operator
+ *               for which that memory cannot be had is solved without the correction.
  *   rtol        the solve returns VOFP_OK only when the residual recomputed from the returned x,
  *               ||b_hat - A_hat x|| (2-norm over the unknowns, FP64), is at most rtol ||b_hat||.
  *               The iteration aims slightly below rtol; when the recomputed residual is still

@@ -2,7 +2,9 @@
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <algorithm>
 #include <cstdint>
+#include <iterator>
 #include <map>
 #include <string>
 #include <tuple>
@@ -247,6 +249,17 @@ struct vofp_ctx {
         bytes += sizeof(T) * count;
         *p = reinterpret_cast<T*>(q);
         return VOFP_OK;
+    }
+    // give back what alloc gave for `count` values (null: nothing), and the tensor maps of it
+    template <typename T>
+    void release(T** p, size_t count) {
+        if (!*p) return;
+        cudaFree(*p);
+        allocs.erase(std::remove(allocs.begin(), allocs.end(), (void*)*p), allocs.end());
+        bytes -= sizeof(T) * count;
+        for (auto it = tma_maps.begin(); it != tma_maps.end();)
+            it = std::get<0>(it->first) == (const void*)*p ? tma_maps.erase(it) : std::next(it);
+        *p = nullptr;
     }
 };
 

@@ -833,6 +833,21 @@ void launch_update(vofp_ctx* c, cudaStream_t st, bool pdl, cudaGraphConditionalH
                (const double*)(c->partials + kPqBase), npq);
 }
 
+// give back a hierarchy's memory
+template <typename T>
+void drop(vofp_ctx* c, MgSet<T>& m) {
+    for (MgLevel<T>& l : m.lv)
+        for (T** p : {&l.tx, &l.ty, &l.tz, &l.di, &l.ex, &l.b, &l.x}) c->release(p, l.n);
+    if (sizeof(T) == 4 && !m.lv.empty()) {
+        c->release(&c->mg_mask, (m.lv[0].n + 3) / 4);
+        c->release(&c->mg_even, 4 * m.lv[0].n);
+    }
+    c->release(&m.w, m.cap);
+    c->release(&m.z, m.cap);
+    c->release(&m.rep, 2 * m.rep_cap);
+    m = MgSet<T>();
+}
+
 // The hierarchy and the weights of the current operator (once per operator and precision).
 template <bool COMPACT, typename T>
 vofp_status build(vofp_ctx* c) {
@@ -841,7 +856,6 @@ vofp_status build(vofp_ctx* c) {
     cudaStream_t st = c->stream;
     vofp_status s;
     if (m.lv.empty()) {
-        std::vector<MgLevel<T>> v;
         int nx = d.nx, ny = d.ny, nz = d.nz;
         do {
             MgLevel<T> l{};
@@ -849,12 +863,12 @@ vofp_status build(vofp_ctx* c) {
             l.ny = ny = (ny + 1) / 2;
             l.nz = nz = (nz + 1) / 2;
             l.n = (long long)nx * ny * nz;
+            m.lv.push_back(l);
+        } while (m.lv.back().n > 1);
+        for (MgLevel<T>& l : m.lv)
             for (T** p : {&l.tx, &l.ty, &l.tz, &l.di, &l.ex, &l.b, &l.x})
                 if ((s = c->alloc(p, l.n))) return s;
-            v.push_back(l);
-        } while (v.back().n > 1);
         if (!c->mg_dmax && (s = c->alloc(&c->mg_dmax, 1))) return s;
-        m.lv = v;
     }
     const MgLevel<T>& l1 = m.lv[0];
     if (COMPACT) {
@@ -866,14 +880,13 @@ vofp_status build(vofp_ctx* c) {
     const long long nv = COMPACT ? c->rbc_cap : d.n;
     if (nv > m.cap) {
         // entries past the vectors in use stay 0 (the tensor copies read whole boxes)
-        if ((s = c->alloc(&m.w, nv)) || (s = c->alloc(&m.z, nv))) return s;
         m.cap = nv;
+        if ((s = c->alloc(&m.w, nv)) || (s = c->alloc(&m.z, nv))) return s;
     }
     VOFP_CUDA_TRY(c, cudaMemsetAsync(m.z, 0, sizeof(T) * m.cap, st));
     if (c->ngroups > m.rep_cap) {
-        const long long cap = c->ngroups + c->ngroups / 2 + 64;
-        if ((s = c->alloc(&m.rep, 2 * cap))) return s;
-        m.rep_cap = cap;
+        m.rep_cap = c->ngroups + c->ngroups / 2 + 64;
+        if ((s = c->alloc(&m.rep, 2 * m.rep_cap))) return s;
     }
     VOFP_CUDA_TRY(c, cudaMemsetAsync(c->mg_dmax, 0, sizeof(unsigned long long), st));
     launch(c, k_mg_max, grid_n(d.n), kNT, st, d.n, (const double*)c->diag, c->mg_dmax);
@@ -919,12 +932,25 @@ bool mg_wanted(const vofp_ctx* c, double rtol) {
     return use == 2 || (use != 0 && c->d.n >= kMgMinCells && rtol <= kMgMaxRtol);
 }
 
+// Where there is no memory for the hierarchy the solves of this operator are plain ones (ok stays false), and
+// what was allocated is given back.
 vofp_status mg_ensure(vofp_ctx* c, bool fp64) {
     bool& built = fp64 ? c->mgd.built : c->mgf.built;
     if (built) return VOFP_OK;
-    built = true;
     (fp64 ? c->mgd.ok : c->mgf.ok) = false;
-    return fp64 ? build<false, double>(c) : c->rbc_ok ? build<true, float>(c) : build<false, float>(c);
+    const vofp_status s = fp64 ? build<false, double>(c) : c->rbc_ok ? build<true, float>(c) : build<false, float>(c);
+    if (s == VOFP_ERR_OOM) {
+        cudaGetLastError();   // (the refused allocation's)
+        c->err.clear();
+        if (fp64)
+            drop(c, c->mgd);
+        else
+            drop(c, c->mgf);
+    } else if (s) {
+        return s;
+    }
+    built = true;
+    return VOFP_OK;
 }
 
 // b_1 (at the start of a loop: from the new residual), the V-cycle, z, r.z and beta

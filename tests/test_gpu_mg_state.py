@@ -1,5 +1,10 @@
 """What a solve with the coarse-grid correction leaves in its context, and what it does where the correction cannot
 be had (csrc/vofp_mg.cu)."""
+import os
+import subprocess
+import sys
+import textwrap
+
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -7,6 +12,7 @@ torch = pytest.importorskip("torch")
 from paper_1410_1937_gb300 import inputs as I
 
 pytestmark = pytest.mark.gpu
+HERE = os.path.dirname(os.path.abspath(__file__))
 
 
 @pytest.fixture(scope="module")
@@ -38,3 +44,57 @@ def test_kernel_timing_does_not_depend_on_the_last_solve(vofp, monkeypatch):
     _, info = ctx.vofp_solve(b, mode=vofp.MODE_MIXED, **kw)
     assert info["status"] == 0 and info["rel_residual"] <= 1e-10
     ctx.close()
+
+
+def _in_child(tmp_path, code):
+    """Run code in a process whose CUDA runtime calls pass through tests/fake_cudart.c (a failing call is made on
+    the host); `fake` sets one of its variables, `fakes` reads one."""
+    lib = str(tmp_path / "fake.so")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-O1", "-Wall", "-o", lib, os.path.join(HERE, "fake_cudart.c"), "-ldl"],
+                   check=True)
+    head = f"""
+import ctypes, sys
+sys.path.insert(0, {os.path.dirname(HERE)!r})
+import torch
+from paper_1410_1937_gb300 import inputs as I, vofp
+lib = ctypes.CDLL({lib!r})
+TYPES = {{"fake_malloc_limit": ctypes.c_size_t}}
+def fakes(name): return TYPES.get(name, ctypes.c_int).in_dll(lib, name).value
+def fake(name, value): TYPES.get(name, ctypes.c_int).in_dll(lib, name).value = value
+"""
+    r = subprocess.run([sys.executable, "-c", head + textwrap.dedent(code)], env={**os.environ, "LD_PRELOAD": lib},
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
+
+
+# bytes above which an allocation is refused: every one, then those after the levels (FP32), then the vectors'
+@pytest.mark.parametrize("limit", [0, 100 * 1000, 250 * 1000])
+@pytest.mark.parametrize("mode", ["mixed", "fp64"])
+def test_solve_goes_on_without_the_correction_when_memory_is_refused(tmp_path, mode, limit):
+    """The plain iteration's result, bit for bit, no memory kept, and the correction again for the next operator."""
+    _in_child(tmp_path, f"""
+        import os
+        prob = I.config1(shape=(64, 48, 40))
+        ctx, t = vofp.context_for(prob)
+        kw = dict(rtol=1e-10, precond=vofp.PRECOND_RBSGS, mode=vofp.MODE_{mode.upper()})
+        b = ctx.vofp_rhs_from_face_velocity(t["u"], t["v"], t["w"])
+        xs = [torch.zeros_like(b) for _ in range(4)]
+        os.environ["VOFP_MG"] = "0"
+        plain = ctx.vofp_solve(b, x=xs[0], x0_zero=1, **kw)[1]
+        held = ctx.vofp_get_stats()["device_bytes"]
+        assert torch.equal(xs[0], xs[0])   # (torch's own memory for it is there)
+        os.environ["VOFP_MG"] = "2"
+        fake("fake_malloc_limit", {limit})
+        for x in xs[1:3]:
+            info = ctx.vofp_solve(b, x=x, x0_zero=1, **kw)[1]
+            assert info["status"] == 0 and info["iterations"] == plain["iterations"], (info, plain)
+            assert torch.equal(x, xs[0])
+            assert ctx.vofp_get_stats()["device_bytes"] - held in (0, 8)   # (8: one word, kept)
+        assert fakes("fake_refused") == 1
+        fake("fake_malloc_limit", 1 << 62)
+        ctx.vofp_build_operator(t["F"], t["ax"], t["ay"], t["az"], t["vf"], prob.bc, prob.rho_liquid, prob.rho_gas,
+                                prob.merge_threshold, prob.density_smoothing, prob.dt)
+        info = ctx.vofp_solve(b, x=xs[3], x0_zero=1, **kw)[1]
+        assert info["status"] == 0 and 2 * info["iterations"] < plain["iterations"], (info, plain)
+        ctx.close()
+    """)
