@@ -880,11 +880,14 @@ vofp_status build(vofp_ctx* c) {
     const long long nv = COMPACT ? c->rbc_cap : d.n;
     if (nv > m.cap) {
         // entries past the vectors in use stay 0 (the tensor copies read whole boxes)
+        c->release(&m.w, m.cap);
+        c->release(&m.z, m.cap);
         m.cap = nv;
         if ((s = c->alloc(&m.w, nv)) || (s = c->alloc(&m.z, nv))) return s;
     }
     VOFP_CUDA_TRY(c, cudaMemsetAsync(m.z, 0, sizeof(T) * m.cap, st));
     if (c->ngroups > m.rep_cap) {
+        c->release(&m.rep, 2 * m.rep_cap);
         m.rep_cap = c->ngroups + c->ngroups / 2 + 64;
         if ((s = c->alloc(&m.rep, 2 * m.rep_cap))) return s;
     }

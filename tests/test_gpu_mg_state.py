@@ -5,6 +5,7 @@ import subprocess
 import sys
 import textwrap
 
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -98,3 +99,29 @@ def test_solve_goes_on_without_the_correction_when_memory_is_refused(tmp_path, m
         assert info["status"] == 0 and 2 * info["iterations"] < plain["iterations"], (info, plain)
         ctx.close()
     """)
+
+
+@pytest.mark.parametrize("mode", ["mixed", "fp64"])
+def test_growing_merge_groups_leave_no_memory_behind(vofp, monkeypatch, mode):
+    """The correction's share of the context's memory (with it less without it) after operators of more and more
+    merge groups is at most that of a context which has seen the last one alone: a buffer is of the size that the
+    last operator asked for which did not fit, and the last one asks for the most."""
+    prob = I.config1(shape=(64, 48, 40))
+    open_cells, part = prob.vf == 1.0, np.random.default_rng(8).random(prob.vf.shape)
+    kw = dict(rtol=1e-10, precond=vofp.PRECOND_RBSGS, mode=vofp.MODE_MIXED if mode == "mixed" else vofp.MODE_FP64)
+
+    def held(flag, shares):
+        monkeypatch.setenv("VOFP_MG", flag)
+        ctx, t = vofp.context_for(prob)
+        for share in shares:
+            t["vf"] = torch.from_numpy(np.where(open_cells & (part < share), 0.05, prob.vf).ravel()).cuda()
+            _rebuild(ctx, t, prob)
+            b = ctx.vofp_rhs_from_face_velocity(t["u"], t["v"], t["w"])
+            assert ctx.vofp_solve(b, **kw)[1]["status"] == 0
+        stats = ctx.vofp_get_stats()
+        assert stats["rb_compact"] == (mode == "mixed")
+        ctx.close()
+        return stats["device_bytes"]
+
+    shares = (0.002, 0.04, 0.13)
+    assert held("2", shares) - held("0", shares) <= held("2", shares[-1:]) - held("0", shares[-1:])
