@@ -1140,15 +1140,17 @@ constexpr double kMixedLoopMargin = 0.5;
 constexpr int kMaxRestarts = 3;
 
 // One pass of the FP64 or mixed-precision solve from x (or 0); fills every field of *info
-// (rel_residual recomputed from x) and returns the loop's own status.
-vofp_status solve_pass(vofp_ctx* c, const double* b, double* x, const vofp_solve_opts* o, vofp_solve_info* info) {
+// (rel_residual recomputed from x) and returns the loop's own status.  correct: with the coarse-grid correction
+// where it is wanted; *rel0: the residual that the pass started from.
+vofp_status solve_pass(vofp_ctx* c, const double* b, double* x, const vofp_solve_opts* o, bool correct,
+                       vofp_solve_info* info, double* rel0) {
     vofp_status s = ensure_workspace(c);
     if (s) return s;
     // colour-compact vectors of the red-black inner solve (built once per operator)
     if (o->mode == VOFP_MODE_MIXED && o->precond == VOFP_PRECOND_RBSGS && (s = rbc_ensure(c))) return s;
     // and the hierarchy of its coarse-grid correction
     c->mg_use = false;
-    if (o->precond == VOFP_PRECOND_RBSGS && mg_wanted(c, o->rtol)) {
+    if (correct && o->precond == VOFP_PRECOND_RBSGS && mg_wanted(c, o->rtol)) {
         const bool fp64 = o->mode != VOFP_MODE_MIXED;
         if ((s = mg_ensure(c, fp64))) return s;
         c->mg_use = fp64 ? c->mgd.ok : c->mgf.ok;
@@ -1239,6 +1241,7 @@ vofp_status solve_pass(vofp_ctx* c, const double* b, double* x, const vofp_solve
         c->set_error("non-finite right-hand side or initial residual");
         return VOFP_ERR_BREAKDOWN;
     }
+    *rel0 = std::sqrt(h.rnorm2 / h.ref2);
     const bool converged0 = !(h.rnorm2 > rtol_loop * rtol_loop * h.ref2);
     if (o->host_loop && !converged0) {
         if ((s = host_loop(c, mixed, rb, U))) return s;
@@ -1311,54 +1314,59 @@ const char* status_text(vofp_status s) {
 
 }  // namespace
 
-// The solve of the contract: VOFP_OK only when the residual recomputed from the returned x is at
-// most rtol.  A pass that stops with its own residual below rtol but the recomputed one above it
-// is restarted from its iterate (a fresh true residual); VOFP_ERR_STAGNATED when a restart fails
-// to halve the recomputed residual or kMaxRestarts do not reach rtol, VOFP_ERR_NOT_CONVERGED when
-// max_iter runs out first.
+// Passes until the residual recomputed from the returned x is at most rtol: a pass that stops with its own
+// residual below rtol but the recomputed one above it is restarted from its iterate (a fresh true residual).
+// VOFP_ERR_STAGNATED when a restart fails to halve the recomputed residual or kMaxRestarts do not reach rtol,
+// VOFP_ERR_NOT_CONVERGED when max_iter runs out first.  *rel0: the residual of the first pass's start.
+static vofp_status solve_restarted(vofp_ctx* c, const double* b, double* x, const vofp_solve_opts* o, bool correct,
+                                   vofp_solve_info* acc, double* rel0) {
+    const long long max_iter = o->max_iter > 0 ? o->max_iter : 100000;
+    vofp_status r = solve_pass(c, b, x, o, correct, acc, rel0);
+    for (int restart = 0; r == VOFP_OK && !(acc->rel_residual <= o->rtol); ++restart) {
+        if (acc->iterations >= max_iter) return VOFP_ERR_NOT_CONVERGED;
+        if (restart == kMaxRestarts) return VOFP_ERR_STAGNATED;
+        vofp_solve_opts o2 = *o;
+        o2.x0_zero = 0;
+        o2.max_iter = (int)(max_iter - acc->iterations);
+        vofp_solve_info i2{};
+        const double before = acc->rel_residual;
+        double rel = 0.0;
+        r = solve_pass(c, b, x, &o2, correct, &i2, &rel);
+        acc->iterations += i2.iterations;
+        acc->outer_iterations += i2.outer_iterations;
+        acc->seconds += i2.seconds;
+        acc->rel_residual = i2.rel_residual;
+        if (r == VOFP_OK && !(acc->rel_residual <= o->rtol) && !(acc->rel_residual <= 0.5 * before))
+            return VOFP_ERR_STAGNATED;
+    }
+    return r;
+}
+
+// The solve of the contract: VOFP_OK only when the residual recomputed from the returned x is at most rtol.  What
+// fails with the coarse-grid correction before max_iter runs out (a breakdown: the correction lost positivity;
+// restarts that stagnate; the mixed loop's limit of refinement steps) goes on with the plain red-black iteration: from
+// the iterate if its residual is at most twice the start's (else it has diverged), otherwise from 0.  After a
+// breakdown the operator's later solves in this precision are plain too.
 vofp_status solve(vofp_ctx* c, const double* b, double* x, const vofp_solve_opts* o, vofp_solve_info* info) {
     prepare_kernels(c);
     if (o->mode == VOFP_MODE_FCG_NN) return solve_fcg(c, b, x, o, info);
     vofp_solve_info acc{};
-    vofp_status r = solve_pass(c, b, x, o, &acc);
     const long long max_iter = o->max_iter > 0 ? o->max_iter : 100000;
-    if (r == VOFP_ERR_BREAKDOWN && c->mg_use && std::isfinite(acc.rel_residual) && acc.iterations < max_iter) {
-        // the coarse-grid correction lost positivity: the plain red-black iteration from the iterate
-        c->mgf.ok = c->mgd.ok = false;
+    double rel0 = 0.0;
+    vofp_status r = solve_restarted(c, b, x, o, true, &acc, &rel0);
+    if ((r == VOFP_ERR_BREAKDOWN || r == VOFP_ERR_STAGNATED || r == VOFP_ERR_NOT_CONVERGED) && c->mg_use &&
+        acc.iterations > 0 && acc.iterations < max_iter) {
+        if (r == VOFP_ERR_BREAKDOWN) (o->mode == VOFP_MODE_MIXED ? c->mgf.ok : c->mgd.ok) = false;
         vofp_solve_opts o2 = *o;
-        o2.x0_zero = 0;
+        o2.x0_zero = !(acc.rel_residual <= 2.0 * rel0);
         o2.max_iter = (int)(max_iter - acc.iterations);
         vofp_solve_info i2{};
         c->err.clear();
-        r = solve_pass(c, b, x, &o2, &i2);
+        r = solve_restarted(c, b, x, &o2, false, &i2, &rel0);
         i2.iterations += acc.iterations;
         i2.outer_iterations += acc.outer_iterations;
         i2.seconds += acc.seconds;
         acc = i2;
-    }
-    for (int restart = 0; r == VOFP_OK && !(acc.rel_residual <= o->rtol); ++restart) {
-        if (acc.iterations >= max_iter) {
-            r = VOFP_ERR_NOT_CONVERGED;
-            break;
-        }
-        if (restart == kMaxRestarts) {
-            r = VOFP_ERR_STAGNATED;
-            break;
-        }
-        vofp_solve_opts o2 = *o;
-        o2.x0_zero = 0;
-        o2.max_iter = (int)(max_iter - acc.iterations);
-        vofp_solve_info i2{};
-        const double before = acc.rel_residual;
-        r = solve_pass(c, b, x, &o2, &i2);
-        acc.iterations += i2.iterations;
-        acc.outer_iterations += i2.outer_iterations;
-        acc.seconds += i2.seconds;
-        acc.rel_residual = i2.rel_residual;
-        if (r == VOFP_OK && !(acc.rel_residual <= o->rtol) && !(acc.rel_residual <= 0.5 * before)) {
-            r = VOFP_ERR_STAGNATED;
-            break;
-        }
     }
     acc.status = r;
     if (info) *info = acc;
