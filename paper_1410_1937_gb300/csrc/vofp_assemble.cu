@@ -627,14 +627,6 @@ k_rhs(Dims d, March m, Bc6 bc, Flux6 nf, double dt, const double* __restrict__ d
     }
 }
 
-__global__ void k_group_expand(int ng, const int* __restrict__ gptr, const int* __restrict__ gcells,
-                               double* __restrict__ v) {
-    int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= ng) return;
-    const double vm = v[gcells[gptr[g]]];
-    for (int t = gptr[g] + 1; t < gptr[g + 1]; ++t) v[gcells[t]] = vm;
-}
-
 __global__ void k_group_fold(int ng, const int* __restrict__ gptr, const int* __restrict__ gcells,
                              double* __restrict__ v, int zero_slaves) {
     int g = blockIdx.x * blockDim.x + threadIdx.x;
@@ -652,11 +644,6 @@ int grid_for(long long n) {
 }
 
 }  // namespace
-
-void launch_group_expand(vofp_ctx* c, double* v) {
-    if (c->ngroups == 0) return;
-    launch(c, k_group_expand, ceil_div(c->ngroups, kNT), kNT, c->stream, c->ngroups, c->gptr, c->gcells, v);
-}
 
 void launch_group_fold(vofp_ctx* c, double* v, bool zero_slaves) {
     if (c->ngroups == 0) return;

@@ -374,7 +374,6 @@ vofp_status vof_advect(vofp_ctx* c, const double* F, const double* ax, const dou
 vofp_status exit_flux(vofp_ctx* c, const double* u, const double* v, const double* w, const double* body, double uc,
                       const double* r1, int balance, double* g_out, double* shift_out);
 
-void launch_group_expand(vofp_ctx* c, double* v);
 void launch_group_fold(vofp_ctx* c, double* v, bool zero_slaves);
 
 // stencil helpers (vofp_stencil.cu)
@@ -392,17 +391,10 @@ inline void launch(vofp_ctx* c, void (*k)(KArgs...), dim3 g, dim3 b, cudaStream_
     k<<<g, b, 0, s>>>(static_cast<KArgs>(args)...);
     ++c->launches;
 }
-// Same, with dynamic shared memory.
-template <typename... KArgs, typename... Args>
-inline void launch_smem(vofp_ctx* c, void (*k)(KArgs...), dim3 g, dim3 b, size_t smem, cudaStream_t s,
-                        Args... args) {
-    k<<<g, b, smem, s>>>(static_cast<KArgs>(args)...);
-    ++c->launches;
-}
-
-// Same, optionally as a programmatic dependent launch: the kernel may be scheduled while the
-// previous kernel on the stream drains, and must call griddepcontrol.wait before it reads what
-// that kernel wrote. A refused launch is recorded in c->launch_err.
+// Same, with dynamic shared memory and optionally as a programmatic dependent launch: the kernel
+// may be scheduled while the previous kernel on the stream drains, and must call
+// griddepcontrol.wait before it reads what that kernel wrote. A refused launch is recorded in
+// c->launch_err.
 template <typename... KArgs, typename... Args>
 inline void launch_dep(vofp_ctx* c, bool pdl, void (*k)(KArgs...), dim3 g, dim3 b, size_t smem, cudaStream_t s,
                        Args... args) {
@@ -457,55 +449,6 @@ __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
-}
-
-// Sum of v over the block, valid in thread 0.  Fixed order: deterministic.
-template <int NT>
-__device__ __forceinline__ double block_sum(double v, double* sh) {
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) sh[wid] = v;
-    __syncthreads();
-    double s = 0.0;
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int w = 0; w < NT / 32; ++w) s += sh[w];
-    }
-    return s;
-}
-
-// Write this block's partial and, in the block that finishes last, reduce all partials in
-// index order.  Returns true (in thread 0 of the last block) with *total set.
-// The ticket counter is reset by the last block for the next launch.
-__device__ __forceinline__ bool last_block_reduce(double part, double* partials,
-                                                  unsigned int* counter, int nblocks,
-                                                  double* total, double* sh) {
-    __shared__ bool is_last;
-    const int b = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-    if (threadIdx.x + blockDim.x * threadIdx.y == 0) {
-        partials[b] = part;
-        __threadfence();
-        unsigned int t = atomicAdd(counter, 1u);
-        is_last = (t == (unsigned int)(nblocks - 1));
-    }
-    __syncthreads();
-    if (!is_last) return false;
-    __threadfence();
-    const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-    const int nt = blockDim.x * blockDim.y;
-    double s = 0.0;
-    if (tid < 32) {
-        for (int i = tid; i < nblocks; i += 32) s += *((volatile double*)&partials[i]);
-        s = warp_sum(s);
-    }
-    if (tid == 0) {
-        *total = s;
-        *counter = 0u;
-    }
-    (void)nt;
-    (void)sh;
-    return tid == 0;
 }
 
 }  // namespace vofp
