@@ -566,10 +566,11 @@ __device__ __noinline__ Flux5 cut_fluxes(double x0, double x1, double y0, double
     f.zp = __dmul_rn(z1 * Sz, w1);
     return f;
 }
-// FP64 arithmetic bounds it: 1057 us with both faces of every direction formed from three factors and a division
-// in every cell, 505 here (512 x 256 x 128; 0.94 GB, 140 us at copy bandwidth).  The division is left out where
-// dt is 1 (HOW 0) and is a multiplication by the exact reciprocal, given as dt, where it is a power of two (1).
-template <int HOW>   // -div (0), -div times dt (1), -div / dt (2)
+// FP64 arithmetic bounds it (512 x 256 x 128; 0.94 GB, 140 us at copy bandwidth): 1057 us with both faces of every
+// direction formed from three factors and a division in every cell; 757 here (23.7 FP64 instructions a cell), as a time
+// step's dt takes it, and 505 (15.4) where dt is a power of two and the division a multiplication by its exact reciprocal,
+// given as dt.  1 is one of them: without the multiplication it took 505 as well.
+template <bool RECIPROCAL>
 __global__ void __launch_bounds__(kNT, 5)
 k_rhs(Dims d, March m, Bc6 bc, Flux6 nf, double dt, const double* __restrict__ dx,
                       const double* __restrict__ dy, const double* __restrict__ dz,
@@ -613,7 +614,7 @@ k_rhs(Dims d, March m, Bc6 bc, Flux6 nf, double dt, const double* __restrict__ d
         if (k == d.nz - 1 && wall[5]) f.zp = 0.0;
         double div = __dadd_rn(__dadd_rn(__dsub_rn(f.xp, f.xm), __dsub_rn(f.yp, f.ym)), __dsub_rn(f.zp, fzm));
         if (body) div += body[c];
-        double bb = HOW == 0 ? -div : HOW == 1 ? -div * dt : -div / dt;
+        double bb = RECIPROCAL ? -div * dt : -div / dt;
         if (edge || (k == 0 && nf.g[4]) || (k == d.nz - 1 && nf.g[5])) {
             if (i == 0 && bc.k[0] == VOFP_BC_NEUMANN && nf.g[0]) bb += axe[fx_idx(d, 0, j, k)] * Sx * nf.g[0][j + (long long)d.ny * k];
             if (i == d.nx - 1 && bc.k[1] == VOFP_BC_NEUMANN && nf.g[1]) bb += axe[fx_idx(d, d.nx, j, k)] * Sx * nf.g[1][j + (long long)d.ny * k];
@@ -951,7 +952,7 @@ vofp_status rhs(vofp_ctx* c, const double* u, const double* v, const double* w, 
     const double dt = c->phys.dt;
     int e = 0;
     const bool pow2 = std::isnormal(dt) && std::fabs(std::frexp(dt, &e)) == 0.5 && std::isnormal(1.0 / dt);
-    launch(c, dt == 1.0 ? k_rhs<0> : pow2 ? k_rhs<1> : k_rhs<2>, ceil_div(d.plane * m.nch, kNT), kNT, c->stream, d, m, b6, nf,
+    launch(c, pow2 ? k_rhs<true> : k_rhs<false>, ceil_div(d.plane * m.nch, kNT), kNT, c->stream, d, m, b6, nf,
            pow2 ? 1.0 / dt : dt, c->dx, c->dy, c->dz, c->axe, c->aye, c->aze, c->inactive, u, v, w, body, b);
     VOFP_CUDA_TRY(c, cudaGetLastError());
     return VOFP_OK;
