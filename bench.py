@@ -62,11 +62,11 @@ def iter_elems(variant):
 # DRAM read+write bytes per cell of one launch of the dominant kernel, from committed ncu captures
 # of the 512x256x128 workload (dram__bytes_read.sum + dram__bytes_write.sum, one pass), each valid
 # only while the sources of that kernel and its launch hash to the value stored with it (else null):
-#   (32, "jacobi"): k_cg_tma<float, 6, 2> (column split), 561.8 MB over 16777216 cells
-#   (32, "rbsgs"):  k_cg_rb_tma<3, 8>, 885.6 MB over 16777216 cells
+#   (32, "jacobi"): k_cg_tma<float, 6, 2> (column split), 566.4 MB over 16777216 cells
+#   (32, "rbsgs"):  k_cg_rb_tma<3, 8>, 885.0 MB over 16777216 cells
 #   (32, "rbsgs-compact"): k_rbc_tma<3, 2> (32 x 16 tiles in 8 x 2 groups, one barrier per step),
 #                          425.9 MB over 16777216 cells (mean of two launches)
-TRAFFIC_PER_CELL = {(32, "jacobi"): (33.49, "7d8c8dd1b0cef8cd"), (32, "rbsgs"): (52.78, "987a1d6fd554bdf8"), (32, "rbsgs-compact"): (25.38, "dd674a48feca84db")}
+TRAFFIC_PER_CELL = {(32, "jacobi"): (33.76, "194b6eedcef00b3e"), (32, "rbsgs"): (52.75, "d23ad2e27f43f7fc"), (32, "rbsgs-compact"): (25.39, "fccb62a9350efee7")}
 KERNEL_FILES = {(32, "jacobi"): ('vofp_kernels.cuh', 'vofp_tma.cuh', 'vofp_tma.cu'),
                 (32, "rbsgs"): ('vofp_kernels.cuh', 'vofp_tma.cuh', 'vofp_rb_tma.cuh', 'vofp_rb_tma.cu'),
                 (32, "rbsgs-compact"): ('vofp_kernels.cuh', 'vofp_tma.cuh', 'vofp_rbc.cuh', 'vofp_rbc.cu')}

@@ -107,7 +107,9 @@ typedef struct {
  *               V-cycle on 2x2x2 aggregates smoothed by red-black Gauss-Seidel (in the precision
  *               of the iteration's vectors).  It takes 10 to 12 bytes per cell in mixed mode and 24 in
  *               FP64 mode, allocated on the first such solve and kept by the context; an operator
- *               for which that memory cannot be had is solved without the correction.
+ *               for which that memory cannot be had is solved without the correction.  A solve
+ *               that fails with it (breakdown, stagnation, the limit of refinement steps) goes on
+ *               without it as far as max_iter allows.
  *   rtol        the solve returns VOFP_OK only when the residual recomputed from the returned x,
  *               ||b_hat - A_hat x|| (2-norm over the unknowns, FP64), is at most rtol ||b_hat||.
  *               The iteration aims slightly below rtol; when the recomputed residual is still
@@ -120,9 +122,10 @@ typedef struct {
  *               steps (the FP64 residual replaces the FP32 one, a "reliable update"); 1 restarts
  *               the inner PCG from p = r at every refinement step.
  *   check_every convergence is tested every check_every iterations (even, 2 .. 64; 0 = default:
- *               16 where the coarse-grid correction runs, 64 in the other mixed solves from 2^20
- *               cells on, where an inner solve runs on to the end of its 64 iterations past its
- *               stop and saves refinement steps, 8 otherwise).
+ *               8 in FP64 mode; in mixed mode 16 where the coarse-grid correction runs on 2^16
+ *               cells or more, 64 in plain solves from 2^20 cells on, where an inner solve runs on
+ *               to the end of its 64 iterations past its stop and saves refinement steps, 8
+ *               otherwise).
  *   x0_zero     1: ignore the contents of x and start from 0.
  *   host_loop   0: the loop runs as a CUDA graph with a device-side WHILE condition (no host round
  *               trip per iteration).  1: the host launches each kernel and reads the convergence
@@ -134,9 +137,11 @@ typedef struct {
  *               The network's steps continue while the inner residual norm falls at least to
  *               stag_ratio of its value stag_window iterations before; otherwise (or on a
  *               breakdown) the solve hands over to VOFP_MODE_MIXED (precond as given) from the
- *               current iterate.  A network application costs about as much as 25 iterations
- *               of the mixed red-black solve, so the defaults (window 2, ratio 0.6) keep it only
- *               while it beats those.
+ *               current iterate.  The defaults (window 2, ratio 0.6) keep the network only while
+ *               it beats the plain mixed red-black iteration, of which an application costs about
+ *               25; of the iterations with the coarse-grid correction, which the hand-over takes
+ *               for rtol <= 1e-7, it costs about 11, and each reduces the residual like nine plain
+ *               ones: such a solve is the faster one without the network.
  *   stag_window, stag_ratio  the hand-over test above (0 selects the defaults; window <= 63). */
 typedef struct {
     int mode;

@@ -95,11 +95,13 @@ struct MgSet {
 };
 // smallest grid whose red-black solves take the coarse-grid correction: from here on they are 1.1 to
 // 5 times faster than the plain iteration (64x48x40 to 1e-12, mixed: 12 against 19 ms, FP64: 16.2 against
-// 18.4); from 16^3 to 48x40x32 the mixed ones took 0.7 to 1 of its time, the FP64 ones 0.9 to 1.15
+// 18.4).  From 16^3 to 48x40x32 the mixed ones took 0.7 to 1 of its time and the FP64 ones 0.9 to 1.15: the
+// limit is one for both precisions, where both gain
 constexpr long long kMgMinCells = 1 << 16;
-// ... and the loosest tolerance that does.  The correction is the faster one at every tolerance (256x128x64
-// to 1e-6: 13.9 against 39.4 ms, 512x256x128 49 against 232 ms), but a pressure solved more loosely is
-// settled only to its first few digits, and which ones depends on the iteration: such solves keep theirs
+// ... and the loosest tolerance that does.  Not for speed (256x128x64 to 1e-6: 13.9 against 39.4 ms with the plain
+// iteration, 512x256x128 49 against 232 ms) nor for accuracy, which is the caller's tolerance either way: a pressure
+// solved more loosely is settled only to its first few digits, and the others depend on the iteration.  Such
+// solves keep the digits that they have always returned
 constexpr double kMgMaxRtol = 1e-7;
 
 }  // namespace vofp
