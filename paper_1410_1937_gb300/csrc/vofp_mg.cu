@@ -173,23 +173,34 @@ __global__ void k_mg_weights(Dims d, long long n, long long nh, const double* __
     }
 }
 
-// merge groups: the master's entry and aggregate (rep) and its weight, -1 for the other members; on the
+// Most that w^2 D^-1 of a master's aggregate may be: the part of its own r that one level adds to its z.  (Cells without a
+// group have about a quarter; see k_mg_groups.)
+constexpr double kMaxSelf = 0.5;
+
+// merge groups: the master's entry and aggregate (rep) and its weight, -1 for the other members.  The master stands
+// for couplings of all of the group's cells, and its aggregate has only those of the cells that lie in it: where they
+// are few the aggregate seems as good as free and answers with a multiple of what it should.  So the weight is at most
+// what keeps w^2 D^-1 at kMaxSelf.  Without that, with cells of less than half their volume merged: 232x32x206 hull with
+// every tenth face closed, to 1e-9, mixed 4160 iterations (1984 without the correction) -> 464; 132x80x102 sphere 608
+// (832) -> 176, FP64 328 (696) -> 152; merging below a tenth is as it was.  On the
 // compact vectors the aggregates' mask bits of even-parity masters and their entries, four per aggregate
 // (read, and written, only where the bit is set).  Member entries: gref (compact) or the cells
 template <bool COMPACT, typename T>
 __global__ void k_mg_groups(Dims d, int ng, int nx1, int ny1, const int* __restrict__ gptr,
                             const int* __restrict__ gcells, const int* __restrict__ gref,
-                            const double* __restrict__ sq, const unsigned long long* dmax, T* __restrict__ w,
-                            int2* __restrict__ rep, uint32_t* __restrict__ mask, int* __restrict__ even) {
+                            const double* __restrict__ sq, const unsigned long long* dmax, const T* __restrict__ di,
+                            T* __restrict__ w, int2* __restrict__ rep, uint32_t* __restrict__ mask, int* __restrict__ even) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= ng) return;
     const double sg = scalbn(1.0, -mg_exponent(dmax));
     const int u0 = gptr[g], u1 = gptr[g + 1];
-    for (int u = u0; u < u1; ++u)
-        w[COMPACT ? gref[u] : gcells[u]] = u == u0 ? (T)(sq[gcells[u]] * sg) : T(-1);
     int i, j, k;
     cell_ijk(d, gcells[u0], i, j, k);
     const int t = (i >> 1) + nx1 * ((j >> 1) + ny1 * (k >> 1)), u = 2 * (k & 1) + (j & 1);
+    double ws = sq[gcells[u0]] * sg;
+    if (ws * ws * (double)di[t] > kMaxSelf) ws = sqrt(kMaxSelf / (double)di[t]);
+    for (int u = u0; u < u1; ++u)
+        w[COMPACT ? gref[u] : gcells[u]] = u == u0 ? (T)ws : T(-1);
     rep[g] = make_int2(COMPACT ? gref[u0] : gcells[u0], t);
     if (!COMPACT || ((i + j + k) & 1)) return;
     atomicOr(&mask[t >> 2], (1u << u) << (8 * (t & 3)));
@@ -911,8 +922,8 @@ vofp_status build(vofp_ctx* c) {
            (const int32_t*)c->root, (const uint32_t*)c->red_bits, dmax, m.w);
     if (c->ngroups > 0)
         launch(c, k_mg_groups<COMPACT, T>, ceil_div(c->ngroups, kNT), kNT, st, d, c->ngroups, l1.nx, l1.ny,
-               (const int*)c->gptr, (const int*)c->gcells, (const int*)c->rbc_gref, (const double*)c->sq, dmax, m.w,
-               reinterpret_cast<int2*>(m.rep), c->mg_mask, c->mg_even);
+               (const int*)c->gptr, (const int*)c->gcells, (const int*)c->rbc_gref, (const double*)c->sq, dmax, (const T*)l1.di,
+               m.w, reinterpret_cast<int2*>(m.rep), c->mg_mask, c->mg_even);
     VOFP_CUDA_TRY(c, cudaGetLastError());
     m.ok = true;
     return VOFP_OK;
