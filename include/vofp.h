@@ -103,7 +103,9 @@ typedef struct {
  *   precond     VOFP_PRECOND_JACOBI (diagonal) or VOFP_PRECOND_RBSGS (red-black symmetric
  *               Gauss-Seidel, applied as CG on the black unknowns after eliminating the red ones
  *               (Eisenstat's form); both modes, and the bench default in mixed mode).  From 2^16
- *               cells and for rtol <= 1e-7 its CG also has a coarse-grid correction: an additive
+ *               cells and for rtol <= 1e-7 its CG also has a coarse-grid correction, unless the
+ *               operator is one that gains nothing by it (couplings that differ by much between
+ *               the axes, many closed faces, p = 0 walls all around a small grid): an additive
  *               V-cycle on 2x2x2 aggregates smoothed by red-black Gauss-Seidel (in the precision
  *               of the iteration's vectors).  It takes 10 to 12 bytes per cell in mixed mode and 24 in
  *               FP64 mode, allocated on the first such solve and kept by the context; an operator

@@ -779,6 +779,7 @@ vofp_status build_operator(vofp_ctx* c, const double* F, const double* ax, const
     c->grp_built = false;
     c->mgf.built = c->mgf.ok = false;
     c->mgd.built = c->mgd.ok = false;
+    c->mg_pays = -1;
     for (int f = 0; f < 6; ++f) c->bc[f] = bc->kind[f];
     c->phys = *phys;
     c->dirichlet = false;

@@ -103,6 +103,8 @@ constexpr long long kMgMinCells = 1 << 16;
 // solved more loosely is settled only to its first few digits, and the others depend on the iteration.  Such
 // solves keep the digits that they have always returned
 constexpr double kMgMaxRtol = 1e-7;
+// ... and which operators (see pays in vofp_mg.cu)
+constexpr double kMgMinCoupling = 0.478, kMgMaxAnisotropy = 90.0, kMgMinScore = 1.33e5;
 
 }  // namespace vofp
 
@@ -230,6 +232,7 @@ struct vofp_ctx {
     // coarse-grid correction of the red-black solves (vofp_mg.cu)
     vofp::MgSet<float> mgf;           // mixed mode
     vofp::MgSet<double> mgd;          // FP64 mode
+    int mg_pays = -1;                 // whether it is likely to pay for the current operator (-1: not looked at)
     bool mg_use = false;              // in use in the current solve (set by each; means nothing outside one)
     uint32_t* mg_mask = nullptr;      // per aggregate (a byte): its even cells that are group masters
     int* mg_even = nullptr;           // their entries, four per aggregate
@@ -288,7 +291,7 @@ void rbc_iteration(vofp_ctx* c, cudaStream_t st, const float* po, float* pn, cud
 void rbc_finish_xf(vofp_ctx* c, cudaStream_t st);                 // xf (full grid) = x_c + alpha p0_c
 int rbc_pq_parts(const vofp_ctx* c);   // block partials of p.Ap the compact iteration leaves for the update
 // coarse-grid correction of the red-black solves (vofp_mg.cu)
-bool mg_wanted(const vofp_ctx* c, double rtol);   // whether a red-black solve takes it
+vofp_status mg_wanted(vofp_ctx* c, double rtol, bool* wanted);   // whether a red-black solve takes it
 vofp_status mg_ensure(vofp_ctx* c, bool fp64);    // hierarchy of the current operator; sets mgf.ok / mgd.ok
 void mg_precondition(vofp_ctx* c, cudaStream_t st, bool fp64, bool pdl, int start);   // z and beta from r
 void mg_update(vofp_ctx* c, cudaStream_t st, bool fp64, bool pdl, cudaGraphConditionalHandle h, int use_h, int npq);

@@ -1150,7 +1150,9 @@ vofp_status solve_pass(vofp_ctx* c, const double* b, double* x, const vofp_solve
     if (o->mode == VOFP_MODE_MIXED && o->precond == VOFP_PRECOND_RBSGS && (s = rbc_ensure(c))) return s;
     // and the hierarchy of its coarse-grid correction
     c->mg_use = false;
-    if (correct && o->precond == VOFP_PRECOND_RBSGS && mg_wanted(c, o->rtol)) {
+    bool wanted = false;
+    if (correct && o->precond == VOFP_PRECOND_RBSGS && (s = mg_wanted(c, o->rtol, &wanted))) return s;
+    if (wanted) {
         const bool fp64 = o->mode != VOFP_MODE_MIXED;
         if ((s = mg_ensure(c, fp64))) return s;
         c->mg_use = fp64 ? c->mgd.ok : c->mgf.ok;
