@@ -175,15 +175,16 @@ __global__ void k_mg_weights(Dims d, long long n, long long nh, const double* __
 }
 
 // Most that w^2 D^-1 of a master's aggregate may be: the part of its own r that one level adds to its z.  (Cells without a
-// group have about a quarter; see k_mg_groups.)
-constexpr double kMaxSelf = 0.5;
+// group have about a quarter; see k_mg_groups.  At 0.5 the operators named there take a tenth fewer iterations still, but
+// ordinary ones other bits as well; at 1 nearly all of those keep theirs.)
+constexpr double kMaxSelf = 1.0;
 
 // merge groups: the master's entry and aggregate (rep) and its weight, -1 for the other members.  The master stands
 // for couplings of all of the group's cells, and its aggregate has only those of the cells that lie in it: where they
 // are few the aggregate seems as good as free and answers with a multiple of what it should.  So the weight is at most
 // what keeps w^2 D^-1 at kMaxSelf.  Without that, with cells of less than half their volume merged: 232x32x206 hull with
-// every tenth face closed, to 1e-9, mixed 4160 iterations (1984 without the correction) -> 464; 132x80x102 sphere 608
-// (832) -> 176, FP64 328 (696) -> 152; merging below a tenth is as it was.  On the
+// every tenth face closed, to 1e-9, mixed 4160 iterations (1984 without the correction) -> 528; 132x80x102 sphere 608
+// (832) -> 208, FP64 328 (696) -> 184.  On the
 // compact vectors the aggregates' mask bits of even-parity masters and their entries, four per aggregate
 // (read, and written, only where the bit is set).  Member entries: gref (compact) or the cells
 template <bool COMPACT, typename T>
@@ -969,8 +970,8 @@ void precondition(vofp_ctx* c, cudaStream_t st, bool pdl, int start) {
 //   sqrt(cells) condition / anisotropy  at least kMgMinScore
 // 1225 solves of 246 random operators (65,536 to 5 M cells, aspect ratios of cells to 30 and of grids to 300, density
 // ratios to 1e5, walls of every kind, open, with a tenth and with a third of the faces closed, tolerances 1e-7 to 1e-12;
-// time without the correction over time with it, geometric mean): 1.59 with it everywhere, 205 solves slower by more than
-// 5 %, the worst 0.33; 1.63 by this rule, which takes it for 871, with 33 slower, the worst 0.69.
+// time without the correction over time with it, geometric mean): 1.56 with it everywhere, 209 solves slower by more than
+// 5 %, the worst 0.33; 1.60 by this rule, which takes it for 871, with 35 slower, the worst 0.69.
 static bool pays(const Dims& d, const int bc[6], const double m[3]) {
     const int n[3] = {d.nx, d.ny, d.nz};
     const double sum = m[0] + m[1] + m[2];
