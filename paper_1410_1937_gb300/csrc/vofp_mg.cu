@@ -184,9 +184,9 @@ constexpr double kMaxSelf = 1.0;
 // are few the aggregate seems as good as free and answers with a multiple of what it should.  So the weight is at most
 // what keeps w^2 D^-1 at kMaxSelf.  Without that, with cells of less than half their volume merged: 232x32x206 hull with
 // every tenth face closed, to 1e-9, mixed 4160 iterations (1984 without the correction) -> 528; 132x80x102 sphere 608
-// (832) -> 208, FP64 328 (696) -> 184.  On the
-// compact vectors the aggregates' mask bits of even-parity masters and their entries, four per aggregate
-// (read, and written, only where the bit is set).  Member entries: gref (compact) or the cells
+// (832) -> 208, FP64 328 (696) -> 184.  On the compact vectors also the aggregates' mask bits of even-parity masters
+// and their entries, four per aggregate (read, and written, only where the bit is set).  Member entries: gref
+// (compact) or the cells
 template <bool COMPACT, typename T>
 __global__ void k_mg_groups(Dims d, int ng, int nx1, int ny1, const int* __restrict__ gptr,
                             const int* __restrict__ gcells, const int* __restrict__ gref,
